@@ -27,6 +27,7 @@
 #include <cstring>
 
 #include "df64.cuh"
+#include "fft_engine.cuh"
 #include "host_math.h"
 #include "wgrid_internal.h"
 
@@ -522,6 +523,247 @@ k_fft_lines_cluster(const __grid_constant__ FftLine L, void* __restrict__ data, 
 }
 
 // ---------------------------------------------------------------------------------------
+// Pairs of lines (fft_engine.cuh): the kernel of every line that splits into 1, 2, 4 or 8 parts
+// of at most kPairMaxPart points with radices up to 12
+//
+// A CTA (a cluster of S CTAs when the line is split) transforms two lines of a plane at once,
+// packed into the two halves of the FP32 x2 instructions.  Bound: the FP32 pipes.  Layout:
+//  * one shared-memory buffer of n packed points, two 16-byte arrays (real pairs, imaginary
+//    pairs); a stage reads its butterflies into registers, synchronises and writes them back in
+//    place (registers hold about 8 - 12 points per thread, so a second buffer would only cost
+//    CTAs per SM);
+//  * the first stage reads its points straight from global memory and the last one writes its
+//    results there, so a three-stage line crosses shared memory twice;
+//  * a split line's radix-S decimation-in-frequency step is done where the points are loaded:
+//    CTA h takes the j-range [h n / S, (h + 1) n / S), forms all S outputs of each butterfly and
+//    writes output r into CTA r's buffer through distributed shared memory;
+//  * radices up to 12 (10, 6 and 12 by coprime factors, no inner twiddles): 1728 = 12 12 12 in
+//    three stages instead of 8 8 3 3 3 in five;
+//  * twiddles are stored per stage in the order the threads read them, each float twice.
+// ---------------------------------------------------------------------------------------
+constexpr int kPairMaxPart = 2048, kPairStages = 12;
+
+struct PairLine {
+  int n, S, T, cls, nst;         // points per CTA, CTAs per line, threads, register class, stages
+  int radix[kPairStages];
+  unsigned magic[kPairStages];   // j / Ns = umulhi(j, magic) for Ns > 1
+  int twofs[kPairStages];        // first entry of the stage's twiddles, entry (kk - 1) Ns + jm
+  const float4* tw;              // two float4 per entry: (rh, rh, rl, rl), (ih, ih, il, il)
+  const float4* tw2;             // split lines: e^{-2 pi i j r / (S n)} at entry (r - 1) n + j
+};
+
+// butterflies of radix R a thread holds at once: class 9 about 8 points, class 12 about 12
+__host__ __device__ constexpr int pair_nb(int cls, int R) {
+  return cls == 9 ? (R >= 5 ? 1 : R == 4 ? 2 : R == 3 ? 3 : 4)
+                  : (R >= 7 ? 1 : R >= 5 ? 2 : R == 4 ? 3 : R == 3 ? 4 : 5);
+}
+
+struct PairIo {
+  float4* data;
+  int64_t base0, base1, es;      // the two lines' first elements, element stride
+  int nfull, lhalf, shalf;
+  bool inv, two;                 // inverse: real and imaginary parts exchanged; second line exists
+  __device__ __forceinline__ Cx<d2> load(int o) const {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+    if (o < lhalf || o >= nfull - lhalf) {
+      a = data[base0 + (int64_t)o * es];
+      if (two) b = data[base1 + (int64_t)o * es];
+    }
+    Cx<d2> x;
+    x.r.h = f2_make(inv ? a.z : a.x, inv ? b.z : b.x);
+    x.r.l = f2_make(inv ? a.w : a.y, inv ? b.w : b.y);
+    x.i.h = f2_make(inv ? a.x : a.z, inv ? b.x : b.z);
+    x.i.l = f2_make(inv ? a.y : a.w, inv ? b.y : b.w);
+    return x;
+  }
+  __device__ __forceinline__ void store(int o, const Cx<d2>& x) const {
+    if (o >= shalf && o < nfull - shalf) return;   // not needed downstream
+    const float2 rh = f2_split(x.r.h), rl = f2_split(x.r.l), ih = f2_split(x.i.h), il = f2_split(x.i.l);
+    data[base0 + (int64_t)o * es] = inv ? make_float4(ih.x, il.x, rh.x, rl.x)
+                                        : make_float4(rh.x, rl.x, ih.x, il.x);
+    if (two)
+      data[base1 + (int64_t)o * es] = inv ? make_float4(ih.y, il.y, rh.y, rl.y)
+                                          : make_float4(rh.y, rl.y, ih.y, il.y);
+  }
+};
+
+// shared-memory slot of point e: the low three bits XORed with the next three (a permutation
+// inside aligned groups of 8; the buffers are allocated in whole groups)
+__device__ __forceinline__ int pair_slot(int e) { return e ^ ((e >> 3) & 7); }
+
+__device__ __forceinline__ Cx<d2> pair_get(const ulonglong2* sr, const ulonglong2* si, int e) {
+  const int s = pair_slot(e);
+  const ulonglong2 a = sr[s], b = si[s];
+  return Cx<d2>{{{a.x}, {a.y}}, {{b.x}, {b.y}}};
+}
+__device__ __forceinline__ void pair_put(ulonglong2* sr, ulonglong2* si, int e, const Cx<d2>& x) {
+  const int s = pair_slot(e);
+  sr[s] = make_ulonglong2(x.r.h.v, x.r.l.v);
+  si[s] = make_ulonglong2(x.i.h.v, x.i.l.v);
+}
+__device__ __forceinline__ Tw<d2> pair_tw(const float4* __restrict__ tw, int t) {
+  const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2*>(tw) + 2 * t);
+  const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(tw) + 2 * t + 1);
+  return Tw<d2>{{a.x}, {a.y}, {b.x}, {b.y}};
+}
+
+struct PairStageArgs {
+  ulonglong2 *sr, *si;
+  const float4* tw;              // the stage's twiddles
+  int n, Ns;
+  unsigned magic;
+  int S, h;                      // the line's element S o + h is result o of this CTA
+};
+// One stage: read the butterflies and transform them, synchronise, write them back in place.
+// kIn: 0 the first stage of a whole line, from global memory; 1 the first stage of a split line,
+// from the buffer that the decimation step has filled (both without twiddles); 2 a later stage.
+// kLast: results to global memory.  (Separate instances: with both destinations in one body the
+// compiler keeps the results in registers for both and spills.)
+template <int R, int CLS, int kIn, bool kLast>
+__device__ __forceinline__ void pair_stage(const PairIo& io, const PairStageArgs& a) {
+  constexpr int NB = pair_nb(CLS, R);
+  const int M = a.n / R, T = blockDim.x, Ns = kIn == 2 ? a.Ns : 1;
+  Cx<d2> x[NB][R];
+  int o[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int j = threadIdx.x + b * T;
+    if (j < M) {
+#pragma unroll
+      for (int k = 0; k < R; ++k)
+        x[b][k] = kIn == 0 ? io.load(j + k * M) : pair_get(a.sr, a.si, j + k * M);
+      o[b] = j * R;
+      if constexpr (kIn == 2) {
+        const int jq = kLast ? 0 : (int)__umulhi((unsigned)j, a.magic), jm = j - jq * Ns;
+        o[b] = jq * Ns * R + jm;
+#pragma unroll
+        for (int k = 1; k < R; ++k) x[b][k] = cx_mul(x[b][k], pair_tw(a.tw, jm + (k - 1) * Ns));
+      }
+      dft<R>(x[b]);
+    }
+  }
+  if (kIn != 0 && !kLast) __syncthreads();   // every point of the buffer has been read
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int j = threadIdx.x + b * T;
+    if (j < M) {
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        if (kLast) io.store(a.S * (o[b] + q * Ns) + a.h, x[b][q]);
+        else pair_put(a.sr, a.si, o[b] + q * Ns, x[b][q]);
+      }
+    }
+  }
+  if (!kLast) __syncthreads();
+}
+template <int CLS, int kIn, bool kLast>
+__device__ __forceinline__ void pair_dispatch(int R, const PairIo& io, const PairStageArgs& a) {
+  if constexpr (kIn != 2) {   // first radix: 8 or 9 (class 9), 8 to 12 (class 12), see pair_plan
+    if constexpr (CLS == 9) {
+      if (R == 8) pair_stage<8, CLS, kIn, kLast>(io, a);
+      else pair_stage<9, CLS, kIn, kLast>(io, a);
+    } else {
+      switch (R) {
+        case 8: pair_stage<8, CLS, kIn, kLast>(io, a); break;
+        case 9: pair_stage<9, CLS, kIn, kLast>(io, a); break;
+        case 10: pair_stage<10, CLS, kIn, kLast>(io, a); break;
+        case 11: pair_stage<11, CLS, kIn, kLast>(io, a); break;
+        default: pair_stage<12, CLS, kIn, kLast>(io, a); break;
+      }
+    }
+  } else {
+    switch (R) {
+      case 2: pair_stage<2, CLS, kIn, kLast>(io, a); break;
+      case 3: pair_stage<3, CLS, kIn, kLast>(io, a); break;
+      case 4: pair_stage<4, CLS, kIn, kLast>(io, a); break;
+      case 5: pair_stage<5, CLS, kIn, kLast>(io, a); break;
+      case 6: pair_stage<6, CLS, kIn, kLast>(io, a); break;
+      case 7: pair_stage<7, CLS, kIn, kLast>(io, a); break;
+      case 8: pair_stage<8, CLS, kIn, kLast>(io, a); break;
+      case 9: pair_stage<9, CLS, kIn, kLast>(io, a); break;
+      default:
+        if constexpr (CLS == 12) {
+          if (R == 10) pair_stage<10, CLS, kIn, kLast>(io, a);
+          else if (R == 11) pair_stage<11, CLS, kIn, kLast>(io, a);
+          else pair_stage<12, CLS, kIn, kLast>(io, a);
+        }
+        break;
+    }
+  }
+}
+
+// the radix-S decimation step of a split line (see above); the cluster barriers are the caller's
+template <int S>
+__device__ __forceinline__ void pair_split(const PairLine& L, const PairIo& io, ulonglong2* sr,
+                                           ulonglong2* si, int h) {
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int n = L.n, per = (n + S - 1) / S;
+  const int j1 = min(n, (h + 1) * per);
+  for (int j = h * per + threadIdx.x; j < j1; j += blockDim.x) {
+    Cx<d2> x[S];
+#pragma unroll
+    for (int r = 0; r < S; ++r) x[r] = io.load(j + r * n);
+    dft<S>(x);
+#pragma unroll
+    for (int r = 0; r < S; ++r) {
+      if (r > 0) x[r] = cx_mul(x[r], pair_tw(L.tw2, (r - 1) * n + j));
+      pair_put(cl.map_shared_rank(sr, r), cl.map_shared_rank(si, r), j, x[r]);
+    }
+  }
+}
+
+// Lines q = 2 p, 2 p + 1 (p = pair index in the plane) of `lines` per plane; line q >= split is
+// shifted by skip.  lhalf, shalf as in k_fft_lines; float pairs in and out.
+template <int CLS, int TMAX>
+__global__ void __launch_bounds__(TMAX, 2)
+k_fft_pairs(const __grid_constant__ PairLine L, float4* __restrict__ data, int64_t plane_elems,
+            int lines, int64_t line_stride, int64_t elem_stride, int inv, int split, int skip,
+            int lhalf, int shalf) {
+  extern __shared__ __align__(16) float4 fsm[];
+  const int S = L.S;
+  const unsigned cid = S > 1 ? blockIdx.x / (unsigned)S : blockIdx.x;
+  const int h = (int)(blockIdx.x - cid * S);   // rank in the cluster (S, 1, 1)
+  const unsigned pairs = (unsigned)(lines + 1) / 2;
+  const unsigned plane = cid / pairs;
+  const int q0 = 2 * (int)(cid - plane * pairs), q1 = q0 + 1;
+  PairIo io;
+  io.data = data;
+  const int64_t pb = (int64_t)plane * plane_elems;
+  io.base0 = pb + (int64_t)(q0 < split ? q0 : q0 + skip) * line_stride;
+  io.base1 = pb + (int64_t)(q1 < split ? q1 : q1 + skip) * line_stride;
+  io.es = elem_stride;
+  io.nfull = S * L.n;
+  io.lhalf = lhalf; io.shalf = shalf;
+  io.inv = inv != 0; io.two = q1 < lines;
+  PairStageArgs a;
+  a.sr = reinterpret_cast<ulonglong2*>(fsm);
+  a.si = a.sr + ((L.n + 7) & ~7);
+  a.n = L.n; a.S = S; a.h = h;
+  if (S > 1) {
+    // every CTA of the cluster must have started before its buffer is written
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    cl.sync();
+    if (S == 2) pair_split<2>(L, io, a.sr, a.si, h);
+    else if (S == 4) pair_split<4>(L, io, a.sr, a.si, h);
+    else pair_split<8>(L, io, a.sr, a.si, h);
+    cl.sync();
+    pair_dispatch<CLS, 1, false>(L.radix[0], io, a);
+  } else {
+    pair_dispatch<CLS, 0, false>(L.radix[0], io, a);
+  }
+  a.Ns = L.radix[0];
+  int st = 1;
+  for (; st < L.nst - 1; ++st) {
+    a.tw = L.tw + 2 * L.twofs[st];
+    a.magic = L.magic[st];
+    pair_dispatch<CLS, 2, false>(L.radix[st], io, a);
+    a.Ns *= L.radix[st];
+  }
+  a.tw = L.tw + 2 * L.twofs[st];
+  pair_dispatch<CLS, 2, true>(L.radix[st], io, a);
+}
+
+// ---------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------
 static dd host_dd(long double v) {
@@ -531,12 +773,169 @@ static dd host_dd(long double v) {
   return x;
 }
 
+// One side's transform: pairs of lines where the side allows it, else one line per CTA / cluster.
+struct SideFft {
+  bool pairs = false;
+  PairLine pl;
+  FftLine fl;
+  float4* tw = nullptr;   // line twiddles, then (split lines) the decimation twiddles
+};
 struct Df64Fft {
   int nu = 0, nv = 0;
-  FftLine lu, lv;
-  float4* tw_u = nullptr;   // line twiddles, then (split lines) the decimation twiddles
-  float4* tw_v = nullptr;
+  SideFft u, v;
 };
+
+// FP32 operations per point of a radix-R butterfly in double-float arithmetic
+static double pair_radix_ops(int R) {
+  switch (R) {
+    case 2: return 22; case 3: return 50; case 4: return 44; case 5: return 86; case 6: return 72;
+    case 7: return 130; case 8: return 75; case 9: return 117; case 10: return 108;
+    case 11: return 190; default: return 97;
+  }
+}
+constexpr int pair_threads(int cls) { return cls == 9 ? 256 : 192; }   // CTA limit of a class
+// Cheapest radices of n points for a register class, largest first: butterflies, 38 per twiddle
+// product and about 60 per trip through shared memory (with its two barriers) from the second
+// stage on; at least two stages, the first of radix 8 or more, all within the class's CTA size.
+// Class 12 (168 registers) counts 1.25 times: 1728 points as 9 8 8 3 measured 1.11 times as fast
+// as 12 12 12, 480 as 8 6 5 2 1.05 times as fast as 12 10 4.
+static void pair_search(int m, int maxr, int depth, double cost, PairLine* cur, double* best,
+                        PairLine* out) {
+  if (m == 1) {
+    if (cur->cls == 12) cost *= 1.25;
+    if (cost >= *best || depth < 2 || cur->radix[0] < 8) return;
+    int T = 32;
+    for (int i = 0; i < depth; ++i) {
+      const int per = cur->n / cur->radix[i], nb = pair_nb(cur->cls, cur->radix[i]);
+      T = std::max(T, ((per + nb - 1) / nb + 31) / 32 * 32);
+    }
+    if (T > pair_threads(cur->cls)) return;
+    *best = cost;
+    *out = *cur;
+    out->nst = depth;
+    out->T = T;
+    return;
+  }
+  if (depth == kPairStages) return;
+  for (int R = std::min(maxr, cur->cls); R >= 2; --R) {
+    if (m % R != 0) continue;
+    cur->radix[depth] = R;
+    pair_search(m / R, R, depth + 1,
+                cost + pair_radix_ops(R) + (depth > 0 ? 38.0 * (R - 1) / R + 60.0 : 0.0), cur, best, out);
+  }
+}
+static bool pair_part(int N, int S, PairLine* L) {
+  if (N % S != 0 || N / S > kPairMaxPart) return false;
+  double best = 1e30;
+  for (int cls : {9, 12}) {
+    PairLine cur;
+    std::memset(&cur, 0, sizeof(cur));
+    cur.n = N / S; cur.S = S; cur.cls = cls;
+    pair_search(cur.n, cls, 0, 0.0, &cur, &best, L);
+  }
+  return best < 1e30;
+}
+// Radices, class and threads for a line of N points; false: the line kernels above.  Measured
+// against those on the pruned transforms of 68 square sides (forward / inverse): one CTA up to
+// 2048 points 0.9 - 1.5 / 1.1 - 4.2 times as fast (512: 7.2 -> 6.4 us and 14.0 -> 6.6 us per
+// plane).  A cluster of four beats two from 3072 points on where the parts are of class 9 and
+// at most 160 threads (3456: 1.10 / 1.06 against 1.06 / 1.02; 4096: 1.31 / 1.28 against 1.26 /
+// 1.21; 3840 in parts of 192 threads: 0.99 / 0.92 against 1.14 / 1.07).  Not better than one line
+// per CTA, and left to it: up to 2048 points what one CTA cannot take (2016: 0.89 / 0.93), and up
+// to 4096 points sides with a factor 11, or with 7 and 5 (3168: 1.01 / 0.89, 3360: 0.97 / 0.82).
+static bool pair_plan(int N, PairLine* L) {
+  if (N <= kPairMaxPart) return pair_part(N, 1, L);
+  if (N < 4096 && (N % 11 == 0 || N % 35 == 0)) return false;
+  if (N >= 3072 && pair_part(N, 4, L) && L->n <= 1024 && L->cls == 9 && L->T <= 160) return true;
+  for (int S : {2, 4, 8})
+    if (pair_part(N, S, L)) return true;
+  return false;
+}
+
+// e^{-2 pi i t / len} as a twiddle entry (each float twice)
+static void pair_entry(int64_t t, int64_t len, float4* e) {
+  // exact octant reduction, then sine and cosine of at most pi / 4 in double (1e-16, against the
+  // pairs' 2e-15)
+  t %= len;
+  const int64_t o = 8 * t / len;                 // octant 0 .. 7
+  const int64_t num = (o & 1) ? (o + 1) * len - 8 * t : 8 * t - o * len;   // distance to the nearer axis or diagonal, of 8 len
+  const double a = 0.78539816339744830962 * ((double)num / (double)len);
+  double c = std::cos(a), s = std::sin(a), cr, sr;
+  switch (o) {
+    case 0: cr = c; sr = s; break;
+    case 1: cr = s; sr = c; break;
+    case 2: cr = -s; sr = c; break;
+    case 3: cr = -c; sr = s; break;
+    case 4: cr = -c; sr = -s; break;
+    case 5: cr = -s; sr = -c; break;
+    case 6: cr = s; sr = -c; break;
+    default: cr = c; sr = -s; break;
+  }
+  sr = -sr;
+  const float ch = (float)cr, cl = (float)(cr - (double)ch), sh = (float)sr, sl = (float)(sr - (double)sh);
+  e[0] = make_float4(ch, ch, cl, cl);
+  e[1] = make_float4(sh, sh, sl, sl);
+}
+
+static cudaError_t make_pairs(PairLine* L, float4** tw) {
+  int entries = 0, Ns = 1;
+  for (int s = 0; s < L->nst; ++s) {
+    L->twofs[s] = entries;
+    L->magic[s] = Ns > 1 ? (unsigned)(0x100000000ull / (unsigned)Ns) + 1u : 0u;
+    if (Ns > 1) entries += (L->radix[s] - 1) * Ns;
+    Ns *= L->radix[s];
+  }
+  const int own = entries;
+  entries += (L->S - 1) * L->n;
+  std::vector<float4> h(2 * (size_t)std::max(1, entries));
+  Ns = 1;
+  for (int s = 0; s < L->nst; ++s) {
+    const int R = L->radix[s];
+    if (Ns > 1)
+      for (int k = 1; k < R; ++k)
+        for (int jm = 0; jm < Ns; ++jm)
+          pair_entry((int64_t)jm * k, (int64_t)Ns * R, &h[2 * (size_t)(L->twofs[s] + (k - 1) * Ns + jm)]);
+    Ns *= R;
+  }
+  for (int r = 1; r < L->S; ++r)
+    for (int j = 0; j < L->n; ++j)
+      pair_entry((int64_t)j * r, (int64_t)L->S * L->n, &h[2 * (size_t)(own + (r - 1) * L->n + j)]);
+  cudaError_t e = cudaMalloc((void**)tw, sizeof(float4) * h.size());
+  if (e != cudaSuccess) return e;
+  e = cudaMemcpy(*tw, h.data(), sizeof(float4) * h.size(), cudaMemcpyHostToDevice);
+  L->tw = *tw;
+  L->tw2 = *tw + 2 * own;
+  return e;
+}
+
+static cudaError_t launch_pairs(const PairLine& L, double2* data, int64_t batch, int64_t plane,
+                                int lines, int64_t line_stride, int64_t elem_stride, int fwd,
+                                int split, int skip, int lhalf, int shalf, cudaStream_t s) {
+  if (lines == 0 || batch == 0) return cudaSuccess;
+  const int64_t blocks = batch * ((lines + 1) / 2) * L.S;
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)L.T);
+  cfg.dynamicSmemBytes = 2 * sizeof(float4) * (size_t)((L.n + 7) & ~7);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  std::memset(attr, 0, sizeof(attr));
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)L.S;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = L.S > 1 ? 1 : 0;
+  float4* d = reinterpret_cast<float4*>(data);
+  const int inv = fwd ? 0 : 1;
+#define WG_PAIRS(C, TM)                                                                          \
+  cudaLaunchKernelEx(&cfg, k_fft_pairs<C, TM>, L, d, plane, lines, line_stride, elem_stride, inv, \
+                     split, skip, lhalf, shalf)
+  return L.cls == 9 ? WG_PAIRS(9, 256) : WG_PAIRS(12, 192);
+#undef WG_PAIRS
+}
 
 // Two buffers of n df64 complex values in shared memory per CTA (two CTAs per SM up to n =
 // 3584); split lines (df64_line_split) run on clusters of two or four CTAs.
@@ -595,34 +994,37 @@ static cudaError_t make_line(int nline, FftLine* L, float4** tw) {
   return cudaSuccess;
 }
 
+static cudaError_t make_side(int n, SideFft* f) {
+  f->pairs = pair_plan(n, &f->pl);
+  return f->pairs ? make_pairs(&f->pl, &f->tw) : make_line(n, &f->fl, &f->tw);
+}
+
 cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
   *out = nullptr;
   if (!df64_fft_supported(nu, nv)) return cudaErrorInvalidValue;
   Df64Fft* f = new Df64Fft();
   f->nu = (int)nu; f->nv = (int)nv;
-  cudaError_t e = make_line((int)nu, &f->lu, &f->tw_u);
-  if (e == cudaSuccess) e = make_line((int)nv, &f->lv, &f->tw_v);
+  cudaError_t e = make_side((int)nu, &f->u);
+  if (e == cudaSuccess) e = make_side((int)nv, &f->v);
   const int smax = (int)(2 * kMaxSide * sizeof(float4));
-#define WG_SMEM_ATTR(TM, MB, A, Y, P)                                                           \
-  if (e == cudaSuccess)                                                                          \
-    e = cudaFuncSetAttribute(k_fft_lines<TM, MB, A, Y, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)
-  WG_SMEM_ATTR(448, 2, false, false, false); WG_SMEM_ATTR(448, 2, false, true, false);
-  WG_SMEM_ATTR(448, 2, true, false, false);  WG_SMEM_ATTR(448, 2, true, true, false);
-  WG_SMEM_ATTR(832, 1, false, false, false); WG_SMEM_ATTR(832, 1, false, true, false);
-  WG_SMEM_ATTR(832, 1, true, false, false);  WG_SMEM_ATTR(832, 1, true, true, false);
-  WG_SMEM_ATTR(448, 2, false, false, true);  WG_SMEM_ATTR(448, 2, true, false, true);
-  WG_SMEM_ATTR(832, 1, false, false, true);  WG_SMEM_ATTR(832, 1, true, false, true);
+#define WG_SMEM_ATTR(K, BYTES)                                                                   \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, BYTES)
+  if (!f->u.pairs || !f->v.pairs) {
+    WG_SMEM_ATTR((k_fft_lines<448, 2, false, false, false>), smax); WG_SMEM_ATTR((k_fft_lines<448, 2, false, true, false>), smax);
+    WG_SMEM_ATTR((k_fft_lines<448, 2, true, false, false>), smax);  WG_SMEM_ATTR((k_fft_lines<448, 2, true, true, false>), smax);
+    WG_SMEM_ATTR((k_fft_lines<832, 1, false, false, false>), smax); WG_SMEM_ATTR((k_fft_lines<832, 1, false, true, false>), smax);
+    WG_SMEM_ATTR((k_fft_lines<832, 1, true, false, false>), smax);  WG_SMEM_ATTR((k_fft_lines<832, 1, true, true, false>), smax);
+    WG_SMEM_ATTR((k_fft_lines<448, 2, false, false, true>), smax);  WG_SMEM_ATTR((k_fft_lines<448, 2, true, false, true>), smax);
+    WG_SMEM_ATTR((k_fft_lines<832, 1, false, false, true>), smax);  WG_SMEM_ATTR((k_fft_lines<832, 1, true, false, true>), smax);
+    WG_SMEM_ATTR((k_fft_lines_cluster<448, 2, false>), smax); WG_SMEM_ATTR((k_fft_lines_cluster<448, 2, true>), smax);
+    WG_SMEM_ATTR((k_fft_lines_cluster<832, 1, false>), smax); WG_SMEM_ATTR((k_fft_lines_cluster<832, 1, true>), smax);
+  }
+  const int spair = (int)(2 * sizeof(float4) * kPairMaxPart);
+  WG_SMEM_ATTR((k_fft_pairs<9, 256>), spair);
+  WG_SMEM_ATTR((k_fft_pairs<12, 192>), spair);
 #undef WG_SMEM_ATTR
-#define WG_SMEM_ATTR_C(TM, MB, A)                                                                \
-  if (e == cudaSuccess)                                                                          \
-    e = cudaFuncSetAttribute(k_fft_lines_cluster<TM, MB, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax)
-  WG_SMEM_ATTR_C(448, 2, false); WG_SMEM_ATTR_C(448, 2, true);
-  WG_SMEM_ATTR_C(832, 1, false); WG_SMEM_ATTR_C(832, 1, true);
-#undef WG_SMEM_ATTR_C
   if (e != cudaSuccess) {
-    if (f->tw_u) cudaFree(f->tw_u);
-    if (f->tw_v) cudaFree(f->tw_v);
-    delete f;
+    df64_fft_destroy(f);
     return e;
   }
   *out = f;
@@ -631,8 +1033,8 @@ cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
 
 void df64_fft_destroy(Df64Fft* f) {
   if (f == nullptr) return;
-  if (f->tw_u) cudaFree(f->tw_u);
-  if (f->tw_v) cudaFree(f->tw_v);
+  if (f->u.tw) cudaFree(f->u.tw);
+  if (f->v.tw) cudaFree(f->v.tw);
   delete f;
 }
 
@@ -706,6 +1108,30 @@ static cudaError_t launch_lines(const FftLine& L, double2* data, int64_t batch, 
   return cudaGetLastError();
 }
 
+static cudaError_t launch_side(const SideFft& f, double2* data, int64_t batch, int64_t plane,
+                               int lines, int64_t line_stride, int64_t elem_stride, int mode,
+                               int fwd, int split, int skip, int lhalf, int shalf, cudaStream_t s) {
+  return f.pairs ? launch_pairs(f.pl, data, batch, plane, lines, line_stride, elem_stride, fwd, split,
+                                skip, lhalf, shalf, s)
+                 : launch_lines(f.fl, data, batch, plane, lines, line_stride, elem_stride, mode, fwd,
+                                split, skip, lhalf, shalf, s);
+}
+
+// complex128 planes to float pairs and back, in place (the FFT utilities; the plans keep pairs)
+__global__ void k_to_pairs(double2* __restrict__ data, int64_t count, int back) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (back) {
+      const float4 v = reinterpret_cast<const float4*>(data)[i];
+      data[i] = make_double2(join_double(dd_make(v.x, v.y)), join_double(dd_make(v.z, v.w)));
+    } else {
+      const double2 d = data[i];
+      const dd r = split_double(d.x), m = split_double(d.y);
+      reinterpret_cast<float4*>(data)[i] = make_float4(r.h, r.l, m.h, m.l);
+    }
+  }
+}
+
 // In-place transform of `batch` nu x nv complex128 planes; sign -1 forward, +1 inverse.
 // df64_planes: the planes on the grid side are double-float pairs (float4 per complex value:
 // re hi, re lo, im hi, im lo) instead of doubles -- the forward transform's output and the
@@ -729,16 +1155,25 @@ cudaError_t df64_fft_exec(Df64Fft* f, double2* data, int64_t batch, int sign, cu
     return cudaErrorInvalidValue;
   // pass modes: 0 loads doubles and stores pairs, 1 loads pairs and stores doubles, 2 pairs
   // in and out; the grid side is the forward output / inverse input, the image side the other
-  const int img_in = image_pairs ? 2 : 0, img_out = image_pairs ? 2 : 1;
-  const int uv_in = df64_planes ? 2 : 0, uv_out = df64_planes ? 2 : 1;
+  // the line-pair kernels take and give pairs only: complex128 data are converted around them
+  const bool conv = f->u.pairs || f->v.pairs;
+  const int img_in = image_pairs || conv ? 2 : 0, img_out = image_pairs || conv ? 2 : 1;
+  const int uv_in = df64_planes || conv ? 2 : 0, uv_out = df64_planes || conv ? 2 : 1;
   cudaError_t e;
+  const bool in_pairs = fwd ? image_pairs : df64_planes, out_pairs = fwd ? df64_planes : image_pairs;
+  auto convert = [&](int back) {
+    k_to_pairs<<<152 * 8, 256, 0, s>>>(data, batch * plane, back);
+    return cudaGetLastError();
+  };
+  if (conv && !in_pairs && (e = convert(0)) != cudaSuccess) return e;
+  auto done = [&](cudaError_t r) { return r == cudaSuccess && conv && !out_pairs ? convert(1) : r; };
   if (!prune) {
     // rows (length nv, contiguous), then columns (length nu, stride nv)
-    e = launch_lines(f->lv, data, batch, plane, f->nu, f->nv, 1, fwd ? img_in : uv_in, fwd,
+    e = launch_side(f->v, data, batch, plane, f->nu, f->nv, 1, fwd ? img_in : uv_in, fwd,
                      f->nu, 0, f->nv, f->nv, s);
     if (e != cudaSuccess) return e;
-    return launch_lines(f->lu, data, batch, plane, f->nv, 1, f->nv, fwd ? uv_out : img_out, fwd,
-                        f->nv, 0, f->nu, f->nu, s);
+    return done(launch_side(f->u, data, batch, plane, f->nv, 1, f->nv, fwd ? uv_out : img_out, fwd,
+                            f->nv, 0, f->nu, f->nu, s));
   }
   const int rh = (int)(keep_rows / 2);   // image half-extent along u (rows)
   const int ch = (int)(keep_cols / 2);   // along v (columns)
@@ -746,17 +1181,17 @@ cudaError_t df64_fft_exec(Df64Fft* f, double2* data, int64_t batch, int sign, cu
   if (fwd) {
     // image columns (length nu, stride nv), image rows loaded; then all rows (length nv),
     // image columns loaded
-    e = launch_lines(f->lu, data, batch, plane, ncols, 1, f->nv, img_in, fwd, ch, cskip, rh,
+    e = launch_side(f->u, data, batch, plane, ncols, 1, f->nv, img_in, fwd, ch, cskip, rh,
                      f->nu, s);
     if (e != cudaSuccess) return e;
-    return launch_lines(f->lv, data, batch, plane, f->nu, f->nv, 1, uv_out, fwd, f->nu, 0, ch,
-                        f->nv, s);
+    return done(launch_side(f->v, data, batch, plane, f->nu, f->nv, 1, uv_out, fwd, f->nu, 0, ch,
+                            f->nv, s));
   }
   // inverse: all rows, image columns stored; then the image columns, image rows stored
-  e = launch_lines(f->lv, data, batch, plane, f->nu, f->nv, 1, uv_in, fwd, f->nu, 0, f->nv, ch, s);
+  e = launch_side(f->v, data, batch, plane, f->nu, f->nv, 1, uv_in, fwd, f->nu, 0, f->nv, ch, s);
   if (e != cudaSuccess) return e;
-  return launch_lines(f->lu, data, batch, plane, ncols, 1, f->nv, img_out, fwd, ch, cskip, f->nu,
-                      rh, s);
+  return done(launch_side(f->u, data, batch, plane, ncols, 1, f->nv, img_out, fwd, ch, cskip, f->nu,
+                          rh, s));
 }
 
 }  // namespace wg

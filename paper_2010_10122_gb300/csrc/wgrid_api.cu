@@ -1171,14 +1171,16 @@ static int fft_util_make(FftUtil& u, int64_t nu, int64_t nv, int64_t batch, int 
   return WG_OK;
 }
 
-static int fft_util_exec(FftUtil& u, void* data, int64_t batch, int precision, int sign, cudaStream_t s) {
+// pairs: the double-float FFT's data are float pairs (as in the plans), not complex128
+static int fft_util_exec(FftUtil& u, void* data, int64_t batch, int precision, int sign, cudaStream_t s,
+                         bool pairs = false) {
   if (u.f != nullptr) {
     cudaError_t e = f32_fft_exec(u.f, (float2*)data, batch, sign, s);
     if (e != cudaSuccess) return set_error(WG_ERR_CUDA, "FP32 FFT: %s", cudaGetErrorString(e));
     return WG_OK;
   }
   if (u.d != nullptr) {
-    cudaError_t e = df64_fft_exec(u.d, (double2*)data, batch, sign, s);
+    cudaError_t e = df64_fft_exec(u.d, (double2*)data, batch, sign, s, 0, 0, pairs, pairs);
     if (e != cudaSuccess) return set_error(WG_ERR_CUDA, "double-float FFT: %s", cudaGetErrorString(e));
     return WG_OK;
   }
@@ -1227,7 +1229,7 @@ int wg_fft_time(int64_t n, int precision, int64_t batch, int reps, int impl, dou
     float ms = 0.f;
     for (int r = 0; r <= reps && rc == WG_OK; ++r) {
       if (r == 1) cudaEventRecord(e0, 0);
-      rc = fft_util_exec(u, data, batch, precision, -1, 0);
+      rc = fft_util_exec(u, data, batch, precision, -1, 0, true);
     }
     if (rc != WG_OK) break;
     cudaEventRecord(e1, 0);

@@ -101,6 +101,23 @@ def test_f32_fft_shapes(wg, tune, sign):
         wg.wgrid.fft_f32_tune(0, 0, 0)
 
 
+@pytest.mark.parametrize("shape", [(2, 15, 16), (1, 9, 256), (1, 33, 704), (3, 7, 1440), (1, 1728, 15),
+                                   (1, 2048, 3), (1, 5, 3072), (1, 3456, 21), (1, 27, 3840),
+                                   (1, 6144, 5), (1, 11, 5632), (1, 8192, 9), (1, 3, 12288)])
+@pytest.mark.parametrize("sign", [-1, 1])
+def test_df64_line_pairs_against_numpy(wg, shape, sign):
+    """The kernels that transform two lines at once: both register classes (radices up to 9, and
+    10 to 12), whole lines and lines split over clusters of 2, 4 and 8 CTAs, rows and strided
+    columns, an odd number of lines (the last one alone in its pair).  The bound is the FFT's own:
+    normwise 5e-14."""
+    rng = np.random.default_rng(sum(shape) + 3 * sign)
+    x = rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
+    a = torch.from_numpy(x).cuda()
+    wg.wgrid.fft2d(a, sign=sign, impl=2)
+    ref = np.fft.fft2(x) if sign < 0 else np.fft.ifft2(x) * (shape[1] * shape[2])
+    assert np.linalg.norm(a.cpu().numpy() - ref) / np.linalg.norm(ref) < 5e-14
+
+
 def test_df64_rejects_unsupported(wg):
     a = torch.zeros((1, 64, 64), dtype=torch.complex64, device="cuda")
     with pytest.raises(wg.WgridError):
