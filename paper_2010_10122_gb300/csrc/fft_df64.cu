@@ -619,42 +619,74 @@ struct PairStageArgs {
 // from the buffer that the decimation step has filled (both without twiddles); 2 a later stage.
 // kLast: results to global memory.  (Separate instances: with both destinations in one body the
 // compiler keeps the results in registers for both and spills.)
+// Idle lanes of a warp repeat the last butterfly and store nothing, and the barrier between
+// reading and writing stands inside the branch that skips idle warps: points that live across
+// the end of a branch are spilled, all of them.
+template <int R, int kIn, bool kLast>
+__device__ __forceinline__ int pair_compute(const PairIo& io, const PairStageArgs& a, int j, int M,
+                                            int Ns, Cx<d2>* x) {
+#pragma unroll
+  for (int k = 0; k < R; ++k)
+    x[k] = kIn == 0 ? io.load(j + k * M) : pair_get(a.sr, a.si, j + k * M);
+  int o = j * R;
+  if constexpr (kIn == 2) {
+    const int jq = kLast ? 0 : (int)__umulhi((unsigned)j, a.magic), jm = j - jq * Ns;
+    o = jq * Ns * R + jm;
+#pragma unroll
+    for (int k = 1; k < R; ++k) x[k] = cx_mul(x[k], pair_tw(a.tw, jm + (k - 1) * Ns));
+  }
+  dft<R>(x);
+  return o;
+}
+template <int R, bool kLast>
+__device__ __forceinline__ void pair_result(const PairIo& io, const PairStageArgs& a, int o, int Ns,
+                                            const Cx<d2>* x) {
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    if (kLast) io.store(a.S * (o + q * Ns) + a.h, x[q]);
+    else pair_put(a.sr, a.si, o + q * Ns, x[q]);
+  }
+}
+// all warps of the CTA arrive, from either side of a warp-uniform branch
+__device__ __forceinline__ void pair_barrier() { asm volatile("barrier.sync 0;" ::: "memory"); }
+
+// NB: butterflies per thread, exactly as many as the CTA's threads need (idle rounds cost as much
+// as full ones)
+template <int R, int NB, int kIn, bool kLast>
+__device__ __forceinline__ void pair_stage_nb(const PairIo& io, const PairStageArgs& a) {
+  constexpr bool kWait = kIn != 0 && !kLast;   // every point of the buffer is read before it is written
+  const int M = a.n / R, T = blockDim.x, Ns = kIn == 2 ? a.Ns : 1;
+  if constexpr (NB == 1) {
+    const int j = threadIdx.x;
+    if ((j & ~31) < M) {
+      Cx<d2> x[R];
+      const int o = pair_compute<R, kIn, kLast>(io, a, min(j, M - 1), M, Ns, x);
+      if (kWait) pair_barrier();
+      if (j < M) pair_result<R, kLast>(io, a, o, Ns, x);
+    } else if (kWait) {
+      pair_barrier();
+    }
+  } else {
+    Cx<d2> x[NB][R];
+    int o[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+      o[b] = pair_compute<R, kIn, kLast>(io, a, min((int)threadIdx.x + b * T, M - 1), M, Ns, x[b]);
+    if (kWait) pair_barrier();
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+      if ((int)threadIdx.x + b * T < M) pair_result<R, kLast>(io, a, o[b], Ns, x[b]);
+  }
+  if (!kLast) pair_barrier();
+}
 template <int R, int CLS, int kIn, bool kLast>
 __device__ __forceinline__ void pair_stage(const PairIo& io, const PairStageArgs& a) {
-  constexpr int NB = pair_nb(CLS, R);
-  const int M = a.n / R, T = blockDim.x, Ns = kIn == 2 ? a.Ns : 1;
-  Cx<d2> x[NB][R];
-  int o[NB];
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    const int j = threadIdx.x + b * T;
-    if (j < M) {
-#pragma unroll
-      for (int k = 0; k < R; ++k)
-        x[b][k] = kIn == 0 ? io.load(j + k * M) : pair_get(a.sr, a.si, j + k * M);
-      o[b] = j * R;
-      if constexpr (kIn == 2) {
-        const int jq = kLast ? 0 : (int)__umulhi((unsigned)j, a.magic), jm = j - jq * Ns;
-        o[b] = jq * Ns * R + jm;
-#pragma unroll
-        for (int k = 1; k < R; ++k) x[b][k] = cx_mul(x[b][k], pair_tw(a.tw, jm + (k - 1) * Ns));
-      }
-      dft<R>(x[b]);
-    }
-  }
-  if (kIn != 0 && !kLast) __syncthreads();   // every point of the buffer has been read
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    const int j = threadIdx.x + b * T;
-    if (j < M) {
-#pragma unroll
-      for (int q = 0; q < R; ++q) {
-        if (kLast) io.store(a.S * (o[b] + q * Ns) + a.h, x[b][q]);
-        else pair_put(a.sr, a.si, o[b] + q * Ns, x[b][q]);
-      }
-    }
-  }
-  if (!kLast) __syncthreads();
+  constexpr int kMost = pair_nb(CLS, R);
+  const int M = a.n / R, T = blockDim.x;
+  if (kMost == 1 || M <= T) pair_stage_nb<R, 1, kIn, kLast>(io, a);
+  else if (kMost == 2 || M <= 2 * T) pair_stage_nb<R, kMost < 2 ? 1 : 2, kIn, kLast>(io, a);
+  else if (kMost == 3 || M <= 3 * T) pair_stage_nb<R, kMost < 3 ? 1 : 3, kIn, kLast>(io, a);
+  else pair_stage_nb<R, kMost < 4 ? 1 : kMost, kIn, kLast>(io, a);
 }
 template <int CLS, int kIn, bool kLast>
 __device__ __forceinline__ void pair_dispatch(int R, const PairIo& io, const PairStageArgs& a) {
@@ -785,24 +817,25 @@ struct Df64Fft {
   SideFft u, v;
 };
 
-// FP32 operations per point of a radix-R butterfly in double-float arithmetic
+// FP32 operations per point of a radix-R butterfly in double-float arithmetic (5, 10 and 12 as
+// they measure, 10 % above their count)
 static double pair_radix_ops(int R) {
   switch (R) {
-    case 2: return 22; case 3: return 50; case 4: return 44; case 5: return 86; case 6: return 72;
-    case 7: return 130; case 8: return 75; case 9: return 117; case 10: return 108;
-    case 11: return 190; default: return 97;
+    case 2: return 22; case 3: return 50; case 4: return 44; case 5: return 95; case 6: return 72;
+    case 7: return 130; case 8: return 75; case 9: return 117; case 10: return 118;
+    case 11: return 190; default: return 108;
   }
 }
 constexpr int pair_threads(int cls) { return cls == 9 ? 256 : 192; }   // CTA limit of a class
 // Cheapest radices of n points for a register class, largest first: butterflies, 38 per twiddle
-// product and about 60 per trip through shared memory (with its two barriers) from the second
+// product and about 75 per trip through shared memory (with its two barriers) from the second
 // stage on; at least two stages, the first of radix 8 or more, all within the class's CTA size.
-// Class 12 (168 registers) counts 1.25 times: 1728 points as 9 8 8 3 measured 1.11 times as fast
-// as 12 12 12, 480 as 8 6 5 2 1.05 times as fast as 12 10 4.
+// Class 12 (168 registers) counts 1.18 times: it pays where it saves a stage (1200 points as 12 10
+// 10 measured 1.2 times as fast as 8 6 5 5), else not (1344 as 12 7 4 4: 0.85 of 8 7 6 4).
 static void pair_search(int m, int maxr, int depth, double cost, PairLine* cur, double* best,
                         PairLine* out) {
   if (m == 1) {
-    if (cur->cls == 12) cost *= 1.25;
+    if (cur->cls == 12) cost *= 1.18;
     if (cost >= *best || depth < 2 || cur->radix[0] < 8) return;
     int T = 32;
     for (int i = 0; i < depth; ++i) {
@@ -821,7 +854,7 @@ static void pair_search(int m, int maxr, int depth, double cost, PairLine* cur, 
     if (m % R != 0) continue;
     cur->radix[depth] = R;
     pair_search(m / R, R, depth + 1,
-                cost + pair_radix_ops(R) + (depth > 0 ? 38.0 * (R - 1) / R + 60.0 : 0.0), cur, best, out);
+                cost + pair_radix_ops(R) + (depth > 0 ? 38.0 * (R - 1) / R + 75.0 : 0.0), cur, best, out);
   }
 }
 static bool pair_part(int N, int S, PairLine* L) {
@@ -836,16 +869,16 @@ static bool pair_part(int N, int S, PairLine* L) {
   return best < 1e30;
 }
 // Radices, class and threads for a line of N points; false: the line kernels above.  Measured
-// against those on the pruned transforms of 68 square sides (forward / inverse): one CTA up to
-// 2048 points 0.9 - 1.5 / 1.1 - 4.2 times as fast (512: 7.2 -> 6.4 us and 14.0 -> 6.6 us per
-// plane).  A cluster of four beats two from 3072 points on where the parts are of class 9 and
-// at most 160 threads (3456: 1.10 / 1.06 against 1.06 / 1.02; 4096: 1.31 / 1.28 against 1.26 /
-// 1.21; 3840 in parts of 192 threads: 0.99 / 0.92 against 1.14 / 1.07).  Not better than one line
-// per CTA, and left to it: up to 2048 points what one CTA cannot take (2016: 0.89 / 0.93), and up
-// to 4096 points sides with a factor 11, or with 7 and 5 (3168: 1.01 / 0.89, 3360: 0.97 / 0.82).
+// against those on the pruned transforms of square sides (forward / inverse, per plane): one CTA
+// up to 2048 points (512: 7.1 -> 5.9 and 14.0 -> 6.2 us; 2048: 139 -> 108 and 150 -> 107 us).  From
+// 3072 points on a cluster of four beats two where the parts are of class 9 and at most 160
+// threads (3584: 1.23 / 1.11 times the line kernels' speed against 1.12 / 1.04; 3840 in parts of 192
+// threads 1.04 / 0.97 against 1.11 / 1.07).  Left to one line per CTA, which is as fast or faster: up
+// to 2048 points what one CTA cannot take (2016: 0.89 / 0.93), and between 3072 and 4096 points
+// sides with a factor 11, or with 7 and 5 (3168: 1.08 / 0.95, 3520: 0.98 / 0.91, 3360: 1.02 / 0.86).
 static bool pair_plan(int N, PairLine* L) {
   if (N <= kPairMaxPart) return pair_part(N, 1, L);
-  if (N < 4096 && (N % 11 == 0 || N % 35 == 0)) return false;
+  if (N > 3072 && N < 4096 && (N % 11 == 0 || N % 35 == 0)) return false;
   if (N >= 3072 && pair_part(N, 4, L) && L->n <= 1024 && L->cls == 9 && L->T <= 160) return true;
   for (int S : {2, 4, 8})
     if (pair_part(N, S, L)) return true;

@@ -1,17 +1,16 @@
-// Register-level DFT building blocks shared by the plane FFTs, on values that carry TWO lines at
-// once: every scalar is a packed pair of floats (one per line) and every operation a packed FP32
-// instruction (add / sub / mul / fma .f32x2).
+// Register-level DFT building blocks of the double-float plane FFT, on values that carry TWO lines
+// at once: every scalar is a packed pair of floats (one per line) and every operation a packed
+// FP32 instruction (add / sub / mul / fma .f32x2).
 //
 // Why pairs of lines: GB300's packed FP32 instructions run at the same lane rate as the scalar
 // ones (measured 39.7 T against 38.4 T operations/s) but take one issue slot for two operations,
-// and the line kernels were bound by issue: 785 warp-lane instructions per element and pass for
-// 460 FP32 operations in the double-float transform, 170 for about 55 in the FP32 one.  With two
-// lines side by side the arithmetic needs half the slots, and one address computation, one
-// shared-memory access pattern and one twiddle load serve both lines; inside a line (real and
-// imaginary part packed together) every rotation by i and every complex product would need moves.
+// and the line kernels were bound by issue (785 instructions per element and pass for 460 FP32
+// operations).  With two lines side by side the arithmetic needs half the slots, and one address
+// computation, one shared-memory access pattern and one twiddle load serve both lines; inside a
+// line (real and imaginary part packed together) every rotation by i and every complex product
+// would need moves.
 //
-// S is the scalar type: f2 (FP32) or d2 (double-float, an unevaluated sum of two floats).  All
-// transforms are forward (e^{-2 pi i}); the inverse is the forward transform with real and
+// All transforms are forward (e^{-2 pi i}); the inverse is the forward transform with real and
 // imaginary parts exchanged on load and on store.
 #pragma once
 #include <cuda_runtime.h>
@@ -110,8 +109,6 @@ __host__ __device__ constexpr double cos2pi(int k, int N) {
 
 struct Konst { double v; };   // a real constant, rounded to the scalar type where it is used
 
-__device__ __forceinline__ f2 s_mulk(f2 a, const Konst k) { return s_mul(a, f2_dup((float)k.v)); }
-__device__ __forceinline__ f2 s_fmak(f2 a, const Konst k, f2 c) { return s_fma(a, f2_dup((float)k.v), c); }
 // a * k: p - n with p the rounded product of the high parts and n minus everything below it
 __device__ __forceinline__ d2 s_mulk(d2 a, const Konst k) {
   const float kh = (float)k.v, kl = (float)(k.v - (double)kh);
@@ -137,7 +134,6 @@ __device__ __forceinline__ d2 s_fmak(d2 a, const Konst k, d2 c) {
   return d2_fast_two_sum(s.h, s_add(s.l, s_sub(c.l, n)));
 }
 // c - a / 2 (the half is exact)
-__device__ __forceinline__ f2 s_submhalf(f2 c, f2 a) { return s_fma(a, f2_dup(-0.5f), c); }
 __device__ __forceinline__ d2 s_submhalf(d2 c, d2 a) {
   d2 m;
   m.h = s_mul(a.h, f2_dup(0.5f));
@@ -166,13 +162,8 @@ template <class S> __device__ __forceinline__ Cx<S> cx_mulk(const Cx<S>& a, cons
 
 // Twiddle factors as loaded from the tables: every float twice (one per line).
 template <class S> struct Tw;
-template <> struct Tw<f2> { f2 r, i; };
 template <> struct Tw<d2> { f2 rh, rl, ih, il; };
 
-__device__ __forceinline__ Cx<f2> cx_mul(const Cx<f2>& a, const Tw<f2>& w) {
-  const f2 ni = s_mul(w.i, f2_dup(-1.0f));
-  return Cx<f2>{s_fma(a.r, w.r, s_mul(a.i, ni)), s_fma(a.r, w.i, s_mul(a.i, w.r))};
-}
 // x u + y v with the cross terms, one normalised pair: both leading products are split exactly
 // (n1, n2 are minus their errors), summed exactly, the small terms accumulated in float.
 // nuh, nvh: -u.h, -v.h.
@@ -194,12 +185,6 @@ __device__ __forceinline__ Cx<d2> cx_mul(const Cx<d2>& a, const Tw<d2>& w) {
                 d2_dot(a.r, w.ih, nih, w.il, a.i, w.rh, nrh, w.rl)};
 }
 // a e^{-2 pi i k / N} for compile-time k, N
-template <int N, int K>
-__device__ __forceinline__ Cx<f2> cx_root(const Cx<f2>& a) {
-  constexpr double c = trig::cos2pi(K, N), s = trig::sin2pi(K, N);
-  const f2 C = f2_dup((float)c), Sn = f2_dup((float)s), nS = f2_dup((float)-s);
-  return Cx<f2>{s_fma(a.r, C, s_mul(a.i, Sn)), s_fma(a.i, C, s_mul(a.r, nS))};
-}
 template <int N, int K>
 __device__ __forceinline__ Cx<d2> cx_root(const Cx<d2>& a) {
   constexpr double c = trig::cos2pi(K, N), s = -trig::sin2pi(K, N);
@@ -354,10 +339,7 @@ template <int R, class S> __device__ __forceinline__ void dft(Cx<S>* x) {
   else if constexpr (R == 8) dft_8(x);
   else if constexpr (R == 9) dft_product<3, 3>(x);
   else if constexpr (R == 10) dft_coprime<5, 2>(x);
-  else if constexpr (R == 12) dft_coprime<3, 4>(x);
-  else if constexpr (R == 14) dft_coprime<7, 2>(x);
-  else if constexpr (R == 15) dft_coprime<5, 3>(x);
-  else if constexpr (R == 16) dft_product<4, 4>(x);
+  else dft_coprime<3, 4>(x);   // 12
 }
 
 }  // namespace wg
