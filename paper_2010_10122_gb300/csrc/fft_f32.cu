@@ -366,11 +366,18 @@ bool f32_line_shape(int N, int C, const F32Tune& tu, F32Lines* L) {
   return false;
 }
 
+// e^{-2 pi i t / len} rounded from double (a long double sine costs microseconds where it is
+// computed in software): an eighth of the turn, and the other octants by symmetry, so that no
+// argument above pi / 4 is rounded
 void host_twiddles(int len, int count, float2* h) {
-  const long double two_pi = 6.283185307179586476925286766559L;
   for (int t = 0; t < count; ++t) {
-    const long double a = two_pi * (long double)t / (long double)len;
-    h[t] = make_float2((float)cosl(a), (float)-sinl(a));
+    const int64_t o = 8 * (int64_t)t / len;
+    const int64_t num = (o & 1) ? (o + 1) * len - 8 * (int64_t)t : 8 * (int64_t)t - o * len;
+    const double a = 0.78539816339744830962 * ((double)num / (double)len);
+    const float c = (float)std::cos(a), s = (float)std::sin(a);
+    const bool swap = o == 1 || o == 2 || o == 5 || o == 6;
+    const float x = swap ? s : c, y = swap ? c : s;
+    h[t] = make_float2(o >= 2 && o <= 5 ? -x : x, o >= 4 ? y : -y);
   }
 }
 

@@ -6,6 +6,10 @@
 #include <cstdio>
 #include <cstring>
 #include <limits>
+#include <map>
+#include <memory>
+#include <mutex>
+#include <tuple>
 
 namespace wg {
 
@@ -241,6 +245,23 @@ std::vector<double> psi_cheb_coeffs(const PolyKernel& K, int m) {
   return c;
 }
 
+const KernelMath& kernel_math(int alpha, double beta, double mu) {
+  static std::mutex m;
+  static std::map<std::tuple<int, double, double>, std::unique_ptr<const KernelMath>> known;
+  const auto key = std::make_tuple(alpha, beta, mu);
+  {
+    std::lock_guard<std::mutex> lk(m);
+    auto it = known.find(key);
+    if (it != known.end()) return *it->second;
+  }
+  std::unique_ptr<KernelMath> k(new KernelMath());
+  k->poly = make_poly_kernel(alpha, beta, mu, alpha + 3);
+  k->psi = psi_cheb_coeffs(k->poly, kPsiChebTerms);
+  std::lock_guard<std::mutex> lk(m);
+  auto it = known.emplace(key, std::move(k)).first;   // another thread's, if it was first
+  return *it->second;
+}
+
 double psi_cheb_eval(const std::vector<double>& c, double k) {
   double y = 8.0 * k * k - 1.0;
   double b1 = 0.0, b2 = 0.0;
@@ -421,9 +442,7 @@ static double fft_ms_square(int64_t n, int kind, int prec) {
 // per line) and the pruned loads / stores of its row pass leave 0.15 + 0.85 x the image
 // fraction of the full transform (measured on GB300: 0.542 ms for a 3456^2 plane with a 2048^2
 // image, against 0.828 ms for the full transform).
-static double fft_ms(int64_t nu, int64_t nv, int kind, int prec, int64_t nx, int64_t ny) {
-  double cu = fft_ms_square(nu, kind, prec) / ((double)nu * nu);
-  double cv = fft_ms_square(nv, kind, prec) / ((double)nv * nv);
+static double fft_ms_cells(int64_t nu, int64_t nv, double cu, double cv, int kind, int64_t nx, int64_t ny) {
   double full = 0.5 * (cu + cv) * (double)nu * nv;
   // image fraction of a side, the geometric mean over the two (square planes: nx / nu); a single
   // side's fraction would favour a plane longer in that direction
@@ -434,6 +453,13 @@ static double fft_ms(int64_t nu, int64_t nv, int kind, int prec, int64_t nx, int
   // bytes (column pass: f^2 loaded, f stored; row pass: f loaded, 1 stored; f = image fraction)
   if (kind == kFftF32) return full * (1.0 + frac) * (1.0 + frac) / 4.0;
   return full;
+}
+// milliseconds per cell of a side
+static double fft_ms_per_cell(int64_t n, int kind, int prec) {
+  return fft_ms_square(n, kind, prec) / ((double)n * n);
+}
+static double fft_ms(int64_t nu, int64_t nv, int kind, int prec, int64_t nx, int64_t ny) {
+  return fft_ms_cells(nu, nv, fft_ms_per_cell(nu, kind, prec), fft_ms_per_cell(nv, kind, prec), kind, nx, ny);
 }
 
 static bool kind_supports(int kind, int64_t n) {
@@ -482,12 +508,24 @@ static bool choose_grid(int64_t nmin_u, int64_t nmin_v, int prec, int kind, int6
                         int64_t nx, int64_t ny, int64_t* nu, int64_t* nv) {
   double k_cell = prec ? 3.0e-12 : 2.5e-12;
   double best = std::numeric_limits<double>::infinity();
-  for (int64_t a : size_candidates(nmin_u, mult, kind))
-    for (int64_t b : size_candidates(nmin_v, mult, kind)) {
-      double c = 1e-3 * fft_ms(a, b, kind, prec, nx, ny) + k_cell * (double)a * b;
+  const std::vector<int64_t> ca = size_candidates(nmin_u, mult, kind), cb = size_candidates(nmin_v, mult, kind);
+  std::vector<double> mb(cb.size());   // each side's table look-up once, not once per pair
+  for (size_t j = 0; j < cb.size(); ++j) mb[j] = fft_ms_per_cell(cb[j], kind, prec);
+  for (int64_t a : ca) {
+    const double ma = fft_ms_per_cell(a, kind, prec);
+    for (size_t j = 0; j < cb.size(); ++j) {
+      const int64_t b = cb[j];
+      double c = 1e-3 * fft_ms_cells(a, b, ma, mb[j], kind, nx, ny) + k_cell * (double)a * b;
       if (c < best) { best = c; *nu = a; *nv = b; }
     }
+  }
   return std::isfinite(best);
+}
+
+bool short_setup_fft(const PlanParams& p, int prec, int64_t nx, int64_t ny) {
+  if (prec != 0 || p.fft_kind != kFftCufft2d || !f32_side_ok(p.nu) || !f32_side_ok(p.nv)) return false;
+  const double more = fft_ms(p.nu, p.nv, kFftF32, prec, nx, ny) - fft_ms(p.nu, p.nv, kFftCufft2d, prec, nx, ny);
+  return p.nw * more < kCufftSetupMs;
 }
 
 int choose_plan(const PlanInput& in, PlanParams& out, char* err, int errlen) {
@@ -526,8 +564,9 @@ int choose_plan(const PlanInput& in, PlanParams& out, char* err, int errlen) {
   best.cost = std::numeric_limits<double>::infinity();
   // kernels: the App. A table (alpha 4, 7, 8, 12, 16) and the searched ones for the other
   // supports (kernel_design.cpp)
-  std::vector<KernelRow> T = kernel_table();
-  for (const auto& r : kernel_table_design()) T.push_back(r);
+  std::vector<const KernelRow*> T;
+  for (const auto& r : kernel_table()) T.push_back(&r);
+  for (const auto& r : kernel_table_design()) T.push_back(&r);
   for (int alpha = 4; alpha <= kMaxAlpha; ++alpha) {
     if (in.force_alpha > 0 && alpha != in.force_alpha) continue;
     // uv tile side: 32 cells; 16 for FP64 kernels wider than 8 (16-lane groups), whose
@@ -535,16 +574,20 @@ int choose_plan(const PlanInput& in, PlanParams& out, char* err, int errlen) {
     int tile = in.tile > 0 ? in.tile : ((in.prec == 1 && alpha > 8) ? 16 : 32);
     if (alpha - 1 > tile) continue;
     std::vector<const KernelRow*> rows;
-    for (const auto& r : T) {
-      if (r.alpha != alpha) continue;
-      if (in.force_sigma > 0 && std::fabs(r.sigma - in.force_sigma) > 1e-9) continue;
-      if (r.eps <= in.eps * safety) rows.push_back(&r);
+    for (const KernelRow* r : T) {
+      if (r->alpha != alpha) continue;
+      if (in.force_sigma > 0 && std::fabs(r->sigma - in.force_sigma) > 1e-9) continue;
+      if (r->eps <= in.eps * safety) rows.push_back(r);
     }
     std::sort(rows.begin(), rows.end(),
               [](const KernelRow* a, const KernelRow* b) { return a->sigma < b->sigma; });
     for (int kind : kinds) {
       // Sec. 4.1: for each alpha the smallest sigma whose kernel meets epsilon -- here the
-      // kernel term together with the plane rounding of this FFT kind (unless sigma is forced)
+      // kernel term together with the plane rounding of this FFT kind (unless sigma is forced).
+      // Grids and costs first: the predicted error takes the kernel's transform and a lattice of
+      // pixels (about a millisecond), and is formed only for candidates up to the last one that
+      // would be cheaper than the best plan so far
+      std::vector<PlanParams> cand;
       for (const KernelRow* pick : rows) {
         PlanParams p;
         p.alpha = alpha; p.sigma = pick->sigma; p.beta = pick->beta; p.mu = pick->mu;
@@ -583,15 +626,20 @@ int choose_plan(const PlanInput& in, PlanParams& out, char* err, int errlen) {
           p.nshift = 0.0; p.dw = 1.0; p.w0 = 0.0; p.nw = 1;
         }
         if (p.nw > 4095) break;  // plane index must fit 12 bits (FP32 phase split)
-        PolyKernel K = make_poly_kernel(alpha, p.beta, p.mu, alpha + 3);
-        std::vector<double> pc = psi_cheb_coeffs(K, kPsiChebTerms);
-        p.gain = rounding_gain(K, pc, in.nx, in.ny, in.psx, in.psy, p.nu, p.nv, in.do_w,
+        p.cost = plan_cost(in.prec, kind, p.nu, p.nv, p.nw, alpha, in.nvis, in.nx, in.ny);
+        cand.push_back(p);
+      }
+      size_t end = cand.size();
+      while (end > 0 && !(cand[end - 1].cost < best.cost)) --end;
+      for (size_t i = 0; i < end; ++i) {
+        PlanParams& p = cand[i];
+        const KernelMath& km = kernel_math(alpha, p.beta, p.mu);
+        p.gain = rounding_gain(km.poly, km.psi, in.nx, in.ny, in.psx, in.psy, p.nu, p.nv, in.do_w,
                                p.nshift, p.dw);
         double e_k = p.eps_kernel / safety;
         double e_r = rounding_coefficient(p.gain) * plane_rounding(kind, in.prec, p.nu, p.nv) * p.gain;
         p.err_model = std::sqrt(e_k * e_k + e_r * e_r);
         if (in.force_sigma <= 0 && p.err_model > in.eps) continue;
-        p.cost = plan_cost(in.prec, kind, p.nu, p.nv, p.nw, alpha, in.nvis, in.nx, in.ny);
         if (p.cost < best.cost) { best = p; found = true; }
         break;
       }

@@ -57,6 +57,16 @@ double psi_poly(const PolyKernel& K, double k);
 std::vector<double> psi_cheb_coeffs(const PolyKernel& K, int m);
 double psi_cheb_eval(const std::vector<double>& c, double k);
 
+// The piecewise polynomial (degree alpha + 3) of a kernel and the coefficients of its psi
+// (kPsiChebTerms): about a millisecond to form, so formed once per kernel and kept.  Meant for rows
+// of the two kernel tables only, which bounds what is kept (a few kilobytes for each of some 200
+// rows); safe from several threads.
+struct KernelMath {
+  PolyKernel poly;
+  std::vector<double> psi;
+};
+const KernelMath& kernel_math(int alpha, double beta, double mu);
+
 // Gauss-Legendre nodes / weights on [-1, 1].
 void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w);
 
@@ -139,6 +149,13 @@ struct PlanParams {
   double gain = 0;       // rounding_gain of the plan
   double err_model = 0;  // predicted eps_rms: kernel term (+) plane rounding term
 };
+
+// Setting up cuFFT's batched 2-D transform takes 75 - 110 ms (1408 x 2048 to 11264 x 11264), the
+// library's FP32 FFT about a millisecond.  A plan that serves one call takes the latter where its
+// slower transforms cost less than that (true below about 8000^2 cells and 60 planes): same grid,
+// same kernel, results equal up to FP32 rounding.
+constexpr double kCufftSetupMs = 60.0;
+bool short_setup_fft(const PlanParams& p, int prec, int64_t nx, int64_t ny);
 
 // Returns 0 on success; on failure fills err (WG_ERR_ARG class problems).
 int choose_plan(const PlanInput& in, PlanParams& out, char* err, int errlen);
