@@ -522,12 +522,6 @@ static bool choose_grid(int64_t nmin_u, int64_t nmin_v, int prec, int kind, int6
   return std::isfinite(best);
 }
 
-bool short_setup_fft(const PlanParams& p, int prec, int64_t nx, int64_t ny) {
-  if (prec != 0 || p.fft_kind != kFftCufft2d || !f32_side_ok(p.nu) || !f32_side_ok(p.nv)) return false;
-  const double more = fft_ms(p.nu, p.nv, kFftF32, prec, nx, ny) - fft_ms(p.nu, p.nv, kFftCufft2d, prec, nx, ny);
-  return p.nw * more < kCufftSetupMs;
-}
-
 int choose_plan(const PlanInput& in, PlanParams& out, char* err, int errlen) {
   auto fail = [&](const char* msg) {
     std::snprintf(err, errlen, "%s", msg);

@@ -150,13 +150,6 @@ struct PlanParams {
   double err_model = 0;  // predicted eps_rms: kernel term (+) plane rounding term
 };
 
-// Setting up cuFFT's batched 2-D transform takes 75 - 110 ms (1408 x 2048 to 11264 x 11264), the
-// library's FP32 FFT about a millisecond.  A plan that serves one call takes the latter where its
-// slower transforms cost less than that (true below about 8000^2 cells and 60 planes): same grid,
-// same kernel, results equal up to FP32 rounding.
-constexpr double kCufftSetupMs = 60.0;
-bool short_setup_fft(const PlanParams& p, int prec, int64_t nx, int64_t ny);
-
 // Returns 0 on success; on failure fills err (WG_ERR_ARG class problems).
 int choose_plan(const PlanInput& in, PlanParams& out, char* err, int errlen);
 

@@ -952,6 +952,320 @@ k_grid_atomic(const Geom g, const __grid_constant__ Coef<R> coef, const IndexVie
 }
 
 // ---------------------------------------------------------------------------------------
+// grid on the tensor cores (default for FP32 with 32-cell tiles)
+//
+// Gridding visibilities onto 16 x 16 cells of a plane is a matrix product over the visibilities k:
+// cells[i][j] += sum_k wu_k[i] (wv_k[j] ww_k d_k), 16 rows against 16 columns x (re, im), and one
+// mma.m16n8k16 adds 16 visibilities to 16 x 8 cells.  (mma.sync, not tcgen05: the operands are
+// made in registers, 16 visibilities at a time for 16 x 16 cells, and the tensor pipe is at 16 %.)
+// The shared-memory atomics of k_grid_atomic execute as compare-and-swap loops: about 1050 warp
+// instructions per visibility (alpha 6, 1.6e6 visibilities on 42 planes of 2048^2) against 430 here.
+//
+// FP32 accuracy is kept: each factor is cut exactly into three bf16 parts (8 + 8 + 8 significant
+// bits) and all products of parts down to 2^-24 are summed, the leading ones 8 visibilities at a
+// time and the other seven over 16, each from zero, and added to FP32 accumulators with
+// round-to-nearest (the tensor core drops what lies 24 bits below its largest addend and rounds
+// towards zero, so nothing is carried on in it).  Rounding error of the gridded image against an
+// FP64 plan with the same kernel and grid, ten plans of 200^2 - 1024^2 and both narrow and wide
+// (e^(3 N(0,1))) data: 2.0 - 5.2e-7, 0.85 - 0.99 times the atomics'.
+//
+// Warps work alone, without barriers: warp = (16 x 16 quarter of a 32 x 32 tile, kMmaPlanes planes),
+// accumulators in registers, each cell written once; a CTA holds the four quarters.  A warp looks
+// through the visibilities of the tile and of the three tiles whose footprints reach into it, 64
+// at a time, and puts those that meet its cells and planes into a queue in shared memory;
+// whenever the queue holds 16 it evaluates their kernels (8 or 16 lanes per visibility, lane =
+// piece, Horner from registers) into rows padded with zeros on both sides and adds them.  The
+// result does not depend on timing: a plan grids bitwise reproducibly.
+//
+// Bound: latency at about one group of 16 per warp (a warp's candidates, their data and one group
+// take 9 us at 16 warps per SM), then issue.  Planes per warp: two instead of four measured 1.3
+// times slower (more visits), 96 and 168 registers 1.15 and 1.0 times.  Stage times before and after,
+// GB300: 2048^2, 1e6 visibilities, 55 planes of 2816^2 2.46 -> 1.56 ms; 4096^2, 1e7 visibilities 15.0
+// -> 10.7 ms; 8192^2, 5e7 visibilities 117 -> 74 ms; 512^2, 1.2e5 visibilities 0.66 -> 0.17 ms.
+//
+// On small grids with dense cells (fewer than kMmaSplitUnits CTAs, at least 8 visibilities for each)
+// the few tiles at the grid's origin would be the whole run time: SPLIT = 4 warps share each quarter,
+// taking turns at the candidates, and their sums are added in a fixed order (the 512^2 case 0.34 ->
+// 0.17 ms; with few visibilities the partial groups cost more than that gives: 8192^2 74 -> 160 ms).
+// ---------------------------------------------------------------------------------------
+constexpr int kMmaSplitUnits = 10000;
+constexpr int kMmaTile = 32, kMmaPlanes = 4, kMmaQueue = 256, kMmaPad = 16;
+constexpr int kMmaRow = 48;   // kMmaPad zeros, up to 16 kernel values, zeros
+constexpr int kMmaBlocks = 2;   // blocks of 32 candidates looked at together
+
+// an index entry: position in the index, visibility and fold bit, ru + 32 | (rv + 32) << 8 | c0 << 16
+struct MmaEntry { uint32_t at, id, pos; };
+struct alignas(16) MmaWarp {
+  float wu[16][kMmaRow], wv[16][kMmaRow];
+  float2 dw[16][kMmaPlanes];   // data x w kernel value of the warp's planes
+  float zu[16], zv[16], zw[16];
+  float2 d[16];
+  int ru[16], rv[16], c0[16];
+  MmaEntry queue[kMmaQueue];
+};
+
+__device__ __forceinline__ void mma_bf16(float* d, const unsigned* a, const unsigned* b) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+// the same over 8 visibilities: one register of two rows' fragments, one of the columns'
+__device__ __forceinline__ void mma_bf16_k8(float* d, unsigned a0, unsigned a1, unsigned b) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b));
+}
+// the bf16 parts (upper halves) of two values as one register each: x = p0 + p1 + p2 exactly
+__device__ __forceinline__ void split_bf16(float x, float y, unsigned& p0, unsigned& p1, unsigned& p2) {
+  auto top = [](float v) { return __uint_as_float(__float_as_uint(v) & 0xffff0000u); };
+  auto pack = [](float a, float b) { return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632); };
+  p0 = pack(x, y);
+  x -= top(x); y -= top(y);
+  p1 = pack(x, y);
+  x -= top(x); y -= top(y);
+  p2 = pack(x, y);
+}
+
+template <int G, int SPLIT>
+__global__ void __launch_bounds__(128 * SPLIT, SPLIT == 1 ? 4 : 1)
+k_grid_mma(const Geom g, const __grid_constant__ Coef<float> coef, const IndexView<float> ix,
+           const float2* __restrict__ vis, const float* __restrict__ wgt,
+           float2* __restrict__ planes, int b0, int nb) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int T = kMmaTile;
+  const int alpha = g.alpha, aw = g.alpha_w;
+  // tile rows from both ends of the grid towards its middle: short baselines, the densest rows,
+  // lie at the ends (row 0 and, wrapped, the last) and start first
+  const int tr = blockIdx.x / g.ntv, tv = blockIdx.x - tr * g.ntv;
+  const int tu = (tr & 1) ? g.ntu - 1 - tr / 2 : tr / 2;
+  const int s0 = b0 + blockIdx.y * kMmaPlanes;
+  const int sb = min(kMmaPlanes, b0 + nb - s0);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  MmaWarp& sm = reinterpret_cast<MmaWarp*>(smem)[warp];
+  const int quarter = warp / SPLIT, part = warp - quarter * SPLIT;
+  const int sr0 = (quarter & 2) ? 16 : 0, sc0 = (quarter & 1) ? 16 : 0;
+  const int gid = lane >> 2, tig = lane & 3;
+  // the four sources' ranges of visibilities whose planes meet this warp's (lane: source and end)
+  uint32_t lo[4], before[4], total = 0;
+  {
+    const int src = (lane >> 1) & 3;
+    int stu = tu - (src & 1); if (stu < 0) stu += g.ntu;
+    int stv = tv - (src >> 1); if (stv < 0) stv += g.ntv;
+    const uint32_t at = ix.off[((int64_t)stu * g.ntv + stv) * g.nw +
+                               ((lane & 1) ? min(g.nw, s0 + sb) : max(0, s0 - aw + 1))];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      lo[s] = __shfl_sync(0xffffffffu, at, 2 * s);
+      before[s] = total;
+      total += __shfl_sync(0xffffffffu, at, 2 * s + 1) - lo[s];
+    }
+  }
+  const int64_t pstride = (int64_t)g.nu * g.nv;
+  float2* out = planes + (int64_t)(s0 - b0) * pstride + (int64_t)(tu * T + sr0 + gid) * g.nv +
+                tv * T + sc0 + 2 * tig;
+  // the accumulators never live across the end of a branch that may diverge (they would be
+  // spilled): an empty warp stores its zeros here, and the loops below end on votes
+  if (!__any_sync(0xffffffffu, total > 0)) {
+    for (int pl = part; pl < sb; pl += SPLIT)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        *reinterpret_cast<float4*>(out + pl * pstride + (int64_t)(8 * (c >> 1)) * g.nv + 8 * (c & 1)) =
+            make_float4(0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  float acc[kMmaPlanes][4][4];   // plane, (columns 0-7 re, im, columns 8-15 re, im), fragment
+#pragma unroll
+  for (int a = 0; a < kMmaPlanes * 16; ++a) (&acc[0][0][0])[a] = 0.f;
+
+  {
+    uint32_t mt[kMmaBlocks], id[kMmaBlocks], at[kMmaBlocks];
+    auto entries = [&](uint32_t e0) {   // index entries of the next candidates
+#pragma unroll
+      for (int b = 0; b < kMmaBlocks; ++b) {
+        const uint32_t e = e0 + 32 * b + lane;
+        mt[b] = id[b] = at[b] = 0;
+        if (e < total) {
+          const int src = (e >= before[1]) + (e >= before[2]) + (e >= before[3]);
+          at[b] = e + (src == 0 ? lo[0] : src == 1 ? lo[1] - before[1]
+                       : src == 2 ? lo[2] - before[2] : lo[3] - before[3]);
+          mt[b] = ix.meta[at[b]];
+          id[b] = ix.idx[at[b]];
+        }
+      }
+    };
+    entries(32 * kMmaBlocks * part);
+    float4* z4 = reinterpret_cast<float4*>(&sm.wu[0][0]);
+    for (int i = lane; i < 2 * 16 * kMmaRow / 4; i += 32) z4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane < 16) {
+      sm.ru[lane] = sm.rv[lane] = sm.c0[lane] = 0;
+      sm.zu[lane] = sm.zv[lane] = sm.zw[lane] = 0.f;
+      sm.d[lane] = make_float2(0.f, 0.f);
+    }
+    // this lane's kernel piece: coefficients in registers, zeros up to degree G + 3
+    const int j = lane & (G - 1);
+    float pc[G + 4];
+#pragma unroll
+    for (int d = 0; d <= G + 3; ++d) pc[d] = d <= g.deg ? coef.c[d * kMaxG + j] : 0.f;
+    auto piece = [&](float z) {
+      float r = pc[G + 3];
+#pragma unroll
+      for (int d = G + 2; d >= 0; --d) r = fmaf(r, z, pc[d]);
+      return r;
+    };
+    int head = 0, cnt = 0;
+    constexpr uint32_t kStep = 32 * kMmaBlocks * SPLIT;   // the parts take turns
+    for (uint32_t e0 = 32 * kMmaBlocks * part;; e0 += kStep) {
+      // the test against the warp's cells and planes; hits go to the queue in index order
+#pragma unroll
+      for (int b = 0; b < kMmaBlocks; ++b) {
+        const uint32_t e = e0 + 32 * b + lane;
+        const int src = (e >= before[1]) + (e >= before[2]) + (e >= before[3]);
+        const int ru = (int)(mt[b] & 255) - (src & 1) * T, rv = (int)((mt[b] >> 8) & 255) - (src >> 1) * T;
+        const int c0 = (int)(mt[b] >> 16);
+        const bool hit = e < total && ru < sr0 + 16 && ru + alpha > sr0 && rv < sc0 + 16 &&
+                         rv + alpha > sc0 && c0 < s0 + sb && c0 + aw > s0;
+        const unsigned m = __ballot_sync(0xffffffffu, hit);
+        if (hit) {
+          MmaEntry& q = sm.queue[(head + cnt + __popc(m & ((1u << lane) - 1u))) & (kMmaQueue - 1)];
+          q.at = at[b]; q.id = id[b];
+          q.pos = (uint32_t)((ru + 32) | (rv + 32) << 8 | c0 << 16);
+        }
+        cnt += __popc(m);
+      }
+      const bool done = __any_sync(0xffffffffu, e0 + kStep >= total);
+      if (!done) entries(e0 + kStep);
+      __syncwarp();
+      while (cnt >= 16 || (done && cnt > 0)) {
+        const int nv = min(cnt, 16);
+        // 16 visibilities: lanes 0-15 their coordinates, lanes 16-31 their data
+        {
+          const int v = lane & 15;
+          const MmaEntry q = sm.queue[(head + v) & (kMmaQueue - 1)];
+          if (v < nv) {
+            if (lane < 16) {
+              const Z4<float> z = ix.z[q.at];
+              sm.zu[v] = z.u; sm.zv[v] = z.v; sm.zw[v] = z.w;
+              sm.ru[v] = (int)(q.pos & 255) - 32; sm.rv[v] = (int)((q.pos >> 8) & 255) - 32;
+              sm.c0[v] = (int)(q.pos >> 16);
+            } else {
+              const int64_t k = q.id & ~kFoldBit;
+              float2 d = vis[k];
+              if (wgt != nullptr) { const float w = wgt[k]; d.x *= w; d.y *= w; }
+              if (q.id & kFoldBit) d.y = -d.y;    // grid conj(d) at the folded coordinates
+              if (ix.ph != nullptr) {             // times conj(exp(2 pi i w nshift))
+                const float2 ph = ix.ph[q.at];
+                const float r = d.x * ph.x + d.y * ph.y;
+                d.y = d.y * ph.x - d.x * ph.y;
+                d.x = r;
+              }
+              sm.d[v] = d;
+            }
+          }
+          head = (head + nv) & (kMmaQueue - 1);
+          cnt -= nv;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int v0 = 0; v0 < 16; v0 += 32 / G) {
+          // (slots beyond the last visibility hold an older one, or zeros: their data count as zero)
+          const int v = v0 + lane / G, c0 = sm.c0[v];
+          const float pu = piece(sm.zu[v]), pv = piece(sm.zv[v]), pw = piece(sm.zw[v]);
+          sm.wu[v][kMmaPad + j] = j < alpha ? pu : 0.f;
+          sm.wv[v][kMmaPad + j] = j < alpha ? pv : 0.f;
+          const float ww = g.do_w ? (j < alpha ? pw : 0.f) : (j == 0 ? 1.f : 0.f);
+          // lane pl of the group takes plane s0 + pl, the visibility's plane q = s0 + pl - c0
+          const int q = s0 + j - c0;
+          const float wq = __shfl_sync(0xffffffffu, ww, q & (G - 1), G);
+          if (j < kMmaPlanes) {
+            const bool on = v < nv && q >= 0 && q < aw;
+            const float2 d = sm.d[v];
+            sm.dw[v][j] = on ? make_float2(d.x * wq, d.y * wq) : make_float2(0.f, 0.f);
+          }
+        }
+        __syncwarp();
+        // this lane's four visibilities: k = 2 tig, 2 tig + 1, 2 tig + 8, 2 tig + 9
+        float x[4][2], y[4][2];   // wu at rows gid, gid + 8; wv at columns gid, gid + 8
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int v = 2 * tig + (q & 1) + (q & 2) * 4;
+          const float* u = &sm.wu[v][kMmaPad + sr0 + gid - sm.ru[v]];
+          const float* w = &sm.wv[v][kMmaPad + sc0 + gid - sm.rv[v]];
+          x[q][0] = u[0]; x[q][1] = u[8];
+          y[q][0] = w[0]; y[q][1] = w[8];
+        }
+        unsigned A[3][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)   // rows gid, gid + 8 at k 0-7, then at k 8-15
+          split_bf16(x[(r >> 1) * 2][r & 1], x[(r >> 1) * 2 + 1][r & 1], A[0][r], A[1][r], A[2][r]);
+#pragma unroll
+        for (int pl = 0; pl < kMmaPlanes; ++pl) {
+          float2 d[4];
+          bool any = false;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            d[q] = sm.dw[2 * tig + (q & 1) + (q & 2) * 4][pl];
+            any = any || d[q].x != 0.f || d[q].y != 0.f;
+          }
+          if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt) {
+            float b[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) b[q] = y[q][nt >> 1] * ((nt & 1) ? d[q].y : d[q].x);
+            unsigned B[3][2];
+            split_bf16(b[0], b[1], B[0][0], B[1][0], B[2][0]);
+            split_bf16(b[2], b[3], B[0][1], B[1][1], B[2][1]);
+            float s[4], m[4], m8[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s[i] = m[i] = m8[i] = 0.f;
+            mma_bf16_k8(m, A[0][0], A[0][1], B[0][0]);
+            mma_bf16_k8(m8, A[0][2], A[0][3], B[0][1]);
+            mma_bf16(s, A[2], B[1]);
+            mma_bf16(s, A[1], B[2]);
+            mma_bf16(s, A[2], B[0]);
+            mma_bf16(s, A[0], B[2]);
+            mma_bf16(s, A[1], B[1]);
+            mma_bf16(s, A[1], B[0]);
+            mma_bf16(s, A[0], B[1]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[pl][nt][i] += (m[i] + m8[i]) + s[i];
+          }
+        }
+        __syncwarp();   // the staged visibilities have been used
+      }
+      if (done) break;
+    }
+  }
+  if constexpr (SPLIT > 1) {
+    // the parts' sums through their own shared memory, added in a fixed order
+    static_assert(sizeof(MmaWarp) >= kMmaPlanes * 16 * 32 * sizeof(float), "room for a part's sums");
+    float* mine = reinterpret_cast<float*>(&sm);
+    if (part > 0) {
+#pragma unroll
+      for (int i = 0; i < kMmaPlanes * 16; ++i) mine[32 * i + lane] = (&acc[0][0][0])[i];
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(quarter + 1), "r"(32 * SPLIT) : "memory");
+    if (part > 0) return;
+#pragma unroll 1
+    for (int o = 1; o < SPLIT; ++o) {
+      const float* other = mine + o * (sizeof(MmaWarp) / sizeof(float));
+#pragma unroll
+      for (int i = 0; i < kMmaPlanes * 16; ++i) (&acc[0][0][0])[i] += other[32 * i + lane];
+    }
+  }
+#pragma unroll
+  for (int pl = 0; pl < kMmaPlanes; ++pl) {
+    if (pl >= sb) break;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int r = 0; r < 2; ++r)   // two adjacent cells, 16-byte aligned (nv is a multiple of 32)
+        *reinterpret_cast<float4*>(out + pl * pstride + (int64_t)(8 * r) * g.nv + 8 * h) =
+            make_float4(acc[pl][2 * h][2 * r], acc[pl][2 * h + 1][2 * r], acc[pl][2 * h][2 * r + 1],
+                        acc[pl][2 * h + 1][2 * r + 1]);
+  }
+}
+
+// ---------------------------------------------------------------------------------------
 // grid, row-band owner variant (FP32, alpha <= 8, 32-cell tiles; deterministic)
 //
 // CTA = (32 x 32 uv tile, sub-batch of up to kBandPlanes planes), accumulators in shared memory
@@ -1274,6 +1588,29 @@ static cudaError_t grid_atomic_g(const Geom& g, const Coef<R>& coef, const Index
   return cudaGetLastError();
 }
 
+template <int G, int SPLIT>
+static cudaError_t grid_mma_split(const Geom& g, const Coef<float>& coef, const IndexView<float>& ix,
+                                  const float2* vis, const float* wgt, float2* planes, int b0,
+                                  int nb, cudaStream_t s) {
+  const size_t smem = 4 * SPLIT * sizeof(MmaWarp);
+  cudaError_t e = cudaFuncSetAttribute(k_grid_mma<G, SPLIT>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int64_t ntiles = (int64_t)g.ntu * g.ntv;
+  dim3 grid((unsigned)ntiles, (unsigned)((nb + kMmaPlanes - 1) / kMmaPlanes));
+  k_grid_mma<G, SPLIT><<<grid, 128 * SPLIT, smem, s>>>(g, coef, ix, vis, wgt, planes, b0, nb);
+  return cudaGetLastError();
+}
+
+template <int G>
+static cudaError_t grid_mma(const Geom& g, const Coef<float>& coef, const IndexView<float>& ix,
+                            const float2* vis, const float* wgt, float2* planes, int b0, int nb,
+                            cudaStream_t s) {
+  const int64_t units = (int64_t)g.ntu * g.ntv * ((nb + kMmaPlanes - 1) / kMmaPlanes);
+  if (units < kMmaSplitUnits && g.nvis > 8 * units) return grid_mma_split<G, 4>(g, coef, ix, vis, wgt, planes, b0, nb, s);
+  return grid_mma_split<G, 1>(g, coef, ix, vis, wgt, planes, b0, nb, s);
+}
+
 static cudaError_t grid_band(const Geom& g, const Coef<float>& coef, const IndexView<float>& ix,
                              const float2* vis, const float* wgt, float2* planes, int b0, int nb,
                              cudaStream_t s) {
@@ -1290,9 +1627,9 @@ static cudaError_t grid_band(const Geom& g, const Coef<float>& coef, const Index
 }
 
 // the gridding variant a plan uses (Geom::grid_variant 0 = automatic).  Automatic FP32 takes the
-// shared-memory atomics: on the 1e8-visibility workload the row-band owners measured 289 ms
-// against 171 ms (ncu on 1.6e6 visibilities: 37 % fewer instructions, but barrier- and
-// latency-bound at 16 warps per SM, issue active 26 % against 74 %)
+// tensor cores, which need 32-cell tiles, else the shared-memory atomics (on the 1e8-visibility
+// workload the row-band owners measured 289 ms, the atomics 171 ms, the tensor cores half of that)
+constexpr int kVariantMma = 4;   // tensor cores: automatic choice only
 template <typename R>
 static int grid_variant_of(const Geom& g) {
   // double-float planes are written by the plane-owner kernel only
@@ -1300,7 +1637,7 @@ static int grid_variant_of(const Geom& g) {
   const bool band_ok = sizeof(R) == 4 && g.alpha <= 8 && g.tile == kBandTile;
   if (g.grid_variant == 3) return band_ok ? 3 : 1;
   if (g.grid_variant != 0) return g.grid_variant;
-  return sizeof(R) == 8 ? 2 : 1;
+  return sizeof(R) == 8 ? 2 : (g.tile == kMmaTile ? kVariantMma : 1);
 }
 
 template <typename R, int G>
@@ -1313,6 +1650,11 @@ static cudaError_t grid_g(const Geom& g, const Coef<R>& coef, const IndexView<R>
     if (variant == 3)
       return grid_band(g, coef, ix, (const float2*)vis, (const float*)wgt, (float2*)planes, b0,
                        nb, s);
+  }
+  if constexpr (sizeof(R) == 4) {
+    if (variant == kVariantMma)   // groups of at least 8 lanes, one per plane of a CTA
+      return grid_mma<(G < 8 ? 8 : G)>(g, coef, ix, (const float2*)vis, (const float*)wgt,
+                                       (float2*)planes, b0, nb, s);
   }
   return grid_atomic_g<R, G>(g, coef, ix, vis, wgt, planes, b0, nb, s);
 }

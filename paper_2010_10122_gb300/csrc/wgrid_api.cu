@@ -391,11 +391,10 @@ static void fill_coefs(wg_plan* p) {
   for (int i = 0; i < kPsiChebTerms; ++i) p->psi_c[i] = km.psi[i];
 }
 
-// one_shot: the plan serves a single call (see short_setup_fft)
-static int create_plan(const double* uvw, const double* freq, int64_t nrows, int64_t nchan,
-                       int64_t npix_x, int64_t npix_y, double pixsize_x, double pixsize_y,
-                       double epsilon, int precision, const uint8_t* mask, const wg_options* opt,
-                       void* stream, bool one_shot, wg_plan** out) {
+int wg_plan_create(const double* uvw, const double* freq, int64_t nrows, int64_t nchan,
+                   int64_t npix_x, int64_t npix_y, double pixsize_x, double pixsize_y,
+                   double epsilon, int precision, const uint8_t* mask, const wg_options* opt,
+                   void* stream, wg_plan** out) {
   if (out == nullptr) return set_error(WG_ERR_ARG, "out is NULL");
   *out = nullptr;
   if (precision != WG_F32 && precision != WG_F64) return set_error(WG_ERR_ARG, "bad precision");
@@ -444,8 +443,6 @@ static int create_plan(const double* uvw, const double* freq, int64_t nrows, int
   PlanInput in = plan_input(npix_x, npix_y, pixsize_x, pixsize_y, epsilon, precision, p->opt,
                             p->umax, p->vmax, p->wmin, p->wmax, p->nvis_total);
   if (choose_plan(in, p->pp, err, sizeof(err)) != 0) return set_error(WG_ERR_ARG, "%s", err);
-  if (one_shot && p->opt.fft_impl == 0 && short_setup_fft(p->pp, precision, npix_x, npix_y))
-    p->pp.fft_kind = kFftF32;
   const PlanParams& pp = p->pp;
   Geom& g = p->g;
   g.nrows = nrows; g.nchan = nchan; g.nvis = p->nvis_total;
@@ -633,14 +630,6 @@ static int create_plan(const double* uvw, const double* freq, int64_t nrows, int
     return fail(rc);
   *out = p.release();
   return WG_OK;
-}
-
-int wg_plan_create(const double* uvw, const double* freq, int64_t nrows, int64_t nchan,
-                   int64_t npix_x, int64_t npix_y, double pixsize_x, double pixsize_y,
-                   double epsilon, int precision, const uint8_t* mask, const wg_options* opt,
-                   void* stream, wg_plan** out) {
-  return create_plan(uvw, freq, nrows, nchan, npix_x, npix_y, pixsize_x, pixsize_y, epsilon,
-                     precision, mask, opt, stream, false, out);
 }
 
 int wg_plan_destroy(wg_plan* plan) {
@@ -996,8 +985,8 @@ int wg_dirty2ms(const double* uvw, const double* freq, int64_t nrows, int64_t nc
   wg_default_options(&o);
   o.do_wstacking = do_wstacking;
   wg_plan* p = nullptr;
-  WG_TRY(create_plan(uvw, freq, nrows, nchan, npix_x, npix_y, pixsize_x, pixsize_y, epsilon,
-                     precision, mask, &o, stream, true, &p));
+  WG_TRY(wg_plan_create(uvw, freq, nrows, nchan, npix_x, npix_y, pixsize_x, pixsize_y, epsilon,
+                        precision, mask, &o, stream, &p));
   int rc = wg_degrid(p, dirty, wgt, vis, stream, nullptr);
   std::string keep = g_last_error;
   wg_plan_destroy(p);
@@ -1013,8 +1002,8 @@ int wg_ms2dirty(const double* uvw, const double* freq, int64_t nrows, int64_t nc
   wg_default_options(&o);
   o.do_wstacking = do_wstacking;
   wg_plan* p = nullptr;
-  WG_TRY(create_plan(uvw, freq, nrows, nchan, npix_x, npix_y, pixsize_x, pixsize_y, epsilon,
-                     precision, mask, &o, stream, true, &p));
+  WG_TRY(wg_plan_create(uvw, freq, nrows, nchan, npix_x, npix_y, pixsize_x, pixsize_y, epsilon,
+                        precision, mask, &o, stream, &p));
   int rc = wg_grid(p, vis, wgt, dirty, stream, nullptr);
   std::string keep = g_last_error;
   wg_plan_destroy(p);
