@@ -983,12 +983,12 @@ k_grid_atomic(const Geom g, const __grid_constant__ Coef<R> coef, const IndexVie
 // GB300: 2048^2, 1e6 visibilities, 55 planes of 2816^2 2.46 -> 1.56 ms; 4096^2, 1e7 visibilities 15.0
 // -> 10.7 ms; 8192^2, 5e7 visibilities 117 -> 74 ms; 512^2, 1.2e5 visibilities 0.66 -> 0.17 ms.
 //
-// On small grids with dense cells (fewer than kMmaSplitUnits CTAs, at least 8 visibilities for each)
-// the few tiles at the grid's origin would be the whole run time: SPLIT = 4 warps share each quarter,
-// taking turns at the candidates, and their sums are added in a fixed order (the 512^2 case 0.34 ->
-// 0.17 ms; with few visibilities the partial groups cost more than that gives: 8192^2 74 -> 160 ms).
+// On small grids the few dense tiles at the grid's origin would be the whole run time: where the
+// densest quarter holds more than twice what a resident warp gets on average (and 64 more, four
+// groups, below which a split costs more than it gives), SPLIT = 4 warps share each quarter, taking
+// turns at the candidates, and their sums are added in a fixed order (the 512^2 case 0.34 -> 0.17 ms;
+// where it is not needed the partial groups cost more than that gives: 8192^2 74 -> 160 ms).
 // ---------------------------------------------------------------------------------------
-constexpr int kMmaSplitUnits = 10000;
 constexpr int kMmaTile = 32, kMmaPlanes = 4, kMmaQueue = 256, kMmaPad = 16;
 constexpr int kMmaRow = 48;   // kMmaPad zeros, up to 16 kernel values, zeros
 constexpr int kMmaBlocks = 2;   // blocks of 32 candidates looked at together
@@ -1606,8 +1606,13 @@ template <int G>
 static cudaError_t grid_mma(const Geom& g, const Coef<float>& coef, const IndexView<float>& ix,
                             const float2* vis, const float* wgt, float2* planes, int b0, int nb,
                             cudaStream_t s) {
-  const int64_t units = (int64_t)g.ntu * g.ntv * ((nb + kMmaPlanes - 1) / kMmaPlanes);
-  if (units < kMmaSplitUnits && g.nvis > 8 * units) return grid_mma_split<G, 4>(g, coef, ix, vis, wgt, planes, b0, nb, s);
+  // hits of the densest quarter (about half of its tile's visibilities, those whose planes meet
+  // the warp's) against the mean over the warps the GPU holds at once (16 on each SM; a visibility
+  // meets 2.1 quarters and (alpha + 3) / 4 plane groups)
+  const double window = std::min(1.0, (double)(g.alpha_w + kMmaPlanes - 1) / g.nw);
+  const double densest = 0.5 * (double)g.max_tile * window;
+  const double mean = 2.1 * (double)g.nvis * (g.alpha_w + kMmaPlanes - 1) / kMmaPlanes / (152.0 * 16.0);
+  if (densest > 2.0 * mean + 64.0) return grid_mma_split<G, 4>(g, coef, ix, vis, wgt, planes, b0, nb, s);
   return grid_mma_split<G, 1>(g, coef, ix, vis, wgt, planes, b0, nb, s);
 }
 

@@ -248,6 +248,20 @@ __device__ __forceinline__ void write_record(const Geom& g, const VisPos& p, uin
   }
 }
 
+// the most visibilities that one tile holds, over all its plane buckets (off: the scanned offsets)
+__global__ void k_max_tile(const Geom g, const uint32_t* __restrict__ off, uint32_t* __restrict__ most) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  uint32_t n = 0;
+  if (t < g.ntu * g.ntv) n = off[(int64_t)(t + 1) * g.nw] - off[(int64_t)t * g.nw];
+  n = __reduce_max_sync(0xffffffffu, n);
+  if ((threadIdx.x & 31) == 0 && n > 0) atomicMax(most, n);
+}
+
+cudaError_t launch_max_tile(const Geom& g, const uint32_t* off, uint32_t* most, cudaStream_t s) {
+  k_max_tile<<<(unsigned)(((int64_t)g.ntu * g.ntv + 255) / 256), 256, 0, s>>>(g, off, most);
+  return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------------------------------
 // Scatter: each visibility writes its index entry (k | fold bit) at off[key] + rank, and, for
 // a full index, its record (meta, z, ph may be null for a compact index).

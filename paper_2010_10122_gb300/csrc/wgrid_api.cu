@@ -289,7 +289,7 @@ static Workspace workspace_layout(const wg_plan* p, int64_t batch, size_t fft_ws
 }
 
 static int build_index(wg_plan* p, const double* uvw, const uint8_t* mask, cudaStream_t s) {
-  const Geom& g = p->g;
+  Geom& g = p->g;
   const int64_t nkeys = (int64_t)g.ntu * g.ntv * g.nw;
   if (nkeys + 1 > (int64_t)std::numeric_limits<uint32_t>::max())
     return set_error(WG_ERR_ARG, "too many (tile, plane) buckets: %lld", (long long)nkeys);
@@ -297,7 +297,7 @@ static int build_index(wg_plan* p, const double* uvw, const uint8_t* mask, cudaS
     return set_error(WG_ERR_ARG, "at most 2^31 - 1 visibilities per plan");
   WG_TRY(dev_alloc(&p->off, (size_t)nkeys + 1));
   uint32_t *key = nullptr, *rank = nullptr, *scratch = nullptr;
-  int* err = nullptr;
+  int* err = nullptr;   // out-of-range flag, then the most visibilities in a tile
   int rc = WG_OK;
   size_t nscr = scan_scratch_elems(nkeys + 1);
   do {
@@ -306,20 +306,22 @@ static int build_index(wg_plan* p, const double* uvw, const uint8_t* mask, cudaS
     if ((rc = pool_alloc((void**)&rank, sizeof(uint32_t) * std::max<int64_t>(1, p->nvis_total),
                          p->device, s)) != WG_OK) break;
     if ((rc = pool_alloc((void**)&scratch, sizeof(uint32_t) * nscr, p->device, s)) != WG_OK) break;
-    if ((rc = pool_alloc((void**)&err, sizeof(int), p->device, s)) != WG_OK) break;
+    if ((rc = pool_alloc((void**)&err, 2 * sizeof(int), p->device, s)) != WG_OK) break;
     cudaError_t e = cudaMemsetAsync(p->off, 0, sizeof(uint32_t) * (nkeys + 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 2 * sizeof(int), s);
     if (e == cudaSuccess) e = launch_bin_count(g, uvw, p->chan4, mask, p->off, key, rank, err, s);
     if (e == cudaSuccess) e = launch_scan(p->off, nkeys + 1, scratch, s);
+    if (e == cudaSuccess) e = launch_max_tile(g, p->off, (uint32_t*)err + 1, s);
     uint32_t nvalid = 0;
-    int herr = 0;
+    int herr[2] = {0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(&nvalid, p->off + nkeys, sizeof(uint32_t),
                                               cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) { rc = set_error(WG_ERR_CUDA, "index build: %s", cudaGetErrorString(e)); break; }
-    if (herr != 0) { rc = set_error(WG_ERR_INTERNAL, "w-plane index out of range in index build"); break; }
+    if (herr[0] != 0) { rc = set_error(WG_ERR_INTERNAL, "w-plane index out of range in index build"); break; }
     p->nvis = nvalid;
+    g.max_tile = (uint32_t)herr[1];
     size_t zsz = z_bytes(p->prec);
     size_t phsz = cplx_bytes(p->prec);
     size_t n = std::max<int64_t>(1, p->nvis);

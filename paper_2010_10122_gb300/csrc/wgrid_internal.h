@@ -38,6 +38,7 @@ struct Geom {
   double psx, psy;
   double w0, dw, nshift;
   double w0_dw;         // w0 / dw
+  int64_t max_tile;     // most visibilities in one tile
   int grid_variant;     // 0 automatic, 1 shared atomics, 2 plane-owner warps, 3 row-band owners
   int df64_planes;      // FP64 plans with the double-float FFT: the uv planes hold double-float
                         // pairs (float4 per cell) and (de)gridding runs in pair arithmetic
@@ -100,6 +101,7 @@ cudaError_t launch_bin_count(const Geom& g, const double* uvw, const double* cha
                              uint32_t* rank, int* err, cudaStream_t s);
 cudaError_t launch_scan(uint32_t* data, int64_t n, uint32_t* scratch, cudaStream_t s);
 size_t scan_scratch_elems(int64_t n);
+cudaError_t launch_max_tile(const Geom& g, const uint32_t* off, uint32_t* most, cudaStream_t s);
 template <typename R>
 cudaError_t launch_bin_scatter(const Geom& g, const double* uvw, const double* chan4,
                                const uint32_t* key, const uint32_t* rank, const uint32_t* off,
