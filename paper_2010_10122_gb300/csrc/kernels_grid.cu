@@ -19,6 +19,7 @@
 //  * FP64 plans with the double-float FFT keep the planes as double-float pairs and run the
 //    degridding and plane-owner gridding in pair arithmetic on the FP32 pipes (df64.cuh).
 #include "df64.cuh"
+#include "fft_engine.cuh"
 #include "wgrid_internal.h"
 
 namespace wg {
@@ -623,174 +624,217 @@ cudaError_t launch_grid_vis_dd(const IndexView<double>& ix, const double2* vis, 
 }
 
 // ---------------------------------------------------------------------------------------
-// grid of double-float planes (FP64 plans with the double-float FFT): the plane-owner scheme
-// of k_grid_owner with the staged 2-D weights, the plane-weighted data and the accumulators as
-// double-float pairs, updated in pair arithmetic on the FP32 pipes (dd_fma), and the planes
-// written as pairs (float4 per cell) for the double-float FFT.
-// ---------------------------------------------------------------------------------------
-template <int G>
-struct GridStageDD {
-  // kernel values in u and v as pairs (the 2-D weight of a cell, one pair product, is formed
-  // where it is used: 7 FP32 instructions, cheaper than staging G^2 weights), and the data
-  // times the w kernel value of plane q (re hi, re lo, im hi, im lo)
-  static constexpr int kChunk = 48;
-  float2 wu[kChunk][G];
-  float2 wv[kChunk][G];
-  float4 dq[kChunk][G];
-  int ru[kChunk], rv[kChunk], c0[kChunk];
+// grid of double-float planes (FP64 plans with the double-float FFT): accumulators in registers
+//
+// CTA = (rows x cols cells of a uv tile, 8 planes).  A half-warp owns 4 x 4 cells and a lane one
+// cell in all 8 planes, its sums in registers as double-float pairs with the real and the imaginary
+// part packed: a cell's update in pair arithmetic is 15 packed FP32 instructions, with nothing
+// read from or written to shared memory but the staged visibility (the plane-owner scheme with
+// pairs in shared memory spent half its issue slots on those).  Visibilities of the tile, and of
+// the tiles whose footprints reach into the cells, form one list, staged in chunks: kernel values
+// in u and v, and data times w kernel value by plane (zero in the planes a visibility does not
+// meet).  Each half-warp walks its own bit mask of the chunk's visibilities that meet its 4 x 4
+// cells (alpha = 15: 69 % of its lanes are inside the footprint, against 57 % for 4 x 8 cells of a
+// whole warp), updating planes two at a time where a visibility of either half meets them.
+// Cells are updated in index order: deterministic.
+//
+// Bound by the FP32 pipe (53 % active) and, of the rest, by warps waiting for the one with the most
+// visibilities of a chunk.  16 planes per lane (118 registers, 2 CTAs per SM) measured 13.3 ms where
+// 8 planes take 11.4, and whole-warp 4 x 8 cells 11.4 where half-warps take 10.6 (3456^2 grid, 1e6
+// visibilities, alpha = 15; the plane-owner kernel 19.6).
+//
+// Shapes, by template (W warps x SPLIT):
+//  * <8, 1>: 16 x 16 cells, every warp walks the whole chunk.
+//  * <2, 4>: 8 x 8 cells, four sets of two warps, each taking every fourth visibility, their sums
+//    added in order at the end: for plans whose densest tile would be the run time.
+constexpr int kCellsPlanes = 8;
+template <int W>
+struct CellsTile {   // cells and visibilities per set of a CTA
+  static constexpr int rows = W == 8 ? 16 : 8, cols = W >= 4 ? 16 : 8;
+  static constexpr int vis = W == 8 ? 64 : 32;
+};
+template <int W, int SPLIT>
+struct CellsStage {
+  static constexpr int kChunk = CellsTile<W>::vis * SPLIT;
+  // row kChunk: no visibility
+  float2 wu[kChunk + 1][kMaxG], wv[kChunk + 1][kMaxG];   // kernel values as pairs
+  float4 dq[kChunk + 1][kCellsPlanes + 1];   // data x w kernel value by plane: re hi, im hi, re lo, im lo
+  int head[kChunk + 1];   // footprint origin (row + 64, column + 64 << 8), plane pairs met << 16; or 0
+  int cum[4], first[4];   // visibilities before each source tile; index position minus that
 };
 
-template <int G, int MC>
-__device__ __forceinline__ void owner_add_dd(const GridStageDD<G>* __restrict__ stg, int v,
-                                             const OwnerFootprint& fp, int lane, int T, int pitch,
-                                             int p1, int phi, int qoff, float4* __restrict__ acc,
-                                             int plane_elems) {
-  const float rw = 1.0f / (float)fp.w;
-  const int dummy = (lane >> 1) * pitch + T + (lane & 1);
-  dd wt[MC];
-  int off[MC];
-#pragma unroll
-  for (int m = 0; m < MC; ++m) {
-    const int c = lane + 32 * m;
-    // c = ii * w + jj; exact in float (see owner_add)
-    const int ii = (int)(((float)c + 0.5f) * rw), jj = c - ii * fp.w;
-    const bool ok = c < fp.cells;
-    const int i = fp.i0 + (ok ? ii : 0), j = fp.j0 + (ok ? jj : 0);
-    const float2 a = stg->wu[v][i], b = stg->wv[v][j];
-    wt[m] = ok ? dd_mul(dd_make(a.x, a.y), dd_make(b.x, b.y)) : dd_make(0.f, 0.f);
-    off[m] = ok ? (fp.ru + i) * pitch + fp.rv + j : dummy;
-  }
-  // all loads of a plane first, then the arithmetic, then all stores: the cells of one lane are
-  // distinct (its idle slots share a padding cell, updated with weight 0), but the compiler
-  // cannot see that, and interleaved load / store would serialise the MC update chains
-  for (int pl = p1; pl < phi; pl += kOwnerWarps) {
-    const float4 q = stg->dq[v][pl + qoff];
-    float4* base = acc + pl * plane_elems;
-    float4 a[MC];
-#pragma unroll
-    for (int m = 0; m < MC; ++m) a[m] = base[off[m]];
-#pragma unroll
-    for (int m = 0; m < MC; ++m) {
-      const dd re = dd_fma(dd_make(q.x, q.y), wt[m], dd_make(a[m].x, a[m].y));
-      const dd im = dd_fma(dd_make(q.z, q.w), wt[m], dd_make(a[m].z, a[m].w));
-      a[m] = make_float4(re.h, re.l, im.h, im.l);
-    }
-#pragma unroll
-    for (int m = 0; m < MC; ++m) base[off[m]] = a[m];
-  }
-}
-
-// vis: the per-position data of k_grid_vis_dd (float4 pairs, 16 bytes like a double2), which
-// already carry the weights, the fold and the w-reference phase
-template <int G>
-__global__ void __launch_bounds__(kOwnerThreads)
-k_grid_owner_dd(const Geom g, const __grid_constant__ Coef<double> coef, const IndexView<double> ix,
-                const double2* __restrict__ vis, double2* __restrict__ planes, int b0, int nb,
-                int bs, int pitch) {
+template <int W, int SPLIT>
+__global__ void __launch_bounds__(32 * W * SPLIT, 32 / (W * SPLIT))
+k_grid_cells_dd(const Geom g, const __grid_constant__ Coef<double> coef, const IndexView<double> ix,
+                const float4* __restrict__ vis, float4* __restrict__ planes, int b0, int nb) {
   extern __shared__ __align__(16) unsigned char smem[];
   double* sc = reinterpret_cast<double*>(smem);
-  using Stage = GridStageDD<G>;
-  constexpr int kChunk = Stage::kChunk;
-  Stage* stg = reinterpret_cast<Stage*>(smem + (kMaxDeg + 1) * kMaxG * sizeof(double));
-  float4* acc = reinterpret_cast<float4*>(reinterpret_cast<unsigned char*>(stg) + sizeof(Stage));
-  const int T = g.tile, alpha = g.alpha, aw = g.alpha_w;
-  const int t = blockIdx.x;
-  const int tu = t / g.ntv, tv = t - tu * g.ntv;
-  const int s0 = b0 + blockIdx.y * bs;
-  const int sb = min(bs, b0 + nb - s0);
-  const int plane_elems = T * pitch;
-  for (int i = threadIdx.x; i < (g.deg + 1) * kMaxG; i += blockDim.x) sc[i] = coef.c[i];
-  for (int e = threadIdx.x; e < sb * plane_elems; e += blockDim.x) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j1 = threadIdx.x & (G - 1), grp = threadIdx.x / G, ngrp = blockDim.x / G;
-  const unsigned gmask = group_mask<G>();
-  const dd zero = dd_make(0.f, 0.f);
-  __syncthreads();   // coefficients staged
+  using Stage = CellsStage<W, SPLIT>;
+  Stage& sm = *reinterpret_cast<Stage*>(smem + (kMaxDeg + 1) * kMaxG * sizeof(double));
+  constexpr int TR = CellsTile<W>::rows, TC = CellsTile<W>::cols, G = 16, PG = kCellsPlanes, N = 32 * W;
+  const int alpha = g.alpha, aw = g.alpha_w;
+  const int nqv = g.nv / TC, nqu = g.nu / TR, peru = g.tile / TR, perv = g.tile / TC;
+  const int tr = blockIdx.x / nqv, qv = blockIdx.x - tr * nqv;
+  // rows from both ends of the grid towards its middle: short baselines, the densest rows, lie at
+  // the ends (row 0 and, wrapped, the last) and start first
+  const int qu = (tr & 1) ? nqu - 1 - tr / 2 : tr / 2;
+  const int tu = qu / peru, tv = qv / perv, su = (qu - tu * peru) * TR, sv = (qv - tv * perv) * TC;
+  const int s0 = b0 + blockIdx.y * PG;
+  const int sb = min(PG, b0 + nb - s0);
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % W;
+  const int set = SPLIT > 1 ? threadIdx.x / N : 0;   // takes every SPLIT-th visibility from here
+  const int row0 = warp / (TC / 8) * 4, col0 = warp % (TC / 8) * 8;
+  const int row = row0 + ((lane >> 2) & 3), col = col0 + ((lane >> 4) << 2) + (lane & 3);
+  if (ix.wts == nullptr)
+    for (int i = threadIdx.x; i < (g.deg + 1) * kMaxG; i += blockDim.x) sc[i] = coef.c[i];
+  if (threadIdx.x < 32) {
+    // the square's tile and, where the square lies on its edge, the three whose footprints reach in
+    const int ou = lane & 1, ov = (lane >> 1) & 1;
+    uint32_t lo = 0, n = 0;
+    if (lane < 4 && !(ou && su >= alpha) && !(ov && sv >= alpha)) {
+      int stu = tu - ou; if (stu < 0) stu += g.ntu;
+      int stv = tv - ov; if (stv < 0) stv += g.ntv;
+      const uint32_t* offs = ix.off + ((int64_t)stu * g.ntv + stv) * g.nw;
+      lo = offs[max(0, s0 - aw + 1)];
+      n = offs[min(g.nw, s0 + sb)] - lo;
+    }
+    uint32_t c = n;
+    for (int o = 1; o < 4; o <<= 1) {
+      const uint32_t up = __shfl_up_sync(0xffffffffu, c, o);
+      if (lane >= o) c += up;
+    }
+    if (lane < 4) { sm.cum[lane] = (int)c; sm.first[lane] = (int)(lo - (c - n)); }
+  }
+  if (threadIdx.x < kCellsPlanes) sm.dq[Stage::kChunk][threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (threadIdx.x == 0) sm.head[Stage::kChunk] = 0;
+  f2 ah[PG], al[PG];   // this lane's cell: (re, im) high parts, low parts
+#pragma unroll
+  for (int p = 0; p < PG; ++p) ah[p] = al[p] = f2_make(0.f, 0.f);
+  __syncthreads();
+  const int total = sm.cum[3];
 
-  for (int src = 0; src < 4; ++src) {
-    const int ou = (src & 1) ? -1 : 0, ov = (src & 2) ? -1 : 0;
-    int stu = tu + ou; if (stu < 0) stu += g.ntu;
-    int stv = tv + ov; if (stv < 0) stv += g.ntv;
-    const uint32_t* offs = ix.off + ((int64_t)stu * g.ntv + stv) * g.nw;
-    const uint32_t lo = offs[max(0, s0 - aw + 1)], hi = offs[min(g.nw, s0 + sb)];
-    for (uint32_t cs = lo; cs < hi; cs += kChunk) {
-      const int nch = (int)min((uint32_t)kChunk, hi - cs);
-      __syncthreads();  // previous chunk consumed (and accumulators zeroed)
-      // ---- phase 1: kernel values and plane-weighted data of the chunk, as pairs ----
-      for (int v = grp; v < nch; v += ngrp) {
-        const uint32_t vi = cs + v;
+  for (int cs = 0; cs < total; cs += Stage::kChunk) {
+    if (cs) __syncthreads();   // previous chunk consumed
+    {
+      const int j1 = threadIdx.x & (G - 1);
+      const unsigned gmask = group_mask<G>();
+      const int nch = min(Stage::kChunk, total - cs);
+      for (int v = threadIdx.x / G; v < nch; v += N * SPLIT / G) {
+        const int k = cs + v;
+        const int src = (k >= sm.cum[0]) + (k >= sm.cum[1]) + (k >= sm.cum[2]);
+        const uint32_t vi = (uint32_t)sm.first[src] + (uint32_t)k;
         const uint32_t mt = ix.meta[vi];
-        // with a kernel-value table, the visibility's table entries and data are loaded
-        // together with its index entry (before the tile test), so their latencies overlap
         const float2* tw = reinterpret_cast<const float2*>(ix.wts);
-        float2 tu = make_float2(0.f, 0.f), tv = tu, tww = tu;
-        if (tw != nullptr) {
+        float2 pu = make_float2(0.f, 0.f), pv = pu, pw = pu;
+        if (tw != nullptr) {   // the table holds zeros beyond alpha
           const int64_t b = (int64_t)vi * (3 * kMaxG) + j1;
-          tu = tw[b]; tv = tw[b + kMaxG]; tww = tw[b + 2 * kMaxG];
+          pu = tw[b]; pv = tw[b + kMaxG]; pw = tw[b + 2 * kMaxG];
         }
-        // the visibility's weighted, folded and phase-rotated data, prepared once per call by
-        // k_grid_vis_dd as pairs in index order (`vis` holds them, 16 bytes per position)
-        const float4 q = reinterpret_cast<const float4*>(vis)[vi];
-        const int ru = (int)(mt & 255) + ou * T, rv = (int)((mt >> 8) & 255) + ov * T;
-        const bool hit = (ru + alpha > 0) && (rv + alpha > 0);
+        const float4 d = vis[vi];
+        const int ru = (int)(mt & 255) - (src & 1) * g.tile - su;
+        const int rv = (int)((mt >> 8) & 255) - (src >> 1) * g.tile - sv;
+        const bool hit = ru < TR && ru + alpha > 0 && rv < TC && rv + alpha > 0;
+        const int plo = (int)(mt >> 16) - s0;   // first plane of the visibility, in the CTA's
         if (j1 == 0) {
-          stg->ru[v] = ru; stg->rv[v] = rv;
-          stg->c0[v] = hit ? (int)(mt >> 16) : -(1 << 20);
+          int m = 0;
+#pragma unroll
+          for (int q = 0; q < PG / 2; ++q)
+            if (2 * q + 2 > plo && 2 * q < plo + aw) m |= 1 << q;
+          sm.head[v] = hit ? (ru + 64) | (rv + 64) << 8 | m << 16 : 0;
         }
         if (!hit) continue;   // uniform within the group
-        const bool lj = j1 < alpha;
-        dd pu = zero, pv = zero, pw = zero;
-        if (lj) {
-          if (tw != nullptr) {   // the table holds zeros beyond alpha as well
-            pu = dd_make(tu.x, tu.y); pv = dd_make(tv.x, tv.y); pw = dd_make(tww.x, tww.y);
-          } else {
-            const Z4<double> zz = ix.z[vi];
-            pu = kernel_value_dd(ix, sc, g.deg, vi, 0, j1, zz.u);
-            pv = kernel_value_dd(ix, sc, g.deg, vi, 1, j1, zz.v);
-            pw = kernel_value_dd(ix, sc, g.deg, vi, 2, j1, zz.w);
-          }
+        if (tw == nullptr && j1 < alpha) {
+          const Z4<double> zz = ix.z[vi];
+          const dd a = split_double(horner(sc, g.deg, j1, zz.u)), b = split_double(horner(sc, g.deg, j1, zz.v));
+          const dd c = split_double(horner(sc, g.deg, j1, zz.w));
+          pu = make_float2(a.h, a.l); pv = make_float2(b.h, b.l); pw = make_float2(c.h, c.l);
         }
-        stg->wu[v][j1] = make_float2(pu.h, pu.l);
-        stg->wv[v][j1] = make_float2(pv.h, pv.l);
-        const dd wwj = g.do_w ? pw : (j1 == 0 ? dd_make(1.f, 0.f) : zero);
-        const dd dr = dd_make(q.x, q.y), di = dd_make(q.z, q.w);
-        const dd qr = dd_mul(dr, wwj), qi = dd_mul(di, wwj);
-        stg->dq[v][j1] = make_float4(qr.h, qr.l, qi.h, qi.l);
+        sm.wu[v][j1] = pu;
+        sm.wv[v][j1] = pv;
+        if (!g.do_w) pw = j1 == 0 ? make_float2(1.f, 0.f) : make_float2(0.f, 0.f);
+        // lane p of the group takes plane s0 + p, the visibility's plane q = p - plo
+        const int q = j1 - plo;
+        const dd w = dd_make(__shfl_sync(gmask, pw.x, q & (G - 1), G), __shfl_sync(gmask, pw.y, q & (G - 1), G));
+        if (j1 < PG) {
+          const bool on = q >= 0 && q < aw;
+          const dd qr = dd_mul(dd_make(d.x, d.y), w), qi = dd_mul(dd_make(d.z, d.w), w);
+          sm.dq[v][j1] = on ? make_float4(qr.h, qi.h, qr.l, qi.l) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
       }
-      __syncthreads();
-      // ---- phase 2: each warp adds the chunk into its own planes ----
-      for (int v = 0; v < nch; ++v) {
-        const int c0 = stg->c0[v];
-        if (c0 < -1000) continue;
-        const int plo = max(0, c0 - s0), phi = min(sb, c0 - s0 + aw);
-        const int p1 = plo + ((warp - plo) & (kOwnerWarps - 1));
-        if (p1 >= phi) continue;
-        const int ru = stg->ru[v], rv = stg->rv[v];
-        const int i0 = max(0, -ru), i1 = min(alpha, T - ru);
-        const int j0 = max(0, -rv), j1c = min(alpha, T - rv);
-        const int w = j1c - j0, cells = (i1 - i0) * w;
-        const OwnerFootprint fp{i0, j0, w, cells, ru, rv};
-        switch ((cells + 31) >> 5) {
-          case 1: owner_add_dd<G, 1>(stg, v, fp, lane, T, pitch, p1, phi, s0 - c0, acc, plane_elems); break;
-          case 2: owner_add_dd<G, 2>(stg, v, fp, lane, T, pitch, p1, phi, s0 - c0, acc, plane_elems); break;
-          case 3: owner_add_dd<G, (G > 8 ? 3 : 1)>(stg, v, fp, lane, T, pitch, p1, phi, s0 - c0, acc, plane_elems); break;
-          case 4: owner_add_dd<G, (G > 8 ? 4 : 1)>(stg, v, fp, lane, T, pitch, p1, phi, s0 - c0, acc, plane_elems); break;
-          case 5: owner_add_dd<G, (G > 8 ? 5 : 1)>(stg, v, fp, lane, T, pitch, p1, phi, s0 - c0, acc, plane_elems); break;
-          case 6: owner_add_dd<G, (G > 8 ? 6 : 1)>(stg, v, fp, lane, T, pitch, p1, phi, s0 - c0, acc, plane_elems); break;
-          case 7: owner_add_dd<G, (G > 8 ? 7 : 1)>(stg, v, fp, lane, T, pitch, p1, phi, s0 - c0, acc, plane_elems); break;
-          default: owner_add_dd<G, (G > 8 ? 8 : 1)>(stg, v, fp, lane, T, pitch, p1, phi, s0 - c0, acc, plane_elems); break;
+    }
+    __syncthreads();
+    // the visibilities whose footprints meet each half-warp's cells, as bit masks
+    uint64_t mA = 0, mB = 0;
+#pragma unroll
+    for (int r = 0; r < CellsTile<W>::vis / 32; ++r) {
+      const int v = SPLIT * (32 * r + lane) + set;
+      const int h = cs + v < total ? sm.head[v] : 0;
+      const int ru = (h & 255) - 64, rv = ((h >> 8) & 255) - 64;
+      const bool rows = ru < row0 + 4 && ru + alpha > row0;
+      const bool a = rows && rv < col0 + 4 && rv + alpha > col0;
+      const bool b = rows && rv < col0 + 8 && rv + alpha > col0 + 4;
+      mA |= (uint64_t)__ballot_sync(0xffffffffu, a) << (32 * r);
+      mB |= (uint64_t)__ballot_sync(0xffffffffu, b) << (32 * r);
+    }
+    const int n = max(__popcll(mA), __popcll(mB));
+    uint64_t m = lane < 16 ? mA : mB;
+    for (int k = 0; k < n; ++k) {
+      const int v = m ? SPLIT * (__ffsll((long long)m) - 1) + set : Stage::kChunk;
+      m &= m - 1;
+      const int h = sm.head[v];
+      const int i = row + 64 - (h & 255), j = col + 64 - ((h >> 8) & 255);
+      const bool in = (unsigned)i < (unsigned)alpha && (unsigned)j < (unsigned)alpha;
+      const float2 a = sm.wu[v][in ? i : 0], b = sm.wv[v][in ? j : 0];
+      const dd w = dd_mul(dd_make(a.x, a.y), dd_make(b.x, b.y));
+      const float wh = in ? w.h : 0.f, wl = in ? w.l : 0.f;
+      const f2 wh2 = f2_make(wh, wh), nwh = f2_make(-wh, -wh), nwl = f2_make(-wl, -wl);
+      const unsigned met = __reduce_or_sync(0xffffffffu, (unsigned)h >> 16);
+#pragma unroll
+      for (int q = 0; q < PG / 2; ++q) {
+        if (!(met & (1u << q))) continue;
+#pragma unroll
+        for (int p = 2 * q; p < 2 * q + 2; ++p) {
+          const ulonglong2 dv = *reinterpret_cast<const ulonglong2*>(&sm.dq[v][p]);
+          const f2 dh{dv.x}, dl{dv.y};
+          // ah + al += d w: pr the rounded product of the high parts, e minus all below it
+          const f2 pr = s_mul(dh, wh2);
+          f2 e = s_fma(dh, nwh, pr);
+          e = s_fma(dh, nwl, e);
+          e = s_fma(dl, nwh, e);
+          const d2 s = d2_two_sum(ah[p], pr);
+          const d2 r = d2_fast_two_sum(s.h, s_add(s.l, s_sub(al[p], e)));
+          ah[p] = r.h;
+          al[p] = r.l;
         }
       }
     }
   }
-  __syncthreads();
+  if constexpr (SPLIT > 1) {   // the sets' sums, in order
+    __syncthreads();
+    static_assert(sizeof(Stage) >= (SPLIT - 1) * PG * N * sizeof(ulonglong2), "partial sums fit the stage");
+    ulonglong2* part = reinterpret_cast<ulonglong2*>(&sm);
+    const int c = threadIdx.x % N;
+    if (set)
+#pragma unroll
+      for (int p = 0; p < PG; ++p) part[((set - 1) * PG + p) * N + c] = make_ulonglong2(ah[p].v, al[p].v);
+    __syncthreads();
+    if (set) return;
+    for (int o = 0; o < SPLIT - 1; ++o)
+#pragma unroll
+      for (int p = 0; p < PG; ++p) {
+        const ulonglong2 x = part[(o * PG + p) * N + c];
+        const d2 r = s_add(d2{ah[p], al[p]}, d2{f2{x.x}, f2{x.y}});
+        ah[p] = r.h;
+        al[p] = r.l;
+      }
+  }
   const int64_t pstride = (int64_t)g.nu * g.nv;
-  float4* out = reinterpret_cast<float4*>(planes);
-  for (int e = threadIdx.x; e < sb * T * T; e += blockDim.x) {
-    const int pl = e / (T * T), rem = e - pl * T * T;
-    const int r = rem / T, c = rem - r * T;
-    out[(int64_t)(s0 - b0 + pl) * pstride + (int64_t)(tu * T + r) * g.nv + tv * T + c] =
-        acc[pl * plane_elems + r * pitch + c];
+  float4* out = planes + (int64_t)(s0 - b0) * pstride + (int64_t)(qu * TR + row) * g.nv + qv * TC + col;
+#pragma unroll
+  for (int p = 0; p < PG; ++p) {
+    if (p >= sb) break;
+    const float2 h = f2_split(ah[p]), l = f2_split(al[p]);
+    out[p * pstride] = make_float4(h.x, l.x, h.y, l.y);
   }
 }
 
@@ -1533,6 +1577,34 @@ static cudaError_t degrid_g(const Geom& g, const Coef<R>& coef, const IndexView<
   return cudaGetLastError();
 }
 
+template <int W, int SPLIT>
+static cudaError_t grid_cells_split(const Geom& g, const Coef<double>& coef, const IndexView<double>& ix,
+                                    const float4* vis, float4* planes, int b0, int nb, cudaStream_t s) {
+  const size_t smem = coef_bytes<double>() + sizeof(CellsStage<W, SPLIT>);
+  cudaError_t e = cudaFuncSetAttribute(k_grid_cells_dd<W, SPLIT>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  dim3 grid((unsigned)((int64_t)(g.nu / CellsTile<W>::rows) * (g.nv / CellsTile<W>::cols)),
+            (unsigned)((nb + kCellsPlanes - 1) / kCellsPlanes));
+  k_grid_cells_dd<W, SPLIT><<<grid, 32 * W * SPLIT, smem, s>>>(g, coef, ix, vis, planes, b0, nb);
+  return cudaGetLastError();
+}
+
+static cudaError_t grid_cells_dd(const Geom& g, const Coef<double>& coef, const IndexView<double>& ix,
+                                 const float4* vis, float4* planes, int b0, int nb, cudaStream_t s) {
+  // visibilities that a warp of the densest tile walks, against the mean over the warps the GPU
+  // holds at once (32 on each SM; a visibility meets (alpha + 3)(alpha + 7) / 32 warps' 4 x 8 cells
+  // and (alpha_w + 7) / 8 plane groups).  Measured <8, 1> against <2, 4>: 0.57 / 0.29 ms at 379
+  // against a mean of 163 (27 000 visibilities, alpha 14), 80 / 29 ms at 150 000 against 2 400;
+  // 10.6 / 16.1 ms at 169 against 7 000, 0.07 / 0.12 ms at 26 against 43 (1e4 visibilities)
+  const double reach = (g.alpha + 3.0) * (g.alpha + 7.0), groups = g.alpha_w + kCellsPlanes - 1.0;
+  const double densest = g.max_tile * std::min(1.0, groups / g.nw) *
+                         std::min(1.0, reach / ((double)g.tile * g.tile));
+  const double mean = g.nvis * groups / kCellsPlanes * reach / 32 / (152.0 * 32.0);
+  if (densest > 1.5 * mean + 64.0) return grid_cells_split<2, 4>(g, coef, ix, vis, planes, b0, nb, s);
+  return grid_cells_split<8, 1>(g, coef, ix, vis, planes, b0, nb, s);
+}
+
 template <typename R, int G>
 static cudaError_t grid_owner_g(const Geom& g, const Coef<R>& coef, const IndexView<R>& ix,
                                 const typename C2<R>::T* vis, const R* wgt,
@@ -1542,8 +1614,7 @@ static cudaError_t grid_owner_g(const Geom& g, const Coef<R>& coef, const IndexV
   // cell for idle updates
   const int pitch = g.tile + 2;
   const size_t per = (size_t)g.tile * pitch * sizeof(typename C2<R>::T);
-  const size_t stage = (sizeof(R) == 8 && g.df64_planes) ? sizeof(GridStageDD<G>) : sizeof(GridStage<R, G>);
-  const size_t fixed = coef_bytes<R>() + stage;
+  const size_t fixed = coef_bytes<R>() + sizeof(GridStage<R, G>);
   const int nwarps = kOwnerWarps;
   int bs = (int)std::max<size_t>(1, (kGridSmemBudget - fixed) / per);
   if (bs > nwarps) bs -= bs % nwarps;  // equal planes per warp
@@ -1552,13 +1623,9 @@ static cudaError_t grid_owner_g(const Geom& g, const Coef<R>& coef, const IndexV
   int64_t ntiles = (int64_t)g.ntu * g.ntv;
   dim3 grid((unsigned)ntiles, (unsigned)((nb + bs - 1) / bs));
   if constexpr (sizeof(R) == 8) {
-    if (g.df64_planes) {
-      cudaError_t e = cudaFuncSetAttribute(k_grid_owner_dd<G>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      k_grid_owner_dd<G><<<grid, kOwnerThreads, smem, s>>>(g, coef, ix, vis, planes, b0, nb, bs, pitch);
-      return cudaGetLastError();
-    }
+    if (g.df64_planes)
+      return grid_cells_dd(g, coef, ix, reinterpret_cast<const float4*>(vis),
+                           reinterpret_cast<float4*>(planes), b0, nb, s);
   }
   cudaError_t e = cudaFuncSetAttribute(k_grid_owner<R, G>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
