@@ -545,6 +545,7 @@ constexpr int kPairMaxPart = 2048, kPairStages = 12;
 
 struct PairLine {
   int n, S, T, cls, nst;         // points per CTA, CTAs per line, threads, register class, stages
+  int P, TL;                     // pairs of lines per CTA, threads of a pair
   int radix[kPairStages];
   unsigned magic[kPairStages];   // j / Ns = umulhi(j, magic) for Ns > 1
   int twofs[kPairStages];        // first entry of the stage's twiddles, entry (kk - 1) Ns + jm
@@ -613,6 +614,7 @@ struct PairStageArgs {
   int n, Ns;
   unsigned magic;
   int S, h;                      // the line's element S o + h is result o of this CTA
+  int j, TL;                     // thread within the pair's, and how many these are
 };
 // One stage: read the butterflies and transform them, synchronise, write them back in place.
 // kIn: 0 the first stage of a whole line, from global memory; 1 the first stage of a split line,
@@ -652,13 +654,13 @@ __device__ __forceinline__ void pair_barrier() { asm volatile("barrier.sync 0;" 
 
 // NB: butterflies per thread, exactly as many as the CTA's threads need (idle rounds cost as much
 // as full ones)
-template <int R, int NB, int kIn, bool kLast>
+template <int R, int NB, int kIn, bool kLast, bool kPack>
 __device__ __forceinline__ void pair_stage_nb(const PairIo& io, const PairStageArgs& a) {
   constexpr bool kWait = kIn != 0 && !kLast;   // every point of the buffer is read before it is written
-  const int M = a.n / R, T = blockDim.x, Ns = kIn == 2 ? a.Ns : 1;
+  const int M = a.n / R, T = kPack ? a.TL : blockDim.x, Ns = kIn == 2 ? a.Ns : 1;
+  const int j = kPack ? a.j : threadIdx.x;
   if constexpr (NB == 1) {
-    const int j = threadIdx.x;
-    if ((j & ~31) < M) {
+    if (kPack ? __any_sync(0xffffffffu, j < M) : (j & ~31) < M) {
       Cx<d2> x[R];
       const int o = pair_compute<R, kIn, kLast>(io, a, min(j, M - 1), M, Ns, x);
       if (kWait) pair_barrier();
@@ -671,53 +673,53 @@ __device__ __forceinline__ void pair_stage_nb(const PairIo& io, const PairStageA
     int o[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b)
-      o[b] = pair_compute<R, kIn, kLast>(io, a, min((int)threadIdx.x + b * T, M - 1), M, Ns, x[b]);
+      o[b] = pair_compute<R, kIn, kLast>(io, a, min(j + b * T, M - 1), M, Ns, x[b]);
     if (kWait) pair_barrier();
 #pragma unroll
     for (int b = 0; b < NB; ++b)
-      if ((int)threadIdx.x + b * T < M) pair_result<R, kLast>(io, a, o[b], Ns, x[b]);
+      if ((!kPack || j < T) && j + b * T < M) pair_result<R, kLast>(io, a, o[b], Ns, x[b]);
   }
   if (!kLast) pair_barrier();
 }
-template <int R, int CLS, int kIn, bool kLast>
+template <int R, int CLS, int kIn, bool kLast, bool kPack>
 __device__ __forceinline__ void pair_stage(const PairIo& io, const PairStageArgs& a) {
   constexpr int kMost = pair_nb(CLS, R);
-  const int M = a.n / R, T = blockDim.x;
-  if (kMost == 1 || M <= T) pair_stage_nb<R, 1, kIn, kLast>(io, a);
-  else if (kMost == 2 || M <= 2 * T) pair_stage_nb<R, kMost < 2 ? 1 : 2, kIn, kLast>(io, a);
-  else if (kMost == 3 || M <= 3 * T) pair_stage_nb<R, kMost < 3 ? 1 : 3, kIn, kLast>(io, a);
-  else pair_stage_nb<R, kMost < 4 ? 1 : kMost, kIn, kLast>(io, a);
+  const int M = a.n / R, T = kPack ? a.TL : blockDim.x;
+  if (kMost == 1 || M <= T) pair_stage_nb<R, 1, kIn, kLast, kPack>(io, a);
+  else if (kMost == 2 || M <= 2 * T) pair_stage_nb<R, kMost < 2 ? 1 : 2, kIn, kLast, kPack>(io, a);
+  else if (kMost == 3 || M <= 3 * T) pair_stage_nb<R, kMost < 3 ? 1 : 3, kIn, kLast, kPack>(io, a);
+  else pair_stage_nb<R, kMost < 4 ? 1 : kMost, kIn, kLast, kPack>(io, a);
 }
-template <int CLS, int kIn, bool kLast>
+template <int CLS, int kIn, bool kLast, bool kPack>
 __device__ __forceinline__ void pair_dispatch(int R, const PairIo& io, const PairStageArgs& a) {
   if constexpr (kIn != 2) {   // first radix: 8 or 9 (class 9), 8 to 12 (class 12), see pair_plan
     if constexpr (CLS == 9) {
-      if (R == 8) pair_stage<8, CLS, kIn, kLast>(io, a);
-      else pair_stage<9, CLS, kIn, kLast>(io, a);
+      if (R == 8) pair_stage<8, CLS, kIn, kLast, kPack>(io, a);
+      else pair_stage<9, CLS, kIn, kLast, kPack>(io, a);
     } else {
       switch (R) {
-        case 8: pair_stage<8, CLS, kIn, kLast>(io, a); break;
-        case 9: pair_stage<9, CLS, kIn, kLast>(io, a); break;
-        case 10: pair_stage<10, CLS, kIn, kLast>(io, a); break;
-        case 11: pair_stage<11, CLS, kIn, kLast>(io, a); break;
-        default: pair_stage<12, CLS, kIn, kLast>(io, a); break;
+        case 8: pair_stage<8, CLS, kIn, kLast, kPack>(io, a); break;
+        case 9: pair_stage<9, CLS, kIn, kLast, kPack>(io, a); break;
+        case 10: pair_stage<10, CLS, kIn, kLast, kPack>(io, a); break;
+        case 11: pair_stage<11, CLS, kIn, kLast, kPack>(io, a); break;
+        default: pair_stage<12, CLS, kIn, kLast, kPack>(io, a); break;
       }
     }
   } else {
     switch (R) {
-      case 2: pair_stage<2, CLS, kIn, kLast>(io, a); break;
-      case 3: pair_stage<3, CLS, kIn, kLast>(io, a); break;
-      case 4: pair_stage<4, CLS, kIn, kLast>(io, a); break;
-      case 5: pair_stage<5, CLS, kIn, kLast>(io, a); break;
-      case 6: pair_stage<6, CLS, kIn, kLast>(io, a); break;
-      case 7: pair_stage<7, CLS, kIn, kLast>(io, a); break;
-      case 8: pair_stage<8, CLS, kIn, kLast>(io, a); break;
-      case 9: pair_stage<9, CLS, kIn, kLast>(io, a); break;
+      case 2: pair_stage<2, CLS, kIn, kLast, kPack>(io, a); break;
+      case 3: pair_stage<3, CLS, kIn, kLast, kPack>(io, a); break;
+      case 4: pair_stage<4, CLS, kIn, kLast, kPack>(io, a); break;
+      case 5: pair_stage<5, CLS, kIn, kLast, kPack>(io, a); break;
+      case 6: pair_stage<6, CLS, kIn, kLast, kPack>(io, a); break;
+      case 7: pair_stage<7, CLS, kIn, kLast, kPack>(io, a); break;
+      case 8: pair_stage<8, CLS, kIn, kLast, kPack>(io, a); break;
+      case 9: pair_stage<9, CLS, kIn, kLast, kPack>(io, a); break;
       default:
         if constexpr (CLS == 12) {
-          if (R == 10) pair_stage<10, CLS, kIn, kLast>(io, a);
-          else if (R == 11) pair_stage<11, CLS, kIn, kLast>(io, a);
-          else pair_stage<12, CLS, kIn, kLast>(io, a);
+          if (R == 10) pair_stage<10, CLS, kIn, kLast, kPack>(io, a);
+          else if (R == 11) pair_stage<11, CLS, kIn, kLast, kPack>(io, a);
+          else pair_stage<12, CLS, kIn, kLast, kPack>(io, a);
         }
         break;
     }
@@ -746,7 +748,7 @@ __device__ __forceinline__ void pair_split(const PairLine& L, const PairIo& io, 
 
 // Lines q = 2 p, 2 p + 1 (p = pair index in the plane) of `lines` per plane; line q >= split is
 // shifted by skip.  lhalf, shalf as in k_fft_lines; float pairs in and out.
-template <int CLS, int TMAX>
+template <int CLS, int TMAX, bool kPack>
 __global__ void __launch_bounds__(TMAX, 2)
 k_fft_pairs(const __grid_constant__ PairLine L, float4* __restrict__ data, int64_t plane_elems,
             int lines, int64_t line_stride, int64_t elem_stride, int inv, int split, int skip,
@@ -755,9 +757,13 @@ k_fft_pairs(const __grid_constant__ PairLine L, float4* __restrict__ data, int64
   const int S = L.S;
   const unsigned cid = S > 1 ? blockIdx.x / (unsigned)S : blockIdx.x;
   const int h = (int)(blockIdx.x - cid * S);   // rank in the cluster (S, 1, 1)
-  const unsigned pairs = (unsigned)(lines + 1) / 2;
-  const unsigned plane = cid / pairs;
-  const int q0 = 2 * (int)(cid - plane * pairs), q1 = q0 + 1;
+  const unsigned pairs = (unsigned)(lines + 1) / 2, groups = kPack ? (pairs + L.P - 1) / L.P : pairs;
+  const unsigned plane = cid / groups;
+  // threads past the last pair's are idle; pairs past the plane's last repeat it (they read and
+  // write what it does, on the same sides of the barriers)
+  const int sub = kPack ? min((int)threadIdx.x / L.TL, L.P - 1) : 0;
+  const int at = (int)(cid - plane * groups);
+  const int q0 = 2 * (kPack ? min(at * L.P + sub, (int)pairs - 1) : at), q1 = q0 + 1;
   PairIo io;
   io.data = data;
   const int64_t pb = (int64_t)plane * plane_elems;
@@ -768,8 +774,10 @@ k_fft_pairs(const __grid_constant__ PairLine L, float4* __restrict__ data, int64
   io.lhalf = lhalf; io.shalf = shalf;
   io.inv = inv != 0; io.two = q1 < lines;
   PairStageArgs a;
-  a.sr = reinterpret_cast<ulonglong2*>(fsm);
-  a.si = a.sr + ((L.n + 7) & ~7);
+  const int room = (L.n + 7) & ~7;
+  a.sr = reinterpret_cast<ulonglong2*>(fsm) + (kPack ? 2 * room * sub : 0);
+  a.si = a.sr + room;
+  if (kPack) { a.j = (int)threadIdx.x - sub * L.TL; a.TL = L.TL; }
   a.n = L.n; a.S = S; a.h = h;
   if (S > 1) {
     // every CTA of the cluster must have started before its buffer is written
@@ -779,20 +787,20 @@ k_fft_pairs(const __grid_constant__ PairLine L, float4* __restrict__ data, int64
     else if (S == 4) pair_split<4>(L, io, a.sr, a.si, h);
     else pair_split<8>(L, io, a.sr, a.si, h);
     cl.sync();
-    pair_dispatch<CLS, 1, false>(L.radix[0], io, a);
+    pair_dispatch<CLS, 1, false, kPack>(L.radix[0], io, a);
   } else {
-    pair_dispatch<CLS, 0, false>(L.radix[0], io, a);
+    pair_dispatch<CLS, 0, false, kPack>(L.radix[0], io, a);
   }
   a.Ns = L.radix[0];
   int st = 1;
   for (; st < L.nst - 1; ++st) {
     a.tw = L.tw + 2 * L.twofs[st];
     a.magic = L.magic[st];
-    pair_dispatch<CLS, 2, false>(L.radix[st], io, a);
+    pair_dispatch<CLS, 2, false, kPack>(L.radix[st], io, a);
     a.Ns *= L.radix[st];
   }
   a.tw = L.tw + 2 * L.twofs[st];
-  pair_dispatch<CLS, 2, true>(L.radix[st], io, a);
+  pair_dispatch<CLS, 2, true, kPack>(L.radix[st], io, a);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -807,10 +815,11 @@ static dd host_dd(long double v) {
 
 // One side's transform: pairs of lines where the side allows it, else one line per CTA / cluster.
 struct SideFft {
-  bool pairs = false;
+  bool pairs = false, fwd_lines = false;   // fwd_lines: one line per CTA for the forward transform
   PairLine pl;
   FftLine fl;
-  float4* tw = nullptr;   // line twiddles, then (split lines) the decimation twiddles
+  // line twiddles, then (split lines) the decimation twiddles; those of fl beside pairs
+  float4 *tw = nullptr, *twl = nullptr;
 };
 struct Df64Fft {
   int nu = 0, nv = 0;
@@ -847,6 +856,8 @@ static void pair_search(int m, int maxr, int depth, double cost, PairLine* cur, 
     *out = *cur;
     out->nst = depth;
     out->T = T;
+    out->P = 1;
+    out->TL = T;
     return;
   }
   if (depth == kPairStages) return;
@@ -876,8 +887,31 @@ static bool pair_part(int N, int S, PairLine* L) {
 // threads 1.04 / 0.97 against 1.11 / 1.07).  Left to one line per CTA, which is as fast or faster: up
 // to 2048 points what one CTA cannot take (2016: 0.89 / 0.93), and between 3072 and 4096 points
 // sides with a factor 11, or with 7 and 5 (3168: 1.08 / 0.95, 3520: 0.98 / 0.91, 3360: 1.02 / 0.86).
+// Several pairs per CTA where their threads fill its warps better: as many as give the most pairs
+// per SM, from 33 threads a pair up (576 points, 72 threads a pair: one to a CTA of 96 measured
+// 0.95 / 1.66 times the line kernels' speed forward / inverse, two to a CTA of 160 1.04 / 1.77;
+// 672, 112 threads: 1.19 / 1.86 alone and 1.09 / 1.74 with two, no more pairs per SM; 128, 16
+// threads: 0.97 / 1.86 alone and 0.78 / 1.40 with four, too few CTAs).
+static void pair_pack(PairLine* L) {
+  int tl = 1;
+  for (int i = 0; i < L->nst; ++i) {
+    const int per = L->n / L->radix[i], nb = pair_nb(L->cls, L->radix[i]);
+    tl = std::max(tl, (per + nb - 1) / nb);
+  }
+  if (tl <= 32) return;
+  const int room = L->cls == 9 ? 512 : 384;   // threads an SM holds
+  int best = room / L->T;
+  for (int P = 2; P * tl <= pair_threads(L->cls) && P * ((L->n + 7) & ~7) <= kPairMaxPart; ++P) {
+    const int T = (P * tl + 31) / 32 * 32;
+    if (P * (room / T) > best) { best = P * (room / T); L->P = P; L->TL = tl; L->T = T; }
+  }
+}
 static bool pair_plan(int N, PairLine* L) {
-  if (N <= kPairMaxPart) return pair_part(N, 1, L);
+  if (N <= kPairMaxPart) {
+    if (!pair_part(N, 1, L)) return false;
+    pair_pack(L);
+    return true;
+  }
   if (N > 3072 && N < 4096 && (N % 11 == 0 || N % 35 == 0)) return false;
   if (N >= 3072 && pair_part(N, 4, L) && L->n <= 1024 && L->cls == 9 && L->T <= 160) return true;
   for (int S : {2, 4, 8})
@@ -945,13 +979,13 @@ static cudaError_t launch_pairs(const PairLine& L, double2* data, int64_t batch,
                                 int lines, int64_t line_stride, int64_t elem_stride, int fwd,
                                 int split, int skip, int lhalf, int shalf, cudaStream_t s) {
   if (lines == 0 || batch == 0) return cudaSuccess;
-  const int64_t blocks = batch * ((lines + 1) / 2) * L.S;
+  const int64_t blocks = batch * (((lines + 1) / 2 + L.P - 1) / L.P) * L.S;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)blocks);
   cfg.blockDim = dim3((unsigned)L.T);
-  cfg.dynamicSmemBytes = 2 * sizeof(float4) * (size_t)((L.n + 7) & ~7);
+  cfg.dynamicSmemBytes = 2 * sizeof(float4) * (size_t)((L.n + 7) & ~7) * L.P;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   std::memset(attr, 0, sizeof(attr));
@@ -963,10 +997,11 @@ static cudaError_t launch_pairs(const PairLine& L, double2* data, int64_t batch,
   cfg.numAttrs = L.S > 1 ? 1 : 0;
   float4* d = reinterpret_cast<float4*>(data);
   const int inv = fwd ? 0 : 1;
-#define WG_PAIRS(C, TM)                                                                          \
-  cudaLaunchKernelEx(&cfg, k_fft_pairs<C, TM>, L, d, plane, lines, line_stride, elem_stride, inv, \
+#define WG_PAIRS(C, TM, P)                                                                       \
+  cudaLaunchKernelEx(&cfg, k_fft_pairs<C, TM, P>, L, d, plane, lines, line_stride, elem_stride, inv, \
                      split, skip, lhalf, shalf)
-  return L.cls == 9 ? WG_PAIRS(9, 256) : WG_PAIRS(12, 192);
+  if (L.P > 1) return L.cls == 9 ? WG_PAIRS(9, 256, true) : WG_PAIRS(12, 192, true);
+  return L.cls == 9 ? WG_PAIRS(9, 256, false) : WG_PAIRS(12, 192, false);
 #undef WG_PAIRS
 }
 
@@ -1029,7 +1064,15 @@ static cudaError_t make_line(int nline, FftLine* L, float4** tw) {
 
 static cudaError_t make_side(int n, SideFft* f) {
   f->pairs = pair_plan(n, &f->pl);
-  return f->pairs ? make_pairs(&f->pl, &f->tw) : make_line(n, &f->fl, &f->tw);
+  if (!f->pairs) return make_line(n, &f->fl, &f->tw);
+  // sides of the radices 2 and 5 only, which pairs take in four stages with idle lanes: forward
+  // and inverse at the pairs' speed against the lines', on square sides with pruning: 640 0.92 /
+  // 1.65, 800 0.98 / 1.44, 1280 1.02 / 1.28, 1600 0.92 / 1.10 (other sides from 0.97 up: 128; 1152
+  // 1.03 / 1.40, 960 and up)
+  f->fwd_lines = f->pl.S == 1 && n >= 640 && n % 5 == 0 && n % 3 && n % 7 && n % 11;
+  cudaError_t e = make_pairs(&f->pl, &f->tw);
+  if (e == cudaSuccess && f->fwd_lines) e = make_line(n, &f->fl, &f->twl);
+  return e;
 }
 
 cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
@@ -1042,7 +1085,7 @@ cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
   const int smax = (int)(2 * kMaxSide * sizeof(float4));
 #define WG_SMEM_ATTR(K, BYTES)                                                                   \
   if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, BYTES)
-  if (!f->u.pairs || !f->v.pairs) {
+  if (!f->u.pairs || !f->v.pairs || f->u.fwd_lines || f->v.fwd_lines) {
     WG_SMEM_ATTR((k_fft_lines<448, 2, false, false, false>), smax); WG_SMEM_ATTR((k_fft_lines<448, 2, false, true, false>), smax);
     WG_SMEM_ATTR((k_fft_lines<448, 2, true, false, false>), smax);  WG_SMEM_ATTR((k_fft_lines<448, 2, true, true, false>), smax);
     WG_SMEM_ATTR((k_fft_lines<832, 1, false, false, false>), smax); WG_SMEM_ATTR((k_fft_lines<832, 1, false, true, false>), smax);
@@ -1053,8 +1096,8 @@ cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
     WG_SMEM_ATTR((k_fft_lines_cluster<832, 1, false>), smax); WG_SMEM_ATTR((k_fft_lines_cluster<832, 1, true>), smax);
   }
   const int spair = (int)(2 * sizeof(float4) * kPairMaxPart);
-  WG_SMEM_ATTR((k_fft_pairs<9, 256>), spair);
-  WG_SMEM_ATTR((k_fft_pairs<12, 192>), spair);
+  WG_SMEM_ATTR((k_fft_pairs<9, 256, false>), spair);  WG_SMEM_ATTR((k_fft_pairs<9, 256, true>), spair);
+  WG_SMEM_ATTR((k_fft_pairs<12, 192, false>), spair); WG_SMEM_ATTR((k_fft_pairs<12, 192, true>), spair);
 #undef WG_SMEM_ATTR
   if (e != cudaSuccess) {
     df64_fft_destroy(f);
@@ -1066,8 +1109,10 @@ cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
 
 void df64_fft_destroy(Df64Fft* f) {
   if (f == nullptr) return;
-  if (f->u.tw) cudaFree(f->u.tw);
-  if (f->v.tw) cudaFree(f->v.tw);
+  for (SideFft* side : {&f->u, &f->v}) {
+    if (side->tw) cudaFree(side->tw);
+    if (side->twl) cudaFree(side->twl);
+  }
   delete f;
 }
 
@@ -1144,10 +1189,11 @@ static cudaError_t launch_lines(const FftLine& L, double2* data, int64_t batch, 
 static cudaError_t launch_side(const SideFft& f, double2* data, int64_t batch, int64_t plane,
                                int lines, int64_t line_stride, int64_t elem_stride, int mode,
                                int fwd, int split, int skip, int lhalf, int shalf, cudaStream_t s) {
-  return f.pairs ? launch_pairs(f.pl, data, batch, plane, lines, line_stride, elem_stride, fwd, split,
-                                skip, lhalf, shalf, s)
-                 : launch_lines(f.fl, data, batch, plane, lines, line_stride, elem_stride, mode, fwd,
-                                split, skip, lhalf, shalf, s);
+  return f.pairs && !(fwd && f.fwd_lines)
+             ? launch_pairs(f.pl, data, batch, plane, lines, line_stride, elem_stride, fwd, split,
+                            skip, lhalf, shalf, s)
+             : launch_lines(f.fl, data, batch, plane, lines, line_stride, elem_stride, mode, fwd,
+                            split, skip, lhalf, shalf, s);
 }
 
 // complex128 planes to float pairs and back, in place (the FFT utilities; the plans keep pairs)

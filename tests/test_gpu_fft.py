@@ -103,12 +103,14 @@ def test_f32_fft_shapes(wg, tune, sign):
 
 @pytest.mark.parametrize("shape", [(2, 15, 16), (1, 9, 256), (1, 33, 704), (3, 7, 1440), (1, 1728, 15),
                                    (1, 2048, 3), (1, 5, 3072), (1, 3456, 21), (1, 27, 3840),
-                                   (1, 6144, 5), (1, 11, 5632), (1, 8192, 9), (1, 3, 12288)])
+                                   (1, 6144, 5), (1, 11, 5632), (1, 8192, 9), (1, 3, 12288),
+                                   (2, 9, 576), (1, 320, 11), (1, 640, 5)])
 @pytest.mark.parametrize("sign", [-1, 1])
 def test_df64_line_pairs_against_numpy(wg, shape, sign):
     """The kernels that transform two lines at once: both register classes (radices up to 9, and
     10 to 12), whole lines and lines split over clusters of 2, 4 and 8 CTAs, rows and strided
-    columns, an odd number of lines (the last one alone in its pair).  The bound is the FFT's own:
+    columns, an odd number of lines (the last one alone in its pair), several pairs per CTA with
+    the last CTA of a plane incomplete, and the side that goes line by line forward.  The bound is the FFT's own:
     normwise 5e-14."""
     rng = np.random.default_rng(sum(shape) + 3 * sign)
     x = rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
