@@ -18,6 +18,9 @@
 //    used for FP64, where shared-memory double atomics occupy the FP64 pipe);
 //  * FP64 plans with the double-float FFT keep the planes as double-float pairs and run the
 //    degridding and plane-owner gridding in pair arithmetic on the FP32 pipes (df64.cuh).
+#include <cmath>
+#include <type_traits>
+
 #include "df64.cuh"
 #include "fft_engine.cuh"
 #include "wgrid_internal.h"
@@ -96,6 +99,45 @@ __device__ __forceinline__ unsigned group_mask() {
   return G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
 }
 
+// The visibilities of tile t that meet each of the planes s0 .. s0 + sb - 1 (at most 32): lane pl
+// holds plane s0 + pl's index range, so that all are known after one load.
+struct DegridRange {
+  uint32_t lo, hi;   // over all the planes; this CTA's share of them after split()
+  unsigned used;     // planes some visibility meets
+  __device__ __forceinline__ DegridRange(const uint32_t* __restrict__ offt, int nw, int aw, int s0, int sb) {
+    const int lane = threadIdx.x & 31, p = s0 + min(lane, sb - 1);
+    const uint32_t a = offt[max(0, p - aw + 1)], b = offt[min(p + 1, nw)];
+    lo = __shfl_sync(0xffffffffu, a, 0);
+    hi = __shfl_sync(0xffffffffu, b, sb - 1);
+    used = __ballot_sync(0xffffffffu, lane < sb && a != b);
+  }
+  // blockIdx.z's share among gridDim.z CTAs, of at least `least` visibilities (a multiple of 64, so
+  // that shares are whole passes of a CTA): only tiles with more are taken by several
+  __device__ __forceinline__ void split(uint32_t least) {
+    if (gridDim.z == 1) return;
+    const uint32_t share = max(least, ((hi - lo + gridDim.z - 1) / gridDim.z + 63) & ~63u);
+    lo = min(hi, lo + blockIdx.z * share);
+    hi = min(hi, lo + share);
+  }
+};
+// f(cell of the buffer, cell of the plane) for the tile and its halo in the used planes: a warp
+// takes whole rows, so a cell costs an addition
+template <typename F>
+__device__ __forceinline__ void degrid_rows(const Geom& g, int tu, int tv, int p0, int sb, unsigned used, F f) {
+  const int T = g.tile, TH = T + g.alpha - 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t pstride = (int64_t)g.nu * g.nv;
+  for (int c = lane; c < TH; c += 32) {
+    int gv = tv * T + c; if (gv >= g.nv) gv -= g.nv;
+    for (int pl = 0; pl < sb; ++pl) {
+      if (!((used >> pl) & 1)) continue;
+      for (int r = warp; r < TH; r += kThreads / 32) {
+        int gu = tu * T + r; if (gu >= g.nu) gu -= g.nu;
+        f((pl * TH + r) * TH + c, (p0 + pl) * pstride + (int64_t)gu * g.nv + gv);
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------------------
 // degrid
 //
@@ -107,12 +149,20 @@ __device__ __forceinline__ unsigned group_mask() {
 // bs over the whole plane range, so a visibility meets at most `nslot` of them; a finalize pass
 // adds its slots in slot order (deterministic, no atomics) and applies the w-reference phase,
 // the Hermitian fold and the weight.
+//
+// Bound by the staged bytes from L2 (half of the time of double-float planes on 16-cell tiles, where
+// the halo makes 3.6 times the tile's cells) and then by the latency of the footprint sums.  So the
+// index ranges of all planes come in one load, rows are copied without a division per cell, the
+// next visibility's index entry is loaded ahead, and dense tiles go to several CTAs (see degrid_g).
+// Measured before and after, FP32: 1e6 visibilities on a 2048^2 image, alpha = 8, 0.69 -> 0.62 ms; 1e7
+// on 4096^2 4.10 -> 3.90; with a tenth of 8e5 visibilities in one tile, alpha = 6, 3.15 -> 0.63.  (Real
+// and imaginary part packed in one FMA: 0.74 / 0.66 / 0.74 ms with one / two / four planes at once.)
 // ---------------------------------------------------------------------------------------
 template <typename R, int G>
 __global__ void __launch_bounds__(kThreads)
 k_degrid(const Geom g, const __grid_constant__ Coef<R> coef, const IndexView<R> ix,
          const typename C2<R>::T* __restrict__ planes, int b0, int nb, int bs,
-         typename C2<R>::T* __restrict__ partial, int64_t nvis_idx) {
+         typename C2<R>::T* __restrict__ partial, int64_t nvis_idx, uint32_t least) {
   using CT = typename C2<R>::T;
   extern __shared__ __align__(16) unsigned char smem[];
   R* sc = reinterpret_cast<R*>(smem);
@@ -124,23 +174,20 @@ k_degrid(const Geom g, const __grid_constant__ Coef<R> coef, const IndexView<R> 
   const int s0 = b0 + blockIdx.y * bs;
   const int sb = min(bs, b0 + nb - s0);
   const int sbid = s0 / bs;                       // global sub-batch id (s0 is a multiple of bs)
-  const uint32_t* offt = ix.off + (int64_t)t * g.nw;
-  const uint32_t lo = offt[max(0, s0 - aw + 1)], hi = offt[min(g.nw, s0 + sb)];
+  DegridRange range(ix.off + (int64_t)t * g.nw, g.nw, aw, s0, sb);
+  range.split(least);
+  const uint32_t lo = range.lo, hi = range.hi;
   if (lo == hi) return;                           // no visibility of this tile meets these planes
+  degrid_rows(g, tu, tv, s0 - b0, sb, range.used,
+              [&](int e, int64_t cell) { stage_copy(st + e, planes + cell); });
   for (int i = threadIdx.x; i < (g.deg + 1) * kMaxG; i += blockDim.x) sc[i] = coef.c[i];
-  const int64_t pstride = (int64_t)g.nu * g.nv;
-  for (int pl = 0; pl < sb; ++pl) {
-    const int p = s0 + pl;
-    if (offt[max(0, p - aw + 1)] == offt[min(p + 1, g.nw)]) continue;  // plane unused here
-    const CT* src = planes + (int64_t)(p - b0) * pstride;
-    CT* dst = st + pl * TH * TH;
-    for (int e = threadIdx.x; e < TH * TH; e += blockDim.x) {
-      int r = e / TH, c = e - r * TH;
-      int gu = tu * T + r; if (gu >= g.nu) gu -= g.nu;
-      int gv = tv * T + c; if (gv >= g.nv) gv -= g.nv;
-      stage_copy(dst + e, src + (int64_t)gu * g.nv + gv);
-    }
-  }
+  // the index entries of a group's next visibility are loaded while the current one is summed,
+  // the first one's while the planes are staged
+  const uint32_t gofs = (threadIdx.x / G) % (32 / G);
+  uint32_t v0 = lo + (threadIdx.x >> 5) * (32 / G), mt_n = 0;
+  Z4<R> zz_n;
+  zz_n.u = zz_n.v = zz_n.w = zz_n.pad = (R)0;
+  if (v0 + gofs < hi) { mt_n = ix.meta[v0 + gofs]; zz_n = ix.z[v0 + gofs]; }
   stage_wait();
   __syncthreads();
   // G lanes per visibility (lane j = piece / footprint column j).  Visibilities of a tile are
@@ -152,13 +199,12 @@ k_degrid(const Geom g, const __grid_constant__ Coef<R> coef, const IndexView<R> 
   if (sizeof(R) == 4) pc.load(sc, g.deg, j);
   const int grp = threadIdx.x / G, ngrp = blockDim.x / G;
   const unsigned gmask = group_mask<G>();
-  for (uint32_t v0 = lo + (threadIdx.x >> 5) * (32 / G); v0 < hi; v0 += ngrp) {
-    const uint32_t vi = v0 + (grp % (32 / G));
+  for (; v0 < hi; v0 += ngrp) {
+    const uint32_t vi = v0 + gofs;
     const bool act = vi < hi;
-    uint32_t mt = 0;
-    Z4<R> zz;
-    zz.u = zz.v = zz.w = zz.pad = (R)0;
-    if (act) { mt = ix.meta[vi]; zz = ix.z[vi]; }
+    const uint32_t mt = act ? mt_n : 0u;
+    const Z4<R> zz = zz_n;
+    if (vi + ngrp < hi) { mt_n = ix.meta[vi + ngrp]; zz_n = ix.z[vi + ngrp]; }
     const int du = mt & 255, dv = (mt >> 8) & 255, c0 = (int)(mt >> 16);
     const bool lj = act && j < alpha;
     R pu = lj ? kernel_value<R, G>(ix, pc, sc, g.deg, vi, 0, j, zz.u) : (R)0;
@@ -208,11 +254,15 @@ k_degrid(const Geom g, const __grid_constant__ Coef<R> coef, const IndexView<R> 
 // degrid of double-float planes (FP64 plans with the double-float FFT)
 //
 // The same decomposition as k_degrid, on planes whose cells are double-float pairs (float4:
-// re hi, re lo, im hi, im lo): the tile + halo is staged as is, kernel values come as pairs
-// (the kernel-value table stores them split), and the footprint sum runs in pair arithmetic on
-// the FP32 pipes (dd_fma: 15 FP32 instructions for an FP64 FMA, which GB300 issues at 1/64 of
-// the FP32 rate).  Each lane sums its column over rows and planes, the lanes' sums are reduced
-// by shuffles in pair arithmetic, and the partial sum is stored in FP64 as in k_degrid.
+// re hi, re lo, im hi, im lo): the tile + halo is staged and then reordered in place to (re hi, im
+// hi, re lo, im lo), kernel values come as pairs (the kernel-value table stores them split), and the
+// footprint sum runs in pair arithmetic on the FP32 pipes, real and imaginary part packed (15
+// packed FP32 instructions for two FP64 FMAs, which GB300 issues at 1/64 of the FP32 rate).  Each
+// lane sums its column over rows, four planes at once (independent chains; two: 8.5 against 8.3 ms),
+// the u weights come from shared memory (in registers they leave room for two planes only: 9.9 ms),
+// the lanes' sums are reduced by shuffles in pair arithmetic, and the partial sum is stored in
+// FP64 as in k_degrid.  1e6 visibilities on a 3456^2 grid, alpha = 15: 9.6 -> 8.3 ms, 4.2 of them
+// with the sums left out.
 // ---------------------------------------------------------------------------------------
 // piece j of direction d of indexed visibility vi as a double-float pair
 __device__ __forceinline__ dd kernel_value_dd(const IndexView<double>& ix, const double* __restrict__ sc,
@@ -228,11 +278,21 @@ __device__ __forceinline__ dd shfl_dd(dd x, int src, int width) {
   return dd_make(__shfl_sync(0xffffffffu, x.h, src, width), __shfl_sync(0xffffffffu, x.l, src, width));
 }
 
+// w d + c for a weight w given as (wh, wh), (-wh, -wh), (-wl, -wl): dd_fma(w, d, c) on packed values
+__device__ __forceinline__ d2 d2_fma_weight(f2 wh, f2 nwh, f2 nwl, d2 d, d2 c) {
+  const f2 p = s_mul(wh, d.h);
+  f2 e = s_fma(nwh, d.h, p);   // minus all of the product below p
+  e = s_fma(nwh, d.l, e);
+  e = s_fma(nwl, d.h, e);
+  const d2 s = d2_two_sum(c.h, p);
+  return d2_fast_two_sum(s.h, s_add(s.l, s_sub(c.l, e)));
+}
+
 template <int G>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 3)
 k_degrid_dd(const Geom g, const __grid_constant__ Coef<double> coef, const IndexView<double> ix,
             const double2* __restrict__ planes, int b0, int nb, int bs,
-            double2* __restrict__ partial, int64_t nvis_idx) {
+            double2* __restrict__ partial, int64_t nvis_idx, uint32_t least) {
   extern __shared__ __align__(16) unsigned char smem[];
   double* sc = reinterpret_cast<double*>(smem);
   double2* st = reinterpret_cast<double2*>(smem + (kMaxDeg + 1) * kMaxG * sizeof(double));
@@ -243,30 +303,18 @@ k_degrid_dd(const Geom g, const __grid_constant__ Coef<double> coef, const Index
   const int s0 = b0 + blockIdx.y * bs;
   const int sb = min(bs, b0 + nb - s0);
   const int sbid = s0 / bs;                       // global sub-batch id (s0 is a multiple of bs)
-  const uint32_t* offt = ix.off + (int64_t)t * g.nw;
-  const uint32_t lo = offt[max(0, s0 - aw + 1)], hi = offt[min(g.nw, s0 + sb)];
+  DegridRange range(ix.off + (int64_t)t * g.nw, g.nw, aw, s0, sb);
+  range.split(least);
+  const uint32_t lo = range.lo, hi = range.hi;
   if (lo == hi) return;                           // no visibility of this tile meets these planes
-  for (int i = threadIdx.x; i < (g.deg + 1) * kMaxG; i += blockDim.x) sc[i] = coef.c[i];
-  const int64_t pstride = (int64_t)g.nu * g.nv;
-  for (int pl = 0; pl < sb; ++pl) {
-    const int p = s0 + pl;
-    if (offt[max(0, p - aw + 1)] == offt[min(p + 1, g.nw)]) continue;  // plane unused here
-    const double2* src = planes + (int64_t)(p - b0) * pstride;
-    double2* dst = st + pl * TH * TH;
-    for (int e = threadIdx.x; e < TH * TH; e += blockDim.x) {
-      int r = e / TH, c = e - r * TH;
-      int gu = tu * T + r; if (gu >= g.nu) gu -= g.nu;
-      int gv = tv * T + c; if (gv >= g.nv) gv -= g.nv;
-      stage_copy(dst + e, src + (int64_t)gu * g.nv + gv);   // 16 bytes, copied as they are
-    }
-  }
-  stage_wait();
-  __syncthreads();
   const int j = threadIdx.x & (G - 1);
   const int grp = threadIdx.x / G, ngrp = blockDim.x / G;
   const dd zero = dd_make(0.f, 0.f);
+  float4* wt = reinterpret_cast<float4*>(st + (size_t)min(bs, nb) * TH * TH) + grp * G;
+  float2* wt2 = reinterpret_cast<float2*>(wt + (ngrp - grp) * G) + grp * G;
   // with a kernel-value table, the group's next visibility's index entry and table values are
-  // loaded while the current one is summed (the loads' latency is otherwise exposed)
+  // loaded while the current one is summed (the loads' latency is otherwise exposed), and the
+  // first one's while the planes are staged
   const float2* tw = reinterpret_cast<const float2*>(ix.wts);
   const uint32_t gofs = grp % (32 / G);
   uint32_t mt_n = 0;
@@ -282,6 +330,19 @@ k_degrid_dd(const Geom g, const __grid_constant__ Coef<double> coef, const Index
   };
   uint32_t v0 = lo + (threadIdx.x >> 5) * (32 / G);
   prefetch(v0 + gofs);
+  if (tw == nullptr)
+    for (int i = threadIdx.x; i < (g.deg + 1) * kMaxG; i += blockDim.x) sc[i] = coef.c[i];
+  degrid_rows(g, tu, tv, s0 - b0, sb, range.used,
+              [&](int e, int64_t cell) { stage_copy(st + e, planes + cell); });
+  stage_wait();
+  // (re hi, re lo, im hi, im lo) to (re hi, im hi, re lo, im lo): each thread the cells it copied
+  degrid_rows(g, tu, tv, s0 - b0, sb, range.used, [&](int e, int64_t) {
+    float4* v = reinterpret_cast<float4*>(st) + e;
+    const float2 m = make_float2(v->y, v->z);
+    v->y = m.y;
+    v->z = m.x;
+  });
+  __syncthreads();
   for (; v0 < hi; v0 += ngrp) {
     const uint32_t vi = v0 + gofs;
     const bool act = vi < hi;
@@ -304,32 +365,53 @@ k_degrid_dd(const Geom g, const __grid_constant__ Coef<double> coef, const Index
       }
     }
     if (!g.do_w) pw = j == 0 ? dd_make(1.f, 0.f) : zero;
-    dd wu[G];
-#pragma unroll
-    for (int i = 0; i < G; ++i) wu[i] = shfl_dd(pu, i, G);
+    __syncwarp();   // the previous visibility's weights are consumed
+    wt[j] = make_float4(-pu.h, -pu.h, -pu.l, -pu.l);
+    wt2[j] = make_float2(pu.h, pu.h);
+    __syncwarp();
     const int qlo = act ? max(0, s0 - c0) : G, qhi = act ? min(aw, s0 + sb - c0) : 0;
     const int wlo = __reduce_min_sync(0xffffffffu, (unsigned)qlo);
     const int whi = __reduce_max_sync(0xffffffffu, (unsigned)qhi);
-    dd ar = zero, ai = zero;
-    for (int q = wlo; q < whi; ++q) {
-      const dd wq = shfl_dd(pw, q, G);
-      if (lj && q >= qlo && q < qhi) {
-        const float4* row = reinterpret_cast<const float4*>(st + (c0 + q - s0) * TH * TH + du * TH + dv + j);
-        dd sr = zero, si = zero;
+    const int cell = du * TH + dv + (lj ? j : 0);
+    d2 acc{f2_make(0.f, 0.f), f2_make(0.f, 0.f)};   // (re, im)
+    // NP planes from q on at once: their column sums are independent chains
+    auto planes_sum = [&](int q, auto np) {
+      constexpr int NP = decltype(np)::value;
+      const ulonglong2* row[NP];
+      bool on[NP];
+      d2 sum[NP];
 #pragma unroll
-        for (int i = 0; i < G; ++i) {
-          if (i < alpha) {
-            const float4 gv = row[i * TH];
-            sr = dd_fma(wu[i], dd_make(gv.x, gv.y), sr);
-            si = dd_fma(wu[i], dd_make(gv.z, gv.w), si);
+      for (int n = 0; n < NP; ++n) {
+        on[n] = lj && q + n >= qlo && q + n < qhi;
+        const int pl = on[n] ? c0 + q + n - s0 : 0;
+        row[n] = reinterpret_cast<const ulonglong2*>(st) + pl * TH * TH + cell;
+        sum[n].h = sum[n].l = f2_make(0.f, 0.f);
+      }
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        if (i < alpha) {
+          const ulonglong2 nw = *reinterpret_cast<const ulonglong2*>(&wt[i]);
+          const f2 wh{*reinterpret_cast<const pk64*>(&wt2[i])}, nwh{nw.x}, nwl{nw.y};
+#pragma unroll
+          for (int n = 0; n < NP; ++n) {
+            const ulonglong2 v = row[n][i * TH];
+            sum[n] = d2_fma_weight(wh, nwh, nwl, d2{f2{v.x}, f2{v.y}}, sum[n]);
           }
         }
-        ar = dd_fma(wq, sr, ar);
-        ai = dd_fma(wq, si, ai);
       }
-    }
-    ar = dd_mul(ar, pv);
-    ai = dd_mul(ai, pv);
+#pragma unroll
+      for (int n = 0; n < NP; ++n) {
+        const dd wq = shfl_dd(pw, q + n, G);
+        // a plane the visibility does not meet (or a lane past its columns) gave what it read
+        if (!on[n]) sum[n].h = sum[n].l = f2_make(0.f, 0.f);
+        acc = d2_fma_weight(f2_make(wq.h, wq.h), f2_make(-wq.h, -wq.h), f2_make(-wq.l, -wq.l), sum[n], acc);
+      }
+    };
+    int q = wlo;
+    for (; q + 2 < whi; q += 4) planes_sum(q, std::integral_constant<int, 4>());
+    if (q < whi) planes_sum(q, std::integral_constant<int, 2>());
+    const float2 ach = f2_split(acc.h), acl = f2_split(acc.l);
+    dd ar = dd_mul(dd_make(ach.x, acl.x), pv), ai = dd_mul(dd_make(ach.y, acl.y), pv);
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) {
       ar = dd_add(ar, dd_make(__shfl_xor_sync(0xffffffffu, ar.h, o, G), __shfl_xor_sync(0xffffffffu, ar.l, o, G)));
@@ -1560,20 +1642,33 @@ static cudaError_t degrid_g(const Geom& g, const Coef<R>& coef, const IndexView<
                             typename C2<R>::T* partial, int64_t nvis_idx, cudaStream_t s) {
   size_t smem = coef_bytes<R>() + (size_t)std::min(bs, nb) * degrid_plane_bytes<R>(g);
   int64_t ntiles = (int64_t)g.ntu * g.ntv;
-  dim3 grid((unsigned)ntiles, (unsigned)((nb + bs - 1) / bs));
+  // several CTAs for the densest tiles, where one would be the run time (they stage the same planes
+  // and sum different visibilities; the sums are the same).  Measured on 8e5 visibilities with a
+  // fifth in one tile, double-float planes, alpha = 10: 78 ms with one CTA, 26 / 14 / 9 ms with 2 / 4 / 8
+  // for every tile, 5.6 ms by this rule; even plans lose by it (2.1 ms alone, 2.4 with two CTAs at a
+  // densest tile of 179 against a mean of 3 000).  Compared: visibilities of the densest
+  // tile's CTA against the mean over the CTAs the GPU holds at once (a visibility meets
+  // (alpha_w + bs - 1) / bs of the sub-batches)
+  const double meets = g.alpha_w + bs - 1.0;
+  const double densest = g.max_tile * std::min(1.0, meets / g.nw);
+  const double mean = g.nvis * meets / bs / (152.0 * 4.0);
+  const uint32_t least = (uint32_t)std::max(128.0, 0.5 * mean) / 64 * 64;
+  const int Z = densest > 1.5 * mean ? (int)std::min(32.0, std::ceil(densest / least)) : 1;
+  dim3 grid((unsigned)ntiles, (unsigned)((nb + bs - 1) / bs), (unsigned)Z);
   if constexpr (sizeof(R) == 8) {
     if (g.df64_planes) {
+      smem += (size_t)kThreads * (sizeof(float4) + sizeof(float2));
       cudaError_t e = cudaFuncSetAttribute(k_degrid_dd<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem);
       if (e != cudaSuccess) return e;
-      k_degrid_dd<G><<<grid, kThreads, smem, s>>>(g, coef, ix, planes, b0, nb, bs, partial, nvis_idx);
+      k_degrid_dd<G><<<grid, kThreads, smem, s>>>(g, coef, ix, planes, b0, nb, bs, partial, nvis_idx, least);
       return cudaGetLastError();
     }
   }
   cudaError_t e = cudaFuncSetAttribute(k_degrid<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  k_degrid<R, G><<<grid, kThreads, smem, s>>>(g, coef, ix, planes, b0, nb, bs, partial, nvis_idx);
+  k_degrid<R, G><<<grid, kThreads, smem, s>>>(g, coef, ix, planes, b0, nb, bs, partial, nvis_idx, least);
   return cudaGetLastError();
 }
 
@@ -1601,7 +1696,7 @@ static cudaError_t grid_cells_dd(const Geom& g, const Coef<double>& coef, const 
   const double densest = g.max_tile * std::min(1.0, groups / g.nw) *
                          std::min(1.0, reach / ((double)g.tile * g.tile));
   const double mean = g.nvis * groups / kCellsPlanes * reach / 32 / (152.0 * 32.0);
-  if (densest > 1.5 * mean + 64.0) return grid_cells_split<2, 4>(g, coef, ix, vis, planes, b0, nb, s);
+  if (densest > 1.2 * mean + 32.0) return grid_cells_split<2, 4>(g, coef, ix, vis, planes, b0, nb, s);
   return grid_cells_split<8, 1>(g, coef, ix, vis, planes, b0, nb, s);
 }
 
