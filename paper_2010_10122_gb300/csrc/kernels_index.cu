@@ -6,6 +6,7 @@
 // paper's mutex-guarded sorted structure (Sec. 4.4).
 #include <cfloat>
 
+#include "df64.cuh"
 #include "wgrid_internal.h"
 
 namespace wg {
@@ -60,11 +61,21 @@ struct VisPos {
   bool bad;         // plane index had to be clamped (should not happen)
 };
 
+// c modulo n, in 32-bit arithmetic where c allows it
+__device__ __forceinline__ int64_t wrap_cell(double c, int64_t n) {
+  if (((unsigned)__double2hiint(c) & 0x7fffffffu) < 0x41d00000u) {   // |c| < 2^30
+    const int i = (int)c % (int)n;
+    return i < 0 ? i + (int)n : i;
+  }
+  const int64_t i = (int64_t)c % n;
+  return i < 0 ? i + n : i;
+}
+
 __device__ __forceinline__ void vis_position(const Geom& g, const double* __restrict__ uvw,
                                              const double* __restrict__ chan4, int64_t k,
                                              VisPos& p) {
-  int64_t row = k / g.nchan;
-  int ch = (int)(k - row * g.nchan);
+  const int64_t row = (uint32_t)k / (uint32_t)g.nchan;   // k < 2^31 (index entries hold a fold bit)
+  const int ch = (int)(k - row * g.nchan);
   double ut = uvw[3 * row], vt = uvw[3 * row + 1], wt = uvw[3 * row + 2];
   p.fold = g.do_w && wt < 0.0;
   if (p.fold) { ut = -ut; vt = -vt; wt = -wt; }
@@ -76,9 +87,8 @@ __device__ __forceinline__ void vis_position(const Geom& g, const double* __rest
   double cv = ceil(__dsub_rn(y, half));
   p.fu = __dsub_rn(cu, x);
   p.fv = __dsub_rn(cv, y);
-  int64_t iu = (int64_t)cu % g.nu, iv = (int64_t)cv % g.nv;
-  p.iu = iu < 0 ? iu + g.nu : iu;
-  p.iv = iv < 0 ? iv + g.nv : iv;
+  p.iu = wrap_cell(cu, g.nu);
+  p.iv = wrap_cell(cv, g.nv);
   p.bad = false;
   p.wlam = g.do_w ? __dmul_rn(wt, sc[3]) : 0.0;
   if (g.do_w) {
@@ -96,7 +106,7 @@ __device__ __forceinline__ void vis_position(const Geom& g, const double* __rest
 }
 
 __device__ __forceinline__ uint32_t bucket_key(const Geom& g, const VisPos& p) {
-  int tu = (int)(p.iu / g.tile), tv = (int)(p.iv / g.tile);
+  const int tu = (int)p.iu / g.tile, tv = (int)p.iv / g.tile;
   return (uint32_t)(((int64_t)tu * g.ntv + tv) * g.nw + p.c0);
 }
 
@@ -223,11 +233,43 @@ cudaError_t launch_scan(uint32_t* data, int64_t n, uint32_t* scratch, cudaStream
 // The record of visibility k at index position pos: meta (first cell inside its tile, first
 // plane), Horner coordinates of the first kernel piece, and e^{2 pi i w_k nshift}.
 // ---------------------------------------------------------------------------------------
+// cos and sin of 2 pi c for |c| <= 1 / 2 to within 2^-40 before the final rounding (one float in 10^4
+// differs from the rounded FP64 sincospi, next to a tie): Taylor polynomials
+// in double-float arithmetic after reduction to a quarter turn.  The FP64 sincospi took two thirds
+// of the FP64 instructions of a record, and GB300 issues those at 1/64 of the FP32 rate (expanding
+// 645 120 records: 92 -> 61 us; 7.6e6: 0.92 -> 0.55 ms, with the cells wrapped in 32 bits).
+__device__ __forceinline__ float2 cis_turn(double c) {
+  const float h = (float)c, l = (float)(c - (double)h);
+  const float q = rintf(4.0f * h);
+  // h - q / 4 is exact, and zero or at least ulp(h) > |l|
+  const dd r = fast_two_sum(__fmaf_rn(-0.25f, q, h), l);
+  const dd t = dd_mul(r, dd_make(6.28318548f, -1.74845553e-7f));
+  const dd x = dd_mul(t, t);   // at most (pi / 4)^2
+  // coefficients 1 / k! as float pairs; terms from x^4 on in float
+  float cf = __fmaf_rn(x.h, 2.0876757e-9f, -2.7557319e-7f);
+  cf = __fmaf_rn(x.h, cf, 2.4801587e-5f);
+  dd cp = dd_fma(x, dd_make(cf, 0.f), dd_make(-1.38888892e-3f, 3.3631094e-11f));
+  cp = dd_fma(x, cp, dd_make(4.16666679e-2f, -1.2417635e-9f));
+  cp = dd_fma(x, cp, dd_make(-0.5f, 0.f));
+  cp = dd_fma(x, cp, dd_make(1.f, 0.f));
+  float sf = __fmaf_rn(x.h, 1.6059044e-10f, -2.5052108e-8f);
+  sf = __fmaf_rn(x.h, sf, 2.7557319e-6f);
+  dd sp = dd_fma(x, dd_make(sf, 0.f), dd_make(-1.98412701e-4f, 2.7255968e-12f));
+  sp = dd_fma(x, sp, dd_make(8.33333377e-3f, -4.3461720e-10f));
+  sp = dd_fma(x, sp, dd_make(-0.16666667f, 4.9670538e-9f));
+  sp = dd_fma(x, sp, dd_make(1.f, 0.f));
+  sp = dd_mul(sp, t);
+  const int k = (int)q & 3;   // quarter turns
+  const float co = cp.h, si = sp.h;
+  return make_float2(k == 0 ? co : k == 1 ? -si : k == 2 ? -co : si,
+                     k == 0 ? si : k == 1 ? co : k == 2 ? -si : -co);
+}
+
 template <typename R>
 __device__ __forceinline__ void write_record(const Geom& g, const VisPos& p, uint32_t pos,
                                              uint32_t* __restrict__ meta, Z4<R>* __restrict__ z,
                                              typename C2<R>::T* __restrict__ ph) {
-  int du = (int)(p.iu % g.tile), dv = (int)(p.iv % g.tile);
+  const int du = (int)p.iu & (g.tile - 1), dv = (int)p.iv & (g.tile - 1);   // tiles of 16 or 32 cells
   meta[pos] = (uint32_t)du | ((uint32_t)dv << 8) | ((uint32_t)p.c0 << 16);
   // Horner coordinate of the first piece: z = 2 (f + alpha/2) - 1 (Sec. 4.2)
   Z4<R> zz;
@@ -240,10 +282,12 @@ __device__ __forceinline__ void write_record(const Geom& g, const VisPos& p, uin
     // exp(2 pi i w_k nshift): the part of the w-term carried by the shifted reference
     double cyc = p.wlam * g.nshift;
     cyc -= rint(cyc);
-    double sn, cs;
-    sincospi(2.0 * cyc, &sn, &cs);
     typename C2<R>::T v;
-    v.x = (R)cs; v.y = (R)sn;
+    if constexpr (sizeof(R) == 4) {
+      v = cis_turn(cyc);
+    } else {
+      sincospi(2.0 * cyc, &v.y, &v.x);
+    }
     ph[pos] = v;
   }
 }
