@@ -238,7 +238,10 @@ DF64_BUTTERFLY = {2: 44, 3: 160, 4: 176, 5: 464, 7: 870, 8: 600, 11: 2050}
 
 def df64_radices(n):
     """Radix plan of a double-float line transform (8s and 4s for the power of two, a single 2
-    only for n = 2 x odd, then 5, 3, 7, 11) -- the plan the library uses."""
+    only for n = 2 x odd, then 5, 3, 7, 11) -- the plan of the library's line kernels.  The
+    accounting counts this transform for every side: the kernels on pairs of lines take other
+    radices, up to 12, with fewer operations (3456 points as 4 x 864, radices 8 6 6 3: 430 per
+    element where this count has 460)."""
     m, p2 = n, 0
     while m % 2 == 0:
         m //= 2
@@ -300,9 +303,17 @@ def df64_line_ops(n):
     return (n // S) * (DF64_BUTTERFLY[S] + 38 * (S - 1)) + S * df64_part_ops(n // S)
 
 
+def df64_fft_kernel(n):
+    """The kernel a double-float line of n points runs on: pairs of lines, except between 3072 and
+    4096 points with a factor 11 or 35 (one line per CTA or cluster)."""
+    if 3072 < n < 4096 and (n % 11 == 0 or n % 35 == 0):
+        return "k_fft_lines_cluster" if df64_line_split(n) > 1 else "k_fft_lines"
+    return "k_fft_pairs"
+
+
 # DRAM bytes the double-float FFT moved per algorithmic byte (one 16-byte read and one 16-byte
-# write per cell and pass), measured by ncu on full 3456^2 transforms (lines as two halves on
-# clusters of 2 CTAs): 30.86 of 32 B per cell and pass (profiles/k_fft_lines_cluster_df64_3456.md);
+# write per cell and pass), measured by ncu on full 3456^2 transforms (pairs of lines on clusters
+# of 4 CTAs): 30.86 of 32 B per cell and pass (profiles/k_fft_pairs_df64_3456.md);
 # the rest stays in L2 when the kernel ends
 DF64_DRAM_PER_ALGORITHMIC_BYTE = 30.86 / 32.0
 
@@ -851,7 +862,7 @@ def main():
         peak = 152 * 128 * 2.07e9   # SMs x FP32 lanes x max SM clock, one instruction per lane
         ach = ops / (stage_ms[dom] * 1e-3)
         abytes = nw * df64_fft_bytes(obs.npix_x, obs.npix_y, nu, nv, dir_d)
-        kname = "k_fft_lines_cluster" if df64_line_split(nu) > 1 else "k_fft_lines"
+        kname = df64_fft_kernel(nu)
         roof = {"bound": "alu", "kernel": f"{kname} (double-float plane FFT, row + column pass)",
                 "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s", "frac": ach / peak,
                 "traffic": DF64_DRAM_PER_ALGORITHMIC_BYTE * abytes,

@@ -93,17 +93,15 @@ typedef struct wg_options {
                               plane-owner warps (deterministic), 3 = row-band owner warps
                               (WG_F32, alpha <= 8, 32-cell tiles: each warp owns 4 rows of the
                               tile in every plane; deterministic; other plans fall back to 1);
-                              WG_F64 plans with the double-float FFT always use plane-owner
-                              warps (their planes are double-float pairs, written by that
-                              kernel only) */
+                              WG_F64 plans with the double-float FFT always keep the sums of
+                              their double-float pairs in registers (each lane owns a cell in
+                              8 planes; deterministic) */
   int fft_impl;            /* plane FFTs: 0 = automatic (WG_F32: cuFFT C2C; WG_F64: the
                               cheaper of 2 and 3 whose predicted error fits epsilon),
                               1 = cuFFT 2-D, 2 = the library's double-float FFT (WG_F64 only,
                               grid sides up to 6400 with prime factors 2, 3, 5, 7, 11, and
-                              sides up to 25600 that are 2 or 4 times such a side (each line
-                              then runs on a thread-block cluster of 2 or 4 CTAs, as do lines
-                              above 2048 points whose half needs only the radices 8, 4, 5,
-                              3); its ~5e-15 rounding is amplified by the
+                              sides up to 25600 that are 2 or 4 times such a side; two lines
+                              at a time, above 2048 points on thread-block clusters); its ~5e-15 rounding is amplified by the
                               1 / psi correction, so the planner may raise sigma for it; the
                               uv planes are then kept as double-float pairs and (de)gridded in
                               pair arithmetic),

@@ -8,17 +8,16 @@
 // transform is ~5e-15 relative (vs ~2e-16 for FP64); the planner accounts for it (its
 // rounding is amplified by the 1 / psi correction, see plane_rounding / rounding_gain).
 //
-// Algorithm: each 1-D transform is a mixed-radix (8 and 4 for the power of two, 5, 3, the
-// symmetric 7 and 11, 2 only for n = 2 * odd) Stockham autosort FFT run by one CTA per
-// line with about n / 8 threads (one radix-8 butterfly each) over two n-element shared-memory
-// buffers (ping-pong); up to n = 3584 two CTAs share an SM.  A pass that reads float pairs in
-// full runs persistent CTAs instead, which copy their next line into the free buffer (cp.async)
-// while storing the current one.  Lines above 6400 points, and lines above 2048 whose half needs
-// only the radices 8, 4, 5, 3, run on a thread-block cluster of 2 or 4 CTAs
-// (k_fft_lines_cluster).  The 2-D plane transform is a pass over rows (contiguous) and a
-// pass over columns.  On the image side planes are complex128 (the pass that reads them splits
-// doubles into float pairs on load, the pass that writes them joins the pairs back); on the uv
-// side they are complex128 or, for the (de)gridding kernels in pair arithmetic, float pairs.
+// Algorithm: each 1-D transform is a mixed-radix Stockham autosort FFT.  Nearly every side runs on
+// PAIRS of lines packed into the FP32 x2 instructions (k_fft_pairs: radices up to 12, one
+// shared-memory buffer, one CTA for up to two thousand points and clusters of 2, 4 or 8 CTAs above;
+// see there).  The kernels of one line per CTA (k_fft_lines: radices 8 and 4 for the power of two, 5, 3,
+// the symmetric 7 and 11, 2 only for n = 2 * odd; about n / 8 threads, two ping-pong buffers;
+// k_fft_lines_cluster: split lines on 2 or 4 CTAs) remain for the sides where they are as fast or
+// faster: see pair_plan and make_side.  The 2-D plane transform is a pass over rows (contiguous)
+// and a pass over columns.  On the image side planes are complex128 (converted around the pairs'
+// passes; the line kernels split and join on load and store); on the uv side they are complex128
+// or, for the (de)gridding kernels in pair arithmetic, float pairs.
 // Transforms are unnormalised, forward = e^{-2 pi i}, like cuFFT's.
 #include <cooperative_groups.h>
 
@@ -537,6 +536,7 @@ k_fft_lines_cluster(const __grid_constant__ FftLine L, void* __restrict__ data, 
 //  * a split line's radix-S decimation-in-frequency step is done where the points are loaded:
 //    CTA h takes the j-range [h n / S, (h + 1) n / S), forms all S outputs of each butterfly and
 //    writes output r into CTA r's buffer through distributed shared memory;
+//  * where one pair leaves lanes of its warps idle, several share a CTA (kPack, see pair_pack);
 //  * radices up to 12 (10, 6 and 12 by coprime factors, no inner twiddles): 1728 = 12 12 12 in
 //    three stages instead of 8 8 3 3 3 in five;
 //  * twiddles are stored per stage in the order the threads read them, each float twice.

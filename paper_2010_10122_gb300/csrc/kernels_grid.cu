@@ -13,11 +13,13 @@
 //  * grid: one CTA per (tile, sub-batch of planes) owns the T x T cells of those planes and
 //    accumulates contributions of visibilities from its own tile and the three tiles whose
 //    footprints reach into it, then writes every cell exactly once (no global atomics, no
-//    separate zeroing pass; empty tiles write zeros).  Two accumulation schemes: shared-memory
-//    atomics (cheap in FP32) or warps that each own whole planes (no atomics, deterministic;
-//    used for FP64, where shared-memory double atomics occupy the FP64 pipe);
-//  * FP64 plans with the double-float FFT keep the planes as double-float pairs and run the
-//    degridding and plane-owner gridding in pair arithmetic on the FP32 pipes (df64.cuh).
+//    separate zeroing pass; empty tiles write zeros).  Accumulation schemes: FP32 on the tensor
+//    cores, products of bf16 slices that lose nothing (k_grid_mma, the automatic choice with 32-cell
+//    tiles), or shared-memory atomics (k_grid_atomic); FP64 planes by warps that each own whole
+//    planes (k_grid_owner: shared-memory double atomics occupy the FP64 pipe);
+//  * FP64 plans with the double-float FFT keep the planes as double-float pairs: k_degrid_dd, and
+//    k_grid_cells_dd with the cells' sums in registers, in pair arithmetic on the FP32 pipes
+//    (df64.cuh).
 #include <cmath>
 #include <type_traits>
 
