@@ -88,7 +88,8 @@ typedef struct wg_options {
   double force_sigma;      /* >0: only consider this oversampling factor (tests) */
   int tile;                /* uv tile side in cells (16 or 32; 0 = automatic) */
   int grid_variant;        /* gridding accumulation: 0 = automatic (WG_F32: tensor cores with
-                              32-cell tiles, deterministic, else shared-memory atomics; WG_F64:
+                              32-cell tiles and a rounding_gain up to 40, deterministic,
+                              else shared-memory atomics; WG_F64:
                               plane-owner warps), 1 = shared-memory atomics, 2 =
                               plane-owner warps (deterministic), 3 = row-band owner warps
                               (WG_F32, alpha <= 8, 32-cell tiles: each warp owns 4 rows of the

@@ -1799,6 +1799,14 @@ static cudaError_t grid_band(const Geom& g, const Coef<float>& coef, const Index
 // tensor cores, which need 32-cell tiles, else the shared-memory atomics (on the 1e8-visibility
 // workload the row-band owners measured 289 ms, the atomics 171 ms, the tensor cores half of that)
 constexpr int kVariantMma = 4;   // tensor cores: automatic choice only
+// ... and only up to this rounding gain of the plan.  The two kernels round differently (atomics
+// each product and sum, the tensor cores sums only), and the image correction amplifies the planes'
+// rounding by the gain: their images differ by about 2e-7 x gain of the norm (4.2e-6 at a gain of 22,
+// 4.4e-6 at 38, 3.8e-5 at 294) and by up to 2.6e-5 x gain in a pixel at the edge.  Plans of a large
+// gain (coarse accuracies, low oversampling, few visibilities) keep the atomics, so that an image
+// stays within 1e-5 of what it was; the transform is most of their time (1876^2, 57 000 visibilities,
+// gain 294: a forward and backward step takes 3.79 ms by atomics, 3.63 by the tensor cores)
+constexpr double kMmaMaxGain = 40.0;
 template <typename R>
 static int grid_variant_of(const Geom& g) {
   // double-float planes are written by the plane-owner kernel only
@@ -1806,7 +1814,7 @@ static int grid_variant_of(const Geom& g) {
   const bool band_ok = sizeof(R) == 4 && g.alpha <= 8 && g.tile == kBandTile;
   if (g.grid_variant == 3) return band_ok ? 3 : 1;
   if (g.grid_variant != 0) return g.grid_variant;
-  return sizeof(R) == 8 ? 2 : (g.tile == kMmaTile ? kVariantMma : 1);
+  return sizeof(R) == 8 ? 2 : (g.tile == kMmaTile && g.gain <= kMmaMaxGain ? kVariantMma : 1);
 }
 
 template <typename R, int G>

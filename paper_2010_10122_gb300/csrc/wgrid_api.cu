@@ -458,6 +458,7 @@ int wg_plan_create(const double* uvw, const double* freq, int64_t nrows, int64_t
   g.w0 = pp.w0; g.dw = pp.dw; g.nshift = pp.nshift;
   g.w0_dw = pp.w0 / pp.dw;
   g.grid_variant = p->opt.grid_variant;
+  g.gain = pp.gain;
   if (g.grid_variant < 0 || g.grid_variant > 3) return set_error(WG_ERR_ARG, "grid_variant must be 0, 1, 2 or 3");
   fill_coefs(p.get());
 

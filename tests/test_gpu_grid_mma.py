@@ -48,3 +48,14 @@ def test_tensor_core_gridding(wg, oracle_lib, nrows, nchan, nx, ny, alpha, eps, 
         fine = wg.Plan(*geom, 1e-11, "f64", mask=mask, do_wstacking=do_w)
         ref = fine.grid(vis.to(torch.complex128), wgt=None if w32 is None else w32.double()).cpu().numpy()
     assert oracle_lib.rel_l2(got.cpu().numpy(), ref) <= eps
+
+
+def test_large_rounding_gain_takes_the_atomics(wg, oracle_lib):
+    obs = S.random_uvw_observation(500, 2, 128, 96, 20.0, seed=5)
+    d = S.complex_normal((500, 2), seed=4)
+    plan = wg.Plan(obs.uvw, obs.freq, 128, 96, obs.pixsize_x, obs.pixsize_y, 1e-3, "f32", force_alpha=7,
+                   force_sigma=1.15)
+    assert plan.info["tile"] == 32 and plan.info["rounding_gain"] > 40
+    got = plan.grid(torch.from_numpy(d.astype(np.complex64)).cuda())
+    ref = oracle_lib.grid(obs.uvw, obs.freq, d, 128, 96, obs.pixsize_x, obs.pixsize_y)
+    assert oracle_lib.rel_l2(got.cpu().numpy(), ref) <= 1e-3
