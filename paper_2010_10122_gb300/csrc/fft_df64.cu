@@ -919,29 +919,12 @@ static bool pair_plan(int N, PairLine* L) {
   return false;
 }
 
-// e^{-2 pi i t / len} as a twiddle entry (each float twice)
-static void pair_entry(int64_t t, int64_t len, float4* e) {
-  // exact octant reduction, then sine and cosine of at most pi / 4 in double (1e-16, against the
-  // pairs' 2e-15)
-  t %= len;
-  const int64_t o = 8 * t / len;                 // octant 0 .. 7
-  const int64_t num = (o & 1) ? (o + 1) * len - 8 * t : 8 * t - o * len;   // distance to the nearer axis or diagonal, of 8 len
-  const double a = 0.78539816339744830962 * ((double)num / (double)len);
-  double c = std::cos(a), s = std::sin(a), cr, sr;
-  switch (o) {
-    case 0: cr = c; sr = s; break;
-    case 1: cr = s; sr = c; break;
-    case 2: cr = -s; sr = c; break;
-    case 3: cr = -c; sr = s; break;
-    case 4: cr = -c; sr = -s; break;
-    case 5: cr = -s; sr = -c; break;
-    case 6: cr = s; sr = -c; break;
-    default: cr = c; sr = -s; break;
-  }
-  sr = -sr;
-  const float ch = (float)cr, cl = (float)(cr - (double)ch), sh = (float)sr, sl = (float)(sr - (double)sh);
-  e[0] = make_float4(ch, ch, cl, cl);
-  e[1] = make_float4(sh, sh, sl, sl);
+// a root of unity as a twiddle entry (each float twice)
+static void pair_entry(const UnitRoots& roots, int64_t t, float4* e) {
+  float w[4];
+  roots.pair(t, w);
+  e[0] = make_float4(w[0], w[0], w[1], w[1]);
+  e[1] = make_float4(w[2], w[2], w[3], w[3]);
 }
 
 static cudaError_t make_pairs(PairLine* L, float4** tw) {
@@ -955,18 +938,21 @@ static cudaError_t make_pairs(PairLine* L, float4** tw) {
   const int own = entries;
   entries += (L->S - 1) * L->n;
   std::vector<float4> h(2 * (size_t)std::max(1, entries));
+  const int64_t N = (int64_t)L->S * L->n;
+  const UnitRoots roots(N);
   Ns = 1;
   for (int s = 0; s < L->nst; ++s) {
     const int R = L->radix[s];
     if (Ns > 1)
       for (int k = 1; k < R; ++k)
         for (int jm = 0; jm < Ns; ++jm)
-          pair_entry((int64_t)jm * k, (int64_t)Ns * R, &h[2 * (size_t)(L->twofs[s] + (k - 1) * Ns + jm)]);
+          pair_entry(roots, (int64_t)jm * k * (N / ((int64_t)Ns * R)),
+                     &h[2 * (size_t)(L->twofs[s] + (k - 1) * Ns + jm)]);
     Ns *= R;
   }
   for (int r = 1; r < L->S; ++r)
     for (int j = 0; j < L->n; ++j)
-      pair_entry((int64_t)j * r, (int64_t)L->S * L->n, &h[2 * (size_t)(own + (r - 1) * L->n + j)]);
+      pair_entry(roots, (int64_t)j * r, &h[2 * (size_t)(own + (r - 1) * L->n + j)]);
   cudaError_t e = cudaMalloc((void**)tw, sizeof(float4) * h.size());
   if (e != cudaSuccess) return e;
   e = cudaMemcpy(*tw, h.data(), sizeof(float4) * h.size(), cudaMemcpyHostToDevice);

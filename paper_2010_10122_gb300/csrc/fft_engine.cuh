@@ -76,43 +76,79 @@ __device__ __forceinline__ d2 s_sub(d2 a, d2 b) {   // a - b, the two-sum writte
 }
 
 // ---- compile-time constants --------------------------------------------------------------
-// cos(2 pi k / N), sin(2 pi k / N) in double, from the Taylor series of the reduced angle
+// cos(2 pi k / N), sin(2 pi k / N) from the Taylor series of the reduced angle, in double-double
+// arithmetic: a pair of floats resolves 2^-50 of a value, and of a double's last bit (2^-53) it would
+// keep the error (in double, 13 of the 74 constants of the radices 3 to 11 were not the nearest
+// pair, among them those of the radices 7 and 9)
 namespace trig {
-constexpr double kPi = 3.14159265358979323846264338327950288;
-__host__ __device__ constexpr double sin_small(double x) {   // |x| <= pi / 4
-  double t = x, s = x;
-  for (int i = 1; i <= 12; ++i) { t *= -x * x / ((2.0 * i) * (2.0 * i + 1.0)); s += t; }
+struct wide { double h, l; };   // h + l
+__host__ __device__ constexpr wide sum(double a, double b) {   // exact (Knuth)
+  const double s = a + b, bb = s - a;
+  return wide{s, (a - (s - bb)) + (b - bb)};
+}
+__host__ __device__ constexpr wide prod(double a, double b) {   // exact (Dekker)
+  const double ca = 134217729.0 * a, cb = 134217729.0 * b;
+  const double ah = ca - (ca - a), al = a - ah, bh = cb - (cb - b), bl = b - bh;
+  const double p = a * b;
+  return wide{p, ((ah * bh - p) + ah * bl + al * bh) + al * bl};
+}
+__host__ __device__ constexpr wide neg(wide a) { return wide{-a.h, -a.l}; }
+__host__ __device__ constexpr wide add(wide a, wide b) {
+  const wide s = sum(a.h, b.h);
+  return sum(s.h, s.l + (a.l + b.l));
+}
+__host__ __device__ constexpr wide mul(wide a, wide b) {
+  const wide p = prod(a.h, b.h);
+  return sum(p.h, p.l + (a.h * b.l + a.l * b.h));
+}
+__host__ __device__ constexpr wide div(wide a, double n) {
+  const double q = a.h / n;
+  const wide p = prod(q, n);
+  return sum(q, (((a.h - p.h) - p.l) + a.l) / n);
+}
+__host__ __device__ constexpr wide angle(int k, int N) {   // 2 pi k / N
+  return div(mul(wide{2.0 * k, 0.0}, wide{3.14159265358979311600e+00, 1.22464679914735317636e-16}), N);
+}
+// |x| <= pi / 4
+__host__ __device__ constexpr wide sin_small(wide x) {
+  const wide x2 = mul(x, x);
+  wide t = x, s = x;
+  for (int i = 1; i <= 14; ++i) { t = neg(div(mul(t, x2), (2.0 * i) * (2.0 * i + 1.0))); s = add(s, t); }
   return s;
 }
-__host__ __device__ constexpr double cos_small(double x) {
-  double t = 1.0, s = 1.0;
-  for (int i = 1; i <= 12; ++i) { t *= -x * x / ((2.0 * i - 1.0) * (2.0 * i)); s += t; }
+__host__ __device__ constexpr wide cos_small(wide x) {
+  const wide x2 = mul(x, x);
+  wide t{1.0, 0.0}, s = t;
+  for (int i = 1; i <= 14; ++i) { t = neg(div(mul(t, x2), (2.0 * i - 1.0) * (2.0 * i))); s = add(s, t); }
   return s;
 }
 // octant reduction in exact integer arithmetic: angle k / N of a turn
-__host__ __device__ constexpr double cos2pi(int k, int N);
-__host__ __device__ constexpr double sin2pi(int k, int N) {
+__host__ __device__ constexpr wide cos2pi(int k, int N);
+__host__ __device__ constexpr wide sin2pi(int k, int N) {
   k %= N; if (k < 0) k += N;
-  if (2 * k > N) return -sin2pi(N - k, N);
+  if (2 * k > N) return neg(sin2pi(N - k, N));
   if (4 * k > N) return sin2pi(N - 2 * k, 2 * N);     // sin(pi - x)
   if (8 * k > N) return cos2pi(N - 4 * k, 4 * N);     // sin(x) = cos(pi/2 - x)
-  return sin_small(2.0 * kPi * k / N);
+  return sin_small(angle(k, N));
 }
-__host__ __device__ constexpr double cos2pi(int k, int N) {
+__host__ __device__ constexpr wide cos2pi(int k, int N) {
   k %= N; if (k < 0) k += N;
   if (2 * k > N) return cos2pi(N - k, N);
-  if (4 * k > N) return -cos2pi(N - 2 * k, 2 * N);
+  if (4 * k > N) return neg(cos2pi(N - 2 * k, 2 * N));
   if (8 * k > N) return sin2pi(N - 4 * k, 4 * N);
-  return cos_small(2.0 * kPi * k / N);
+  return cos_small(angle(k, N));
 }
 }  // namespace trig
 
-struct Konst { double v; };   // a real constant, rounded to the scalar type where it is used
+struct Konst {   // a real constant, the nearest pair of floats
+  float h, l;
+  __host__ __device__ constexpr explicit Konst(trig::wide v)
+      : h((float)v.h), l((float)((v.h - (double)(float)v.h) + v.l)) {}
+};
 
 // a * k: p - n with p the rounded product of the high parts and n minus everything below it
 __device__ __forceinline__ d2 s_mulk(d2 a, const Konst k) {
-  const float kh = (float)k.v, kl = (float)(k.v - (double)kh);
-  const f2 H = f2_dup(kh), nH = f2_dup(-kh), nL = f2_dup(-kl);
+  const f2 H = f2_dup(k.h), nH = f2_dup(-k.h), nL = f2_dup(-k.l);
   const f2 p = s_mul(a.h, H);
   f2 n = s_fma(a.h, nH, p);
   n = s_fma(a.h, nL, n);
@@ -124,8 +160,7 @@ __device__ __forceinline__ d2 s_mulk(d2 a, const Konst k) {
 }
 // a * k + c
 __device__ __forceinline__ d2 s_fmak(d2 a, const Konst k, d2 c) {
-  const float kh = (float)k.v, kl = (float)(k.v - (double)kh);
-  const f2 H = f2_dup(kh), nH = f2_dup(-kh), nL = f2_dup(-kl);
+  const f2 H = f2_dup(k.h), nH = f2_dup(-k.h), nL = f2_dup(-k.l);
   const f2 p = s_mul(a.h, H);
   f2 n = s_fma(a.h, nH, p);
   n = s_fma(a.h, nL, n);
@@ -187,11 +222,9 @@ __device__ __forceinline__ Cx<d2> cx_mul(const Cx<d2>& a, const Tw<d2>& w) {
 // a e^{-2 pi i k / N} for compile-time k, N
 template <int N, int K>
 __device__ __forceinline__ Cx<d2> cx_root(const Cx<d2>& a) {
-  constexpr double c = trig::cos2pi(K, N), s = -trig::sin2pi(K, N);
-  constexpr float ch = (float)c, cl = (float)(c - (double)(float)c);
-  constexpr float sh = (float)s, sl = (float)(s - (double)(float)s);
-  return Cx<d2>{d2_dot(a.r, f2_dup(ch), f2_dup(-ch), f2_dup(cl), a.i, f2_dup(-sh), f2_dup(sh), f2_dup(-sl)),
-                d2_dot(a.r, f2_dup(sh), f2_dup(-sh), f2_dup(sl), a.i, f2_dup(ch), f2_dup(-ch), f2_dup(cl))};
+  constexpr Konst c{trig::cos2pi(K, N)}, s{trig::neg(trig::sin2pi(K, N))};
+  return Cx<d2>{d2_dot(a.r, f2_dup(c.h), f2_dup(-c.h), f2_dup(c.l), a.i, f2_dup(-s.h), f2_dup(s.h), f2_dup(-s.l)),
+                d2_dot(a.r, f2_dup(s.h), f2_dup(-s.h), f2_dup(s.l), a.i, f2_dup(c.h), f2_dup(-c.h), f2_dup(c.l))};
 }
 
 // ---- DFTs of R values in registers (in place, natural order in and out) -------------------

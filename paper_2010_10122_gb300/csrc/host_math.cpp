@@ -262,6 +262,48 @@ const KernelMath& kernel_math(int alpha, double beta, double mu) {
   return *it->second;
 }
 
+UnitRoots::UnitRoots(int64_t n) : n_(n), step_(1) {
+  while (step_ * step_ < n) step_ *= 2;
+  const long double unit = 6.283185307179586476925286766559L / (8.0L * (long double)n);   // at most n units: pi / 4
+  auto root = [&](int64_t k) {
+    const long double c = cosl(unit * (long double)k), s = sinl(unit * (long double)k);
+    Root r;
+    r.ch = (double)c; r.cl = (double)(c - (long double)r.ch);
+    r.sh = (double)s; r.sl = (double)(s - (long double)r.sh);
+    return r;
+  };
+  for (int64_t a = 0; a * step_ <= n; ++a) coarse_.push_back(root(a * step_));
+  for (int64_t b = 0; b < step_; ++b) fine_.push_back(root(b));
+}
+
+// a b + sgn c d as hi + lo, the pair of floats nearest to it in out.  volatile: the rounded products
+// must not be contracted into the sum below, their errors are added apart.
+static void pair_of_products(double ah, double al, double bh, double bl, double sgn, double ch, double cl,
+                             double dh, double dl, float* out) {
+  const volatile double p = ah * bh, q = sgn * ch * dh;
+  const double pe = std::fma(ah, bh, -p), qe = std::fma(sgn * ch, dh, -q);
+  const double s = p + q, v = s - p, e = (p - (s - v)) + (q - v);
+  const double lo = e + ((pe + qe) + ((ah * bl + al * bh) + sgn * (ch * dl + cl * dh)));
+  const double r = s + lo;
+  out[0] = (float)r;
+  out[1] = (float)((r - (double)out[0]) + (lo - (r - s)));
+}
+
+void UnitRoots::pair(int64_t t, float* out) const {
+  t %= n_;
+  const int64_t o = 8 * t / n_;   // octant 0 .. 7; k of 8 n units from its nearer axis or diagonal
+  const int64_t k = (o & 1) ? (o + 1) * n_ - 8 * t : 8 * t - o * n_;
+  const Root &A = coarse_[(size_t)(k / step_)], &B = fine_[(size_t)(k % step_)];
+  float c[2], s[2];
+  pair_of_products(A.ch, A.cl, B.ch, B.cl, -1.0, A.sh, A.sl, B.sh, B.sl, c);
+  pair_of_products(A.sh, A.sl, B.ch, B.cl, 1.0, A.ch, A.cl, B.sh, B.sl, s);
+  const bool swap = o == 1 || o == 2 || o == 5 || o == 6;
+  const float *x = swap ? s : c, *y = swap ? c : s;
+  const float sx = o >= 2 && o <= 5 ? -1.f : 1.f, sy = o >= 4 ? 1.f : -1.f;
+  out[0] = sx * x[0]; out[1] = sx * x[1];
+  out[2] = sy * y[0]; out[3] = sy * y[1];
+}
+
 double psi_cheb_eval(const std::vector<double>& c, double k) {
   double y = 8.0 * k * k - 1.0;
   double b1 = 0.0, b2 = 0.0;

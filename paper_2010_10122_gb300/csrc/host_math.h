@@ -103,6 +103,21 @@ bool df64_line_plan(int64_t n, Df64LinePlan* plan);
 int df64_line_split(int64_t n);
 bool df64_side_ok(int64_t n);
 
+// Roots of unity e^{-2 pi i t / n} as pairs of floats (re hi, re lo, im hi, im lo), each the nearest pair
+// to its value: tables of about sqrt(n) angles each, in twice a double's precision, and one complex
+// product per root.  (The double functions alone left one pair in eleven off by a last bit; an
+// extended-precision sine for each root takes microseconds where it is computed in software.)
+class UnitRoots {
+ public:
+  explicit UnitRoots(int64_t n);
+  void pair(int64_t t, float* out) const;
+
+ private:
+  struct Root { double ch, cl, sh, sl; };   // cos and sin, each hi + lo
+  int64_t n_, step_;
+  std::vector<Root> coarse_, fine_;         // angles a step_ / (8 n) and b / (8 n) of a turn
+};
+
 // Gain of plane rounding into the result.  A plane value perturbed by a relative (normwise)
 // rounding delta reaches the degridded visibilities / gridded image through the kernel
 // footprint and the correction 1 / (n psi_u psi_v psi_w) of Eqs. R1 / Rad1; for an image with
