@@ -961,30 +961,65 @@ static cudaError_t make_pairs(PairLine* L, float4** tw) {
   return e;
 }
 
+// Launch configuration of `blocks` CTAs (a multiple of L.S) of the pair kernel
+struct PairLaunch {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  PairLaunch(const PairLine& L, unsigned blocks, cudaStream_t s) {
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3((unsigned)L.T);
+    cfg.dynamicSmemBytes = 2 * sizeof(float4) * (size_t)((L.n + 7) & ~7) * L.P;
+    cfg.stream = s;
+    std::memset(attr, 0, sizeof(attr));
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)L.S;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = L.S > 1 ? 1 : 0;
+  }
+  PairLaunch(const PairLaunch&) = delete;   // cfg points into the object
+};
+
+static cudaError_t pair_smem_attributes() {
+  const int bytes = (int)(2 * sizeof(float4) * kPairMaxPart);
+  cudaError_t e = cudaSuccess;
+#define WG_SMEM_ATTR(...)                                                                        \
+  if (e == cudaSuccess)                                                                          \
+    e = cudaFuncSetAttribute(k_fft_pairs<__VA_ARGS__>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)
+  WG_SMEM_ATTR(9, 256, false);  WG_SMEM_ATTR(9, 256, true);
+  WG_SMEM_ATTR(12, 192, false); WG_SMEM_ATTR(12, 192, true);
+#undef WG_SMEM_ATTR
+  return e;
+}
+
+// whether the GPU, as the process sees it, can place a cluster of the line's CTAs at all (a share of
+// it with few SMs to a cluster's domain may not): where it cannot, the line goes to the kernels of
+// one line per CTA, which do without clusters when they must
+static bool pair_cluster_fits(const PairLine& L) {
+  if (L.S == 1) return true;
+  const PairLaunch l(L, (unsigned)L.S, 0);
+  int clusters = 0;
+  const cudaError_t e = L.cls == 9
+      ? cudaOccupancyMaxActiveClusters(&clusters, k_fft_pairs<9, 256, false>, &l.cfg)
+      : cudaOccupancyMaxActiveClusters(&clusters, k_fft_pairs<12, 192, false>, &l.cfg);
+  if (e == cudaSuccess) return clusters > 0;
+  cudaGetLastError();
+  return false;
+}
+
 static cudaError_t launch_pairs(const PairLine& L, double2* data, int64_t batch, int64_t plane,
                                 int lines, int64_t line_stride, int64_t elem_stride, int fwd,
                                 int split, int skip, int lhalf, int shalf, cudaStream_t s) {
   if (lines == 0 || batch == 0) return cudaSuccess;
   const int64_t blocks = batch * (((lines + 1) / 2 + L.P - 1) / L.P) * L.S;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg;
-  std::memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)blocks);
-  cfg.blockDim = dim3((unsigned)L.T);
-  cfg.dynamicSmemBytes = 2 * sizeof(float4) * (size_t)((L.n + 7) & ~7) * L.P;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  std::memset(attr, 0, sizeof(attr));
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)L.S;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = L.S > 1 ? 1 : 0;
+  const PairLaunch l(L, (unsigned)blocks, s);
   float4* d = reinterpret_cast<float4*>(data);
   const int inv = fwd ? 0 : 1;
 #define WG_PAIRS(C, TM, P)                                                                       \
-  cudaLaunchKernelEx(&cfg, k_fft_pairs<C, TM, P>, L, d, plane, lines, line_stride, elem_stride, inv, \
+  cudaLaunchKernelEx(&l.cfg, k_fft_pairs<C, TM, P>, L, d, plane, lines, line_stride, elem_stride, inv, \
                      split, skip, lhalf, shalf)
   if (L.P > 1) return L.cls == 9 ? WG_PAIRS(9, 256, true) : WG_PAIRS(12, 192, true);
   return L.cls == 9 ? WG_PAIRS(9, 256, false) : WG_PAIRS(12, 192, false);
@@ -1049,7 +1084,7 @@ static cudaError_t make_line(int nline, FftLine* L, float4** tw) {
 }
 
 static cudaError_t make_side(int n, SideFft* f) {
-  f->pairs = pair_plan(n, &f->pl);
+  f->pairs = pair_plan(n, &f->pl) && pair_cluster_fits(f->pl);
   if (!f->pairs) return make_line(n, &f->fl, &f->tw);
   // sides of the radices 2 and 5 only, which pairs take in four stages with idle lanes: forward
   // and inverse at the pairs' speed against the lines', on square sides with pruning: 640 0.92 /
@@ -1066,7 +1101,8 @@ cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
   if (!df64_fft_supported(nu, nv)) return cudaErrorInvalidValue;
   Df64Fft* f = new Df64Fft();
   f->nu = (int)nu; f->nv = (int)nv;
-  cudaError_t e = make_side((int)nu, &f->u);
+  cudaError_t e = pair_smem_attributes();
+  if (e == cudaSuccess) e = make_side((int)nu, &f->u);
   if (e == cudaSuccess) e = make_side((int)nv, &f->v);
   const int smax = (int)(2 * kMaxSide * sizeof(float4));
 #define WG_SMEM_ATTR(K, BYTES)                                                                   \
@@ -1081,9 +1117,6 @@ cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
     WG_SMEM_ATTR((k_fft_lines_cluster<448, 2, false>), smax); WG_SMEM_ATTR((k_fft_lines_cluster<448, 2, true>), smax);
     WG_SMEM_ATTR((k_fft_lines_cluster<832, 1, false>), smax); WG_SMEM_ATTR((k_fft_lines_cluster<832, 1, true>), smax);
   }
-  const int spair = (int)(2 * sizeof(float4) * kPairMaxPart);
-  WG_SMEM_ATTR((k_fft_pairs<9, 256, false>), spair);  WG_SMEM_ATTR((k_fft_pairs<9, 256, true>), spair);
-  WG_SMEM_ATTR((k_fft_pairs<12, 192, false>), spair); WG_SMEM_ATTR((k_fft_pairs<12, 192, true>), spair);
 #undef WG_SMEM_ATTR
   if (e != cudaSuccess) {
     df64_fft_destroy(f);
