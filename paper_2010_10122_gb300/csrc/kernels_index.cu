@@ -233,11 +233,18 @@ cudaError_t launch_scan(uint32_t* data, int64_t n, uint32_t* scratch, cudaStream
 // The record of visibility k at index position pos: meta (first cell inside its tile, first
 // plane), Horner coordinates of the first kernel piece, and e^{2 pi i w_k nshift}.
 // ---------------------------------------------------------------------------------------
-// cos and sin of 2 pi c for |c| <= 1 / 2 to within 2^-40 before the final rounding (one float in 10^4
-// differs from the rounded FP64 sincospi, next to a tie): Taylor polynomials
-// in double-float arithmetic after reduction to a quarter turn.  The FP64 sincospi took two thirds
-// of the FP64 instructions of a record, and GB300 issues those at 1/64 of the FP32 rate (expanding
-// 645 120 records: 92 -> 61 us; 7.6e6: 0.92 -> 0.55 ms, with the cells wrapped in 32 bits).
+// cos and sin of 2 pi c for |c| <= 1 / 2, both the FP64 sincospi's rounded to float.  Taylor polynomials
+// in double-float arithmetic after reduction to a quarter turn, off by less than kCisError (the reduced
+// angle and the last steps 2^-46 each, the cut series and its float coefficients 2^-45); where a value
+// that far from the pair would round to another float (one float in 10^5, next to a tie, or a value near
+// zero), the FP64 functions decide.  They took two thirds of the FP64 instructions of a record, and GB300
+// issues those at 1/64 of the FP32 rate.
+constexpr float kCisError = 1.1368684e-13f;   // 2^-43
+__device__ __noinline__ float2 cis_turn_f64(double c) {
+  double s, k;
+  sincospi(2.0 * c, &s, &k);
+  return make_float2((float)k, (float)s);
+}
 __device__ __forceinline__ float2 cis_turn(double c) {
   const float h = (float)c, l = (float)(c - (double)h);
   const float q = rintf(4.0f * h);
@@ -245,20 +252,26 @@ __device__ __forceinline__ float2 cis_turn(double c) {
   const dd r = fast_two_sum(__fmaf_rn(-0.25f, q, h), l);
   const dd t = dd_mul(r, dd_make(6.28318548f, -1.74845553e-7f));
   const dd x = dd_mul(t, t);   // at most (pi / 4)^2
-  // coefficients 1 / k! as float pairs; terms from x^4 on in float
-  float cf = __fmaf_rn(x.h, 2.0876757e-9f, -2.7557319e-7f);
-  cf = __fmaf_rn(x.h, cf, 2.4801587e-5f);
-  dd cp = dd_fma(x, dd_make(cf, 0.f), dd_make(-1.38888892e-3f, 3.3631094e-11f));
+  // coefficients 1 / k! as float pairs; terms from x^5 on in float
+  float cf = __fmaf_rn(x.h, -1.1470746e-11f, 2.0876757e-9f);
+  cf = __fmaf_rn(x.h, cf, -2.7557319e-7f);
+  dd cp = dd_fma(x, dd_make(cf, 0.f), dd_make(2.48015876e-5f, -3.4069961e-13f));
+  cp = dd_fma(x, cp, dd_make(-1.38888892e-3f, 3.3631094e-11f));
   cp = dd_fma(x, cp, dd_make(4.16666679e-2f, -1.2417635e-9f));
   cp = dd_fma(x, cp, dd_make(-0.5f, 0.f));
   cp = dd_fma(x, cp, dd_make(1.f, 0.f));
-  float sf = __fmaf_rn(x.h, 1.6059044e-10f, -2.5052108e-8f);
-  sf = __fmaf_rn(x.h, sf, 2.7557319e-6f);
-  dd sp = dd_fma(x, dd_make(sf, 0.f), dd_make(-1.98412701e-4f, 2.7255968e-12f));
+  float sf = __fmaf_rn(x.h, -7.6471637e-13f, 1.6059044e-10f);
+  sf = __fmaf_rn(x.h, sf, -2.5052108e-8f);
+  dd sp = dd_fma(x, dd_make(sf, 0.f), dd_make(2.75573188e-6f, 3.7935712e-14f));
+  sp = dd_fma(x, sp, dd_make(-1.98412701e-4f, 2.7255968e-12f));
   sp = dd_fma(x, sp, dd_make(8.33333377e-3f, -4.3461720e-10f));
   sp = dd_fma(x, sp, dd_make(-0.16666667f, 4.9670538e-9f));
   sp = dd_fma(x, sp, dd_make(1.f, 0.f));
   sp = dd_mul(sp, t);
+  // (a quarter turn exactly: cp = 1 and sp = 0 are exact)
+  const bool sure = __fadd_rn(cp.h, cp.l + kCisError) == cp.h && __fadd_rn(cp.h, cp.l - kCisError) == cp.h &&
+                    __fadd_rn(sp.h, sp.l + kCisError) == sp.h && __fadd_rn(sp.h, sp.l - kCisError) == sp.h;
+  if (!sure && !(r.h == 0.f && r.l == 0.f)) return cis_turn_f64(c);
   const int k = (int)q & 3;   // quarter turns
   const float co = cp.h, si = sp.h;
   return make_float2(k == 0 ? co : k == 1 ? -si : k == 2 ? -co : si,
