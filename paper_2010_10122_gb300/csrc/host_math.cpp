@@ -564,6 +564,12 @@ static bool choose_grid(int64_t nmin_u, int64_t nmin_v, int prec, int kind, int6
   return std::isfinite(best);
 }
 
+int degrid_shares(double densest, double mean, double least, double ctas, bool f32) {
+  if (!(densest > 1.5 * mean)) return 1;
+  const double pays = std::sqrt(densest / ((f32 ? 0.03 : 0.0065) * std::max(1.0, ctas)));
+  return (int)std::max(1.0, std::min({32.0, std::ceil(densest / least), pays}));
+}
+
 int choose_plan(const PlanInput& in, PlanParams& out, char* err, int errlen) {
   auto fail = [&](const char* msg) {
     std::snprintf(err, errlen, "%s", msg);

@@ -136,6 +136,18 @@ double rounding_gain(const PolyKernel& K, const std::vector<double>& psi_c, int6
 double plane_rounding(int kind, int prec, int64_t nu, int64_t nv);   // u log2(nu nv)
 double rounding_coefficient(double gain);                              // c(G) of the rounding term
 
+// CTAs that share a tile's visibilities when degridding: `densest` visibilities of the fullest CTA
+// against the `mean` over the CTAs the GPU holds at once (a visibility meets (alpha_w + bs - 1) / bs
+// sub-batches of planes), shares of at least `least`, `ctas` tiles x sub-batches.  Every tile gets as many
+// CTAs, and one without work still costs 0.5 - 1.3 ns: Z of them pay while the fullest one's time, which
+// goes as densest / Z, falls by more, up to Z = sqrt(densest / (k ctas)), k the cost of an empty CTA over
+// that of a visibility: 0.03 for FP32 planes, 0.0065 for FP64 and double-float ones.  k fitted to 689 plans
+// (array and random observations, even and crowded, 256^2 - 4096^2, with and without w) with Z = 1 .. 32 each:
+// the rule is 2 - 3 % above the best Z on average.  8e5 visibilities with a fifth in one tile, alpha = 10: 78
+// ms with one CTA, 5.6 by this rule; 2e5 visibilities on 2816^2, half of them in 16 tiles: 0.58 ms with one,
+// 1.01 with the 7 that densest / least alone would give; on 4000^2 without w 0.25 and 0.50.
+int degrid_shares(double densest, double mean, double least, double ctas, bool f32);
+
 struct PlanInput {
   int64_t nx, ny;
   double psx, psy;

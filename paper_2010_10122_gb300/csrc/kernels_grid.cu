@@ -1671,18 +1671,14 @@ static cudaError_t degrid_g(const Geom& g, const Coef<R>& coef, const IndexView<
   size_t smem = coef_bytes<R>() + (size_t)std::min(bs, nb) * degrid_plane_bytes<R>(g);
   int64_t ntiles = (int64_t)g.ntu * g.ntv;
   // several CTAs for the densest tiles, where one would be the run time (they stage the same planes
-  // and sum different visibilities; the sums are the same).  Measured on 8e5 visibilities with a
-  // fifth in one tile, double-float planes, alpha = 10: 78 ms with one CTA, 26 / 14 / 9 ms with 2 / 4 / 8
-  // for every tile, 5.6 ms by this rule; even plans lose by it (2.1 ms alone, 2.4 with two CTAs at a
-  // densest tile of 179 against a mean of 3 000).  Compared: visibilities of the densest
-  // tile's CTA against the mean over the CTAs the GPU holds at once (a visibility meets
-  // (alpha_w + bs - 1) / bs of the sub-batches)
+  // and sum different visibilities; the sums are the same): see degrid_shares
+  const int64_t nsub = (nb + bs - 1) / bs;
   const double meets = g.alpha_w + bs - 1.0;
   const double densest = g.max_tile * std::min(1.0, meets / g.nw);
   const double mean = g.nvis * meets / bs / (152.0 * 4.0);
   const uint32_t least = (uint32_t)std::max(128.0, 0.5 * mean) / 64 * 64;
-  const int Z = densest > 1.5 * mean ? (int)std::min(32.0, std::ceil(densest / least)) : 1;
-  dim3 grid((unsigned)ntiles, (unsigned)((nb + bs - 1) / bs), (unsigned)Z);
+  const int Z = degrid_shares(densest, mean, least, (double)(ntiles * nsub), sizeof(R) == 4);
+  dim3 grid((unsigned)ntiles, (unsigned)nsub, (unsigned)Z);
   if constexpr (sizeof(R) == 8) {
     if (g.df64_planes) {
       smem += (size_t)kThreads * (sizeof(float4) + sizeof(float2));
