@@ -262,46 +262,55 @@ const KernelMath& kernel_math(int alpha, double beta, double mu) {
   return *it->second;
 }
 
-UnitRoots::UnitRoots(int64_t n) : n_(n), step_(1) {
-  while (step_ * step_ < n) step_ *= 2;
-  const long double unit = 6.283185307179586476925286766559L / (8.0L * (long double)n);   // at most n units: pi / 4
-  auto root = [&](int64_t k) {
-    const long double c = cosl(unit * (long double)k), s = sinl(unit * (long double)k);
-    Root r;
-    r.ch = (double)c; r.cl = (double)(c - (long double)r.ch);
-    r.sh = (double)s; r.sl = (double)(s - (long double)r.sh);
-    return r;
-  };
-  for (int64_t a = 0; a * step_ <= n; ++a) coarse_.push_back(root(a * step_));
-  for (int64_t b = 0; b < step_; ++b) fine_.push_back(root(b));
-}
-
-// a b + sgn c d as hi + lo, the pair of floats nearest to it in out.  volatile: the rounded products
-// must not be contracted into the sum below, their errors are added apart.
-static void pair_of_products(double ah, double al, double bh, double bl, double sgn, double ch, double cl,
-                             double dh, double dl, float* out) {
+// a b + sgn c d of hi + lo values, as hi + lo.  volatile: the rounded products must not be contracted
+// into the sum below, their errors are added apart.
+static void sum_of_products(double ah, double al, double bh, double bl, double sgn, double ch, double cl,
+                            double dh, double dl, double* hi, double* lo) {
   const volatile double p = ah * bh, q = sgn * ch * dh;
   const double pe = std::fma(ah, bh, -p), qe = std::fma(sgn * ch, dh, -q);
   const double s = p + q, v = s - p, e = (p - (s - v)) + (q - v);
-  const double lo = e + ((pe + qe) + ((ah * bl + al * bh) + sgn * (ch * dl + cl * dh)));
-  const double r = s + lo;
-  out[0] = (float)r;
-  out[1] = (float)((r - (double)out[0]) + (lo - (r - s)));
+  const double t = e + ((pe + qe) + ((ah * bl + al * bh) + sgn * (ch * dl + cl * dh)));
+  *hi = s + t;
+  *lo = t - (*hi - s);
+}
+
+UnitRoots::Root UnitRoots::product(const Root& a, const Root& b) {
+  Root r;
+  sum_of_products(a.ch, a.cl, b.ch, b.cl, -1.0, a.sh, a.sl, b.sh, b.sl, &r.ch, &r.cl);
+  sum_of_products(a.sh, a.sl, b.ch, b.cl, 1.0, a.ch, a.cl, b.sh, b.sl, &r.sh, &r.sl);
+  return r;
+}
+
+UnitRoots::UnitRoots(int64_t n) : n_(n), step_(1) {
+  while (step_ * step_ < n) step_ *= 2;
+  const long double unit = 6.283185307179586476925286766559L / (8.0L * (long double)n);   // at most n units: pi / 4
+  // roots of k = 0, 1, .. count - 1 times `angle`: the powers of two, the others as products
+  auto fill = [](std::vector<Root>& t, int64_t count, long double angle) {
+    t.push_back(Root{1.0, 0.0, 0.0, 0.0});
+    for (int64_t k = 1; k < count; ++k) {
+      const int64_t low = k & -k;
+      if (k != low) { t.push_back(product(t[(size_t)(k - low)], t[(size_t)low])); continue; }
+      const long double c = cosl(angle * (long double)k), s = sinl(angle * (long double)k);
+      Root r;
+      r.ch = (double)c; r.cl = (double)(c - (long double)r.ch);
+      r.sh = (double)s; r.sl = (double)(s - (long double)r.sh);
+      t.push_back(r);
+    }
+  };
+  fill(fine_, step_, unit);
+  fill(coarse_, n / step_ + 1, unit * (long double)step_);
 }
 
 void UnitRoots::pair(int64_t t, float* out) const {
   t %= n_;
   const int64_t o = 8 * t / n_;   // octant 0 .. 7; k of 8 n units from its nearer axis or diagonal
   const int64_t k = (o & 1) ? (o + 1) * n_ - 8 * t : 8 * t - o * n_;
-  const Root &A = coarse_[(size_t)(k / step_)], &B = fine_[(size_t)(k % step_)];
-  float c[2], s[2];
-  pair_of_products(A.ch, A.cl, B.ch, B.cl, -1.0, A.sh, A.sl, B.sh, B.sl, c);
-  pair_of_products(A.sh, A.sl, B.ch, B.cl, 1.0, A.ch, A.cl, B.sh, B.sl, s);
+  const Root r = product(coarse_[(size_t)(k / step_)], fine_[(size_t)(k % step_)]);
   const bool swap = o == 1 || o == 2 || o == 5 || o == 6;
-  const float *x = swap ? s : c, *y = swap ? c : s;
-  const float sx = o >= 2 && o <= 5 ? -1.f : 1.f, sy = o >= 4 ? 1.f : -1.f;
-  out[0] = sx * x[0]; out[1] = sx * x[1];
-  out[2] = sy * y[0]; out[3] = sy * y[1];
+  const double xh = swap ? r.sh : r.ch, xl = swap ? r.sl : r.cl, yh = swap ? r.ch : r.sh, yl = swap ? r.cl : r.sl;
+  const double sx = o >= 2 && o <= 5 ? -1.0 : 1.0, sy = o >= 4 ? 1.0 : -1.0;
+  out[0] = (float)(sx * xh); out[1] = (float)((sx * xh - (double)out[0]) + sx * xl);
+  out[2] = (float)(sy * yh); out[3] = (float)((sy * yh - (double)out[2]) + sy * yl);
 }
 
 double psi_cheb_eval(const std::vector<double>& c, double k) {

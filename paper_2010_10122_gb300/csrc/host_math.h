@@ -114,6 +114,7 @@ class UnitRoots {
 
  private:
   struct Root { double ch, cl, sh, sl; };   // cos and sin, each hi + lo
+  static Root product(const Root& a, const Root& b);
   int64_t n_, step_;
   std::vector<Root> coarse_, fine_;         // angles a step_ / (8 n) and b / (8 n) of a turn
 };
