@@ -1090,7 +1090,7 @@ k_grid_atomic(const Geom g, const __grid_constant__ Coef<R> coef, const IndexVie
 // instructions per visibility (alpha 6, 1.6e6 visibilities on 42 planes of 2048^2) against 430 here.
 //
 // FP32 accuracy is kept: each factor is cut exactly into three bf16 parts (8 + 8 + 8 significant
-// bits; groups of data below 2^-63 are summed in FP32 instead) and all products of parts down to 2^-24 are summed, the leading ones 8 visibilities at a
+// bits; groups of products with the w kernel below 2^-63 are summed in FP32 instead) and all products of parts down to 2^-24 are summed, the leading ones 8 visibilities at a
 // time and the other seven over 16, each from zero, and added to FP32 accumulators with
 // round-to-nearest (the tensor core drops what lies 24 bits below its largest addend and rounds
 // towards zero, so nothing is carried on in it).  Rounding error of the gridded image against an
@@ -1264,12 +1264,10 @@ k_grid_mma(const Geom g, const __grid_constant__ Coef<float> coef, const IndexVi
       __syncwarp();
       while (cnt >= 16 || (done && cnt > 0)) {
         const int nv = min(cnt, 16);
-        bool tiny;
         // 16 visibilities: lanes 0-15 their coordinates, lanes 16-31 their data
         {
           const int v = lane & 15;
           const MmaEntry q = sm.queue[(head + v) & (kMmaQueue - 1)];
-          bool sizable = false;
           if (v < nv) {
             if (lane < 16) {
               const Z4<float> z = ix.z[q.at];
@@ -1288,11 +1286,8 @@ k_grid_mma(const Geom g, const __grid_constant__ Coef<float> coef, const IndexVi
                 d.x = r;
               }
               sm.d[v] = d;
-              sizable = !(fmaxf(fabsf(d.x), fabsf(d.y)) < 0x1p-63f);
             }
           }
-          // the slices of smaller data would reach into the bf16 subnormals, which end at 2^-133
-          tiny = !__any_sync(0xffffffffu, sizable);
           head = (head + nv) & (kMmaQueue - 1);
           cnt -= nv;
         }
@@ -1315,27 +1310,6 @@ k_grid_mma(const Geom g, const __grid_constant__ Coef<float> coef, const IndexVi
           }
         }
         __syncwarp();
-        if (tiny) {   // in FP32 as they are, each lane the cells of its fragments
-#pragma unroll 1
-          for (int v = 0; v < nv; ++v) {
-            const float* u = &sm.wu[v][kMmaPad + sr0 + gid - sm.ru[v]];
-            const float* w = &sm.wv[v][kMmaPad + sc0 + 2 * tig - sm.rv[v]];
-            const float x[2] = {u[0], u[8]}, y[4] = {w[0], w[1], w[8], w[9]};
-#pragma unroll
-            for (int pl = 0; pl < kMmaPlanes; ++pl) {
-              const float2 d = sm.dw[v][pl];
-#pragma unroll
-              for (int c = 0; c < 4; ++c)
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                  acc[pl][c & 2][2 * r + (c & 1)] = __fmaf_rn(x[r], y[c] * d.x, acc[pl][c & 2][2 * r + (c & 1)]);
-                  acc[pl][(c & 2) + 1][2 * r + (c & 1)] = __fmaf_rn(x[r], y[c] * d.y, acc[pl][(c & 2) + 1][2 * r + (c & 1)]);
-                }
-            }
-          }
-          __syncwarp();
-          continue;
-        }
         // this lane's four visibilities: k = 2 tig, 2 tig + 1, 2 tig + 8, 2 tig + 9
         float x[4][2], y[4][2];   // wu at rows gid, gid + 8; wv at columns gid, gid + 8
 #pragma unroll
@@ -1353,13 +1327,34 @@ k_grid_mma(const Geom g, const __grid_constant__ Coef<float> coef, const IndexVi
 #pragma unroll
         for (int pl = 0; pl < kMmaPlanes; ++pl) {
           float2 d[4];
-          bool any = false;
+          bool sizable = false, any = false;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             d[q] = sm.dw[2 * tig + (q & 1) + (q & 2) * 4][pl];
+            sizable = sizable || !(fabsf(d[q].x) < 0x1p-63f) || !(fabsf(d[q].y) < 0x1p-63f);
             any = any || d[q].x != 0.f || d[q].y != 0.f;
           }
-          if (!__any_sync(0xffffffffu, any)) continue;
+          if (!__any_sync(0xffffffffu, sizable)) {
+            if (!__any_sync(0xffffffffu, any)) continue;
+            // the slices of such data would reach into the bf16 subnormals, which end at 2^-133: in FP32
+            // as they are, each lane the cells of its fragments
+#pragma unroll 1
+            for (int v = 0; v < nv; ++v) {
+              const float* u = &sm.wu[v][kMmaPad + sr0 + gid - sm.ru[v]];
+              const float* w = &sm.wv[v][kMmaPad + sc0 + 2 * tig - sm.rv[v]];
+              const float2 e = sm.dw[v][pl];
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                  const float wc = w[(c & 1) + 4 * (c & 2)], ur = u[8 * r];
+                  float &re = acc[pl][c & 2][2 * r + (c & 1)], &im = acc[pl][(c & 2) + 1][2 * r + (c & 1)];
+                  re = __fmaf_rn(ur, wc * e.x, re);
+                  im = __fmaf_rn(ur, wc * e.y, im);
+                }
+            }
+            continue;
+          }
 #pragma unroll
           for (int nt = 0; nt < 4; ++nt) {
             float b[4];
