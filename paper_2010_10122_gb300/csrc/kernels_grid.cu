@@ -104,22 +104,24 @@ __device__ __forceinline__ unsigned group_mask() {
 // The visibilities of tile t that meet each of the planes s0 .. s0 + sb - 1 (at most 32): lane pl
 // holds plane s0 + pl's index range, so that all are known after one load.
 struct DegridRange {
-  uint32_t lo, hi;   // over all the planes; this CTA's share of them after split()
-  unsigned used;     // planes some visibility meets
+  uint32_t first, end;   // of this lane's plane
+  unsigned used;         // planes some visibility meets
+  uint32_t lo, hi;       // this CTA's visibilities (share)
   __device__ __forceinline__ DegridRange(const uint32_t* __restrict__ offt, int nw, int aw, int s0, int sb) {
     const int lane = threadIdx.x & 31, p = s0 + min(lane, sb - 1);
-    const uint32_t a = offt[max(0, p - aw + 1)], b = offt[min(p + 1, nw)];
-    lo = __shfl_sync(0xffffffffu, a, 0);
-    hi = __shfl_sync(0xffffffffu, b, sb - 1);
-    used = __ballot_sync(0xffffffffu, lane < sb && a != b);
+    first = offt[max(0, p - aw + 1)];
+    end = offt[min(p + 1, nw)];
+    used = __ballot_sync(0xffffffffu, lane < sb && first != end);
   }
   // blockIdx.z's share among gridDim.z CTAs, of at least `least` visibilities (a multiple of 64, so
   // that shares are whole passes of a CTA): only tiles with more are taken by several
-  __device__ __forceinline__ void split(uint32_t least) {
+  __device__ __forceinline__ void share(int sb, uint32_t least) {
+    lo = __shfl_sync(0xffffffffu, first, 0);
+    hi = __shfl_sync(0xffffffffu, end, sb - 1);
     if (gridDim.z == 1) return;
-    const uint32_t share = max(least, ((hi - lo + gridDim.z - 1) / gridDim.z + 63) & ~63u);
-    lo = min(hi, lo + blockIdx.z * share);
-    hi = min(hi, lo + share);
+    const uint32_t n = max(least, ((hi - lo + gridDim.z - 1) / gridDim.z + 63) & ~63u);
+    lo = min(hi, lo + blockIdx.z * n);
+    hi = min(hi, lo + n);
   }
 };
 // f(cell of the buffer, cell of the plane) for the tile and its halo in the used planes: a warp
@@ -177,9 +179,10 @@ k_degrid(const Geom g, const __grid_constant__ Coef<R> coef, const IndexView<R> 
   const int sb = min(bs, b0 + nb - s0);
   const int sbid = s0 / bs;                       // global sub-batch id (s0 is a multiple of bs)
   DegridRange range(ix.off + (int64_t)t * g.nw, g.nw, aw, s0, sb);
-  range.split(least);
+  if (range.used == 0) return;                    // no visibility of this tile meets these planes
+  range.share(sb, least);
   const uint32_t lo = range.lo, hi = range.hi;
-  if (lo == hi) return;                           // no visibility of this tile meets these planes
+  if (lo == hi) return;
   degrid_rows(g, tu, tv, s0 - b0, sb, range.used,
               [&](int e, int64_t cell) { stage_copy(st + e, planes + cell); });
   for (int i = threadIdx.x; i < (g.deg + 1) * kMaxG; i += blockDim.x) sc[i] = coef.c[i];
@@ -256,15 +259,20 @@ k_degrid(const Geom g, const __grid_constant__ Coef<R> coef, const IndexView<R> 
 // degrid of double-float planes (FP64 plans with the double-float FFT)
 //
 // The same decomposition as k_degrid, on planes whose cells are double-float pairs (float4:
-// re hi, re lo, im hi, im lo): the tile + halo is staged and then reordered in place to (re hi, im
-// hi, re lo, im lo), kernel values come as pairs (the kernel-value table stores them split), and the
-// footprint sum runs in pair arithmetic on the FP32 pipes, real and imaginary part packed (15
-// packed FP32 instructions for two FP64 FMAs, which GB300 issues at 1/64 of the FP32 rate).  Each
-// lane sums its column over rows, four planes at once (independent chains; two: 8.5 against 8.3 ms),
-// the u weights come from shared memory (in registers they leave room for two planes only: 9.9 ms),
-// the lanes' sums are reduced by shuffles in pair arithmetic, and the partial sum is stored in
-// FP64 as in k_degrid.  1e6 visibilities on a 3456^2 grid, alpha = 15: 9.6 -> 8.3 ms, 4.2 of them
-// with the sums left out.
+// re hi, re lo, im hi, im lo): kernel values come as pairs (the kernel-value table stores them split), and the
+// footprint sum runs in pair arithmetic on the FP32 pipes (15 instructions for an FP64 FMA, which GB300
+// issues at 1/64 of the FP32 rate).  Two forms:
+//  * packed (supports above 8, with w): real and imaginary part in one packed instruction, the staged cells
+//    reordered in place to (re hi, im hi, re lo, im lo); each lane sums its column over rows, four planes
+//    at once (independent chains; two: 8.5 against 8.3 ms), the u weights from shared memory (in
+//    registers they leave room for two planes only: 9.9 ms).  1e6 visibilities on a 3456^2 grid, alpha = 15:
+//    10.1 -> 8.6 ms, 4.2 of them with the sums left out.
+//  * one plane at a time, unpacked, u weights in registers: without w there is one plane (1e6 visibilities on
+//    1024 x 768, alpha = 14: 0.54 ms, packed 0.72), and 32-cell tiles leave two or three planes to a CTA, which
+//    a group of four fills badly, and room for four CTAs per SM where the packed form's registers take three
+//    (alpha = 7, 1e6 visibilities on 3072^2: 2.42 ms, packed 3.18).
+// The lanes' sums are reduced by shuffles in pair arithmetic, and the partial sum is stored in FP64 as
+// in k_degrid.
 // ---------------------------------------------------------------------------------------
 // piece j of direction d of indexed visibility vi as a double-float pair
 __device__ __forceinline__ dd kernel_value_dd(const IndexView<double>& ix, const double* __restrict__ sc,
@@ -290,14 +298,22 @@ __device__ __forceinline__ d2 d2_fma_weight(f2 wh, f2 nwh, f2 nwl, d2 d, d2 c) {
   return d2_fast_two_sum(s.h, s_add(s.l, s_sub(c.l, e)));
 }
 
-template <int G>
-__global__ void __launch_bounds__(kThreads, 3)
+constexpr size_t kDegridWeights = kThreads * (sizeof(float4) + sizeof(float2));
+// shared memory of k_degrid_dd beside the planes.  With a kernel-value table at most 76 KB in all for every
+// support, so that an SM holds three CTAs
+__host__ __device__ constexpr size_t degrid_dd_fixed(bool packed, bool table) {
+  return (packed ? kDegridWeights : 0) + (packed && table ? 0 : (kMaxDeg + 1) * kMaxG * sizeof(double));
+}
+
+template <int G, bool kPacked>
+__global__ void __launch_bounds__(kThreads, G == 16 ? 3 : 4)
 k_degrid_dd(const Geom g, const __grid_constant__ Coef<double> coef, const IndexView<double> ix,
             const double2* __restrict__ planes, int b0, int nb, int bs,
             double2* __restrict__ partial, int64_t nvis_idx, uint32_t least) {
   extern __shared__ __align__(16) unsigned char smem[];
+  // the coefficients where there is no kernel-value table, the planes, the groups' u weights (packed form)
   double* sc = reinterpret_cast<double*>(smem);
-  double2* st = reinterpret_cast<double2*>(smem + (kMaxDeg + 1) * kMaxG * sizeof(double));
+  double2* st = reinterpret_cast<double2*>(smem + degrid_dd_fixed(kPacked, ix.wts != nullptr) - (kPacked ? kDegridWeights : 0));
   const int T = g.tile, alpha = g.alpha, aw = g.alpha_w;
   const int TH = T + alpha - 1;
   const int t = blockIdx.x;
@@ -306,14 +322,15 @@ k_degrid_dd(const Geom g, const __grid_constant__ Coef<double> coef, const Index
   const int sb = min(bs, b0 + nb - s0);
   const int sbid = s0 / bs;                       // global sub-batch id (s0 is a multiple of bs)
   DegridRange range(ix.off + (int64_t)t * g.nw, g.nw, aw, s0, sb);
-  range.split(least);
+  if (range.used == 0) return;                    // no visibility of this tile meets these planes
+  range.share(sb, least);
   const uint32_t lo = range.lo, hi = range.hi;
-  if (lo == hi) return;                           // no visibility of this tile meets these planes
+  if (lo == hi) return;
   const int j = threadIdx.x & (G - 1);
   const int grp = threadIdx.x / G, ngrp = blockDim.x / G;
   const dd zero = dd_make(0.f, 0.f);
-  float4* wt = reinterpret_cast<float4*>(st + (size_t)min(bs, nb) * TH * TH) + grp * G;
-  float2* wt2 = reinterpret_cast<float2*>(wt + (ngrp - grp) * G) + grp * G;
+  [[maybe_unused]] float4* wt = reinterpret_cast<float4*>(st + (size_t)min(bs, nb) * TH * TH) + grp * G;
+  [[maybe_unused]] float2* wt2 = reinterpret_cast<float2*>(wt + (ngrp - grp) * G) + grp * G;
   // with a kernel-value table, the group's next visibility's index entry and table values are
   // loaded while the current one is summed (the loads' latency is otherwise exposed), and the
   // first one's while the planes are staged
@@ -337,13 +354,15 @@ k_degrid_dd(const Geom g, const __grid_constant__ Coef<double> coef, const Index
   degrid_rows(g, tu, tv, s0 - b0, sb, range.used,
               [&](int e, int64_t cell) { stage_copy(st + e, planes + cell); });
   stage_wait();
-  // (re hi, re lo, im hi, im lo) to (re hi, im hi, re lo, im lo): each thread the cells it copied
-  degrid_rows(g, tu, tv, s0 - b0, sb, range.used, [&](int e, int64_t) {
-    float4* v = reinterpret_cast<float4*>(st) + e;
-    const float2 m = make_float2(v->y, v->z);
-    v->y = m.y;
-    v->z = m.x;
-  });
+  if constexpr (kPacked) {
+    // (re hi, re lo, im hi, im lo) to (re hi, im hi, re lo, im lo): each thread the cells it copied
+    degrid_rows(g, tu, tv, s0 - b0, sb, range.used, [&](int e, int64_t) {
+      float4* v = reinterpret_cast<float4*>(st) + e;
+      const float2 m = make_float2(v->y, v->z);
+      v->y = m.y;
+      v->z = m.x;
+    });
+  }
   __syncthreads();
   for (; v0 < hi; v0 += ngrp) {
     const uint32_t vi = v0 + gofs;
@@ -367,53 +386,80 @@ k_degrid_dd(const Geom g, const __grid_constant__ Coef<double> coef, const Index
       }
     }
     if (!g.do_w) pw = j == 0 ? dd_make(1.f, 0.f) : zero;
-    __syncwarp();   // the previous visibility's weights are consumed
-    wt[j] = make_float4(-pu.h, -pu.h, -pu.l, -pu.l);
-    wt2[j] = make_float2(pu.h, pu.h);
-    __syncwarp();
     const int qlo = act ? max(0, s0 - c0) : G, qhi = act ? min(aw, s0 + sb - c0) : 0;
     const int wlo = __reduce_min_sync(0xffffffffu, (unsigned)qlo);
     const int whi = __reduce_max_sync(0xffffffffu, (unsigned)qhi);
-    const int cell = du * TH + dv + (lj ? j : 0);
-    d2 acc{f2_make(0.f, 0.f), f2_make(0.f, 0.f)};   // (re, im)
-    // NP planes from q on at once: their column sums are independent chains
-    auto planes_sum = [&](int q, auto np) {
-      constexpr int NP = decltype(np)::value;
-      const ulonglong2* row[NP];
-      bool on[NP];
-      d2 sum[NP];
+    dd ar = zero, ai = zero;
+    if constexpr (kPacked) {
+      __syncwarp();   // the previous visibility's weights are consumed
+      wt[j] = make_float4(-pu.h, -pu.h, -pu.l, -pu.l);
+      wt2[j] = make_float2(pu.h, pu.h);
+      __syncwarp();
+      const int cell = du * TH + dv + (lj ? j : 0);
+      d2 acc{f2_make(0.f, 0.f), f2_make(0.f, 0.f)};   // (re, im)
+      // NP planes from q on at once: their column sums are independent chains
+      auto planes_sum = [&](int q, auto np) {
+        constexpr int NP = decltype(np)::value;
+        const ulonglong2* row[NP];
+        bool on[NP];
+        d2 sum[NP];
 #pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        on[n] = lj && q + n >= qlo && q + n < qhi;
-        const int pl = on[n] ? c0 + q + n - s0 : 0;
-        row[n] = reinterpret_cast<const ulonglong2*>(st) + pl * TH * TH + cell;
-        sum[n].h = sum[n].l = f2_make(0.f, 0.f);
-      }
+        for (int n = 0; n < NP; ++n) {
+          on[n] = lj && q + n >= qlo && q + n < qhi;
+          const int pl = on[n] ? c0 + q + n - s0 : 0;
+          row[n] = reinterpret_cast<const ulonglong2*>(st) + pl * TH * TH + cell;
+          sum[n].h = sum[n].l = f2_make(0.f, 0.f);
+        }
 #pragma unroll
-      for (int i = 0; i < G; ++i) {
-        if (i < alpha) {
-          const ulonglong2 nw = *reinterpret_cast<const ulonglong2*>(&wt[i]);
-          const f2 wh{*reinterpret_cast<const pk64*>(&wt2[i])}, nwh{nw.x}, nwl{nw.y};
+        for (int i = 0; i < G; ++i) {
+          if (i < alpha) {
+            const ulonglong2 nw = *reinterpret_cast<const ulonglong2*>(&wt[i]);
+            const f2 wh{*reinterpret_cast<const pk64*>(&wt2[i])}, nwh{nw.x}, nwl{nw.y};
 #pragma unroll
-          for (int n = 0; n < NP; ++n) {
-            const ulonglong2 v = row[n][i * TH];
-            sum[n] = d2_fma_weight(wh, nwh, nwl, d2{f2{v.x}, f2{v.y}}, sum[n]);
+            for (int n = 0; n < NP; ++n) {
+              const ulonglong2 v = row[n][i * TH];
+              sum[n] = d2_fma_weight(wh, nwh, nwl, d2{f2{v.x}, f2{v.y}}, sum[n]);
+            }
           }
         }
-      }
 #pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        const dd wq = shfl_dd(pw, q + n, G);
-        // a plane the visibility does not meet (or a lane past its columns) gave what it read
-        if (!on[n]) sum[n].h = sum[n].l = f2_make(0.f, 0.f);
-        acc = d2_fma_weight(f2_make(wq.h, wq.h), f2_make(-wq.h, -wq.h), f2_make(-wq.l, -wq.l), sum[n], acc);
+        for (int n = 0; n < NP; ++n) {
+          const dd wq = shfl_dd(pw, q + n, G);
+          // a plane the visibility does not meet (or a lane past its columns) gave what it read
+          if (!on[n]) sum[n].h = sum[n].l = f2_make(0.f, 0.f);
+          acc = d2_fma_weight(f2_make(wq.h, wq.h), f2_make(-wq.h, -wq.h), f2_make(-wq.l, -wq.l), sum[n], acc);
+        }
+      };
+      int q = wlo;
+      for (; q + 2 < whi; q += 4) planes_sum(q, std::integral_constant<int, 4>());
+      if (q < whi) planes_sum(q, std::integral_constant<int, 2>());
+      const float2 ach = f2_split(acc.h), acl = f2_split(acc.l);
+      ar = dd_make(ach.x, acl.x);
+      ai = dd_make(ach.y, acl.y);
+    } else {
+      dd wu[G];
+#pragma unroll
+      for (int i = 0; i < G; ++i) wu[i] = shfl_dd(pu, i, G);
+      for (int q = wlo; q < whi; ++q) {
+        const dd wq = shfl_dd(pw, q, G);
+        if (lj && q >= qlo && q < qhi) {
+          const float4* row = reinterpret_cast<const float4*>(st + (c0 + q - s0) * TH * TH + du * TH + dv + j);
+          dd sr = zero, si = zero;
+#pragma unroll
+          for (int i = 0; i < G; ++i) {
+            if (i < alpha) {
+              const float4 gv = row[i * TH];
+              sr = dd_fma(wu[i], dd_make(gv.x, gv.y), sr);
+              si = dd_fma(wu[i], dd_make(gv.z, gv.w), si);
+            }
+          }
+          ar = dd_fma(wq, sr, ar);
+          ai = dd_fma(wq, si, ai);
+        }
       }
-    };
-    int q = wlo;
-    for (; q + 2 < whi; q += 4) planes_sum(q, std::integral_constant<int, 4>());
-    if (q < whi) planes_sum(q, std::integral_constant<int, 2>());
-    const float2 ach = f2_split(acc.h), acl = f2_split(acc.l);
-    dd ar = dd_mul(dd_make(ach.x, acl.x), pv), ai = dd_mul(dd_make(ach.y, acl.y), pv);
+    }
+    ar = dd_mul(ar, pv);
+    ai = dd_mul(ai, pv);
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) {
       ar = dd_add(ar, dd_make(__shfl_xor_sync(0xffffffffu, ar.h, o, G), __shfl_xor_sync(0xffffffffu, ar.l, o, G)));
@@ -1676,12 +1722,16 @@ static cudaError_t degrid_g(const Geom& g, const Coef<R>& coef, const IndexView<
   dim3 grid((unsigned)ntiles, (unsigned)nsub, (unsigned)Z);
   if constexpr (sizeof(R) == 8) {
     if (g.df64_planes) {
-      smem += (size_t)kThreads * (sizeof(float4) + sizeof(float2));
-      cudaError_t e = cudaFuncSetAttribute(k_degrid_dd<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
-      if (e != cudaSuccess) return e;
-      k_degrid_dd<G><<<grid, kThreads, smem, s>>>(g, coef, ix, planes, b0, nb, bs, partial, nvis_idx, least);
-      return cudaGetLastError();
+      auto launch = [&](auto kernel, bool packed) {
+        const size_t bytes = smem - coef_bytes<R>() + degrid_dd_fixed(packed, ix.wts != nullptr);
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+        kernel<<<grid, kThreads, bytes, s>>>(g, coef, ix, planes, b0, nb, bs, partial, nvis_idx, least);
+        return cudaGetLastError();
+      };
+      if constexpr (G == 16)
+        if (g.do_w) return launch(k_degrid_dd<G, true>, true);
+      return launch(k_degrid_dd<G, false>, false);
     }
   }
   cudaError_t e = cudaFuncSetAttribute(k_degrid<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
