@@ -1205,10 +1205,12 @@ static cudaError_t launch_lines(const FftLine& L, double2* data, int64_t batch, 
   return cudaGetLastError();
 }
 
+static bool on_pairs(const SideFft& f, int fwd) { return f.pairs && !(fwd && f.fwd_lines); }
+
 static cudaError_t launch_side(const SideFft& f, double2* data, int64_t batch, int64_t plane,
                                int lines, int64_t line_stride, int64_t elem_stride, int mode,
                                int fwd, int split, int skip, int lhalf, int shalf, cudaStream_t s) {
-  return f.pairs && !(fwd && f.fwd_lines)
+  return on_pairs(f, fwd)
              ? launch_pairs(f.pl, data, batch, plane, lines, line_stride, elem_stride, fwd, split,
                             skip, lhalf, shalf, s)
              : launch_lines(f.fl, data, batch, plane, lines, line_stride, elem_stride, mode, fwd,
@@ -1251,26 +1253,26 @@ cudaError_t df64_fft_exec(Df64Fft* f, double2* data, int64_t batch, int sign, cu
   const bool prune = keep_rows > 0 && keep_cols > 0;
   if (prune && ((keep_rows & 1) || (keep_cols & 1) || keep_rows > f->nu || keep_cols > f->nv))
     return cudaErrorInvalidValue;
-  // pass modes: 0 loads doubles and stores pairs, 1 loads pairs and stores doubles, 2 pairs
-  // in and out; the grid side is the forward output / inverse input, the image side the other
-  // the line-pair kernels take and give pairs only: complex128 data are converted around them
-  const bool conv = f->u.pairs || f->v.pairs;
-  const int img_in = image_pairs || conv ? 2 : 0, img_out = image_pairs || conv ? 2 : 1;
-  const int uv_in = df64_planes || conv ? 2 : 0, uv_out = df64_planes || conv ? 2 : 1;
-  cudaError_t e;
+  // pass modes of the line kernels: 0 loads doubles and stores pairs, 1 loads pairs and stores
+  // doubles, 2 pairs in and out; between the passes pairs.  The line-pair kernels take and give pairs
+  // only: complex128 data are converted before a first pass and after a second pass that they run
+  const SideFft &first = prune && fwd ? f->u : f->v, &second = prune && fwd ? f->v : f->u;
   const bool in_pairs = fwd ? image_pairs : df64_planes, out_pairs = fwd ? df64_planes : image_pairs;
+  const bool conv_in = !in_pairs && on_pairs(first, fwd), conv_out = !out_pairs && on_pairs(second, fwd);
+  const int mode_in = in_pairs || conv_in ? 2 : 0, mode_out = out_pairs || conv_out ? 2 : 1;
+  cudaError_t e;
   auto convert = [&](int back) {
     k_to_pairs<<<152 * 8, 256, 0, s>>>(data, batch * plane, back);
     return cudaGetLastError();
   };
-  if (conv && !in_pairs && (e = convert(0)) != cudaSuccess) return e;
-  auto done = [&](cudaError_t r) { return r == cudaSuccess && conv && !out_pairs ? convert(1) : r; };
+  if (conv_in && (e = convert(0)) != cudaSuccess) return e;
+  auto done = [&](cudaError_t r) { return r == cudaSuccess && conv_out ? convert(1) : r; };
   if (!prune) {
     // rows (length nv, contiguous), then columns (length nu, stride nv)
-    e = launch_side(f->v, data, batch, plane, f->nu, f->nv, 1, fwd ? img_in : uv_in, fwd,
+    e = launch_side(f->v, data, batch, plane, f->nu, f->nv, 1, mode_in, fwd,
                      f->nu, 0, f->nv, f->nv, s);
     if (e != cudaSuccess) return e;
-    return done(launch_side(f->u, data, batch, plane, f->nv, 1, f->nv, fwd ? uv_out : img_out, fwd,
+    return done(launch_side(f->u, data, batch, plane, f->nv, 1, f->nv, mode_out, fwd,
                             f->nv, 0, f->nu, f->nu, s));
   }
   const int rh = (int)(keep_rows / 2);   // image half-extent along u (rows)
@@ -1279,16 +1281,16 @@ cudaError_t df64_fft_exec(Df64Fft* f, double2* data, int64_t batch, int sign, cu
   if (fwd) {
     // image columns (length nu, stride nv), image rows loaded; then all rows (length nv),
     // image columns loaded
-    e = launch_side(f->u, data, batch, plane, ncols, 1, f->nv, img_in, fwd, ch, cskip, rh,
+    e = launch_side(f->u, data, batch, plane, ncols, 1, f->nv, mode_in, fwd, ch, cskip, rh,
                      f->nu, s);
     if (e != cudaSuccess) return e;
-    return done(launch_side(f->v, data, batch, plane, f->nu, f->nv, 1, uv_out, fwd, f->nu, 0, ch,
+    return done(launch_side(f->v, data, batch, plane, f->nu, f->nv, 1, mode_out, fwd, f->nu, 0, ch,
                             f->nv, s));
   }
   // inverse: all rows, image columns stored; then the image columns, image rows stored
-  e = launch_side(f->v, data, batch, plane, f->nu, f->nv, 1, uv_in, fwd, f->nu, 0, f->nv, ch, s);
+  e = launch_side(f->v, data, batch, plane, f->nu, f->nv, 1, mode_in, fwd, f->nu, 0, f->nv, ch, s);
   if (e != cudaSuccess) return e;
-  return done(launch_side(f->u, data, batch, plane, ncols, 1, f->nv, img_out, fwd, ch, cskip, f->nu,
+  return done(launch_side(f->u, data, batch, plane, ncols, 1, f->nv, mode_out, fwd, ch, cskip, f->nu,
                           rh, s));
 }
 
