@@ -814,12 +814,14 @@ static dd host_dd(long double v) {
 }
 
 // One side's transform: pairs of lines where the side allows it, else one line per CTA / cluster.
+constexpr int kFewLines = 1024;   // lines of a pass, points of a line: see on_pairs
 struct SideFft {
-  bool pairs = false, fwd_lines = false;   // fwd_lines: one line per CTA for the forward transform
-  PairLine pl;
-  FftLine fl;
-  // line twiddles, then (split lines) the decimation twiddles; those of fl beside pairs
-  float4 *tw = nullptr, *twl = nullptr;
+  bool pairs = false, lines = false;   // which kernels have tables
+  bool fwd_lines = false;              // one line per CTA for the forward transform
+  PairLine pl{};
+  FftLine fl{};
+  // twiddles of pl, then those of fl: each the line's, then (split lines) the decimation step's
+  float4* tw = nullptr;
 };
 struct Df64Fft {
   int nu = 0, nv = 0;
@@ -927,7 +929,8 @@ static void pair_entry(const UnitRoots& roots, int64_t t, float4* e) {
   e[1] = make_float4(w[2], w[2], w[3], w[3]);
 }
 
-static cudaError_t make_pairs(PairLine* L, float4** tw) {
+// appends the line's twiddles; returns where those of the decimation step start
+static size_t pair_table(PairLine* L, std::vector<float4>* table) {
   int entries = 0, Ns = 1;
   for (int s = 0; s < L->nst; ++s) {
     L->twofs[s] = entries;
@@ -937,7 +940,9 @@ static cudaError_t make_pairs(PairLine* L, float4** tw) {
   }
   const int own = entries;
   entries += (L->S - 1) * L->n;
-  std::vector<float4> h(2 * (size_t)std::max(1, entries));
+  const size_t at = table->size();
+  table->resize(at + 2 * (size_t)std::max(1, entries));
+  float4* h = table->data() + at;
   const int64_t N = (int64_t)L->S * L->n;
   const UnitRoots roots(N);
   Ns = 1;
@@ -953,12 +958,7 @@ static cudaError_t make_pairs(PairLine* L, float4** tw) {
   for (int r = 1; r < L->S; ++r)
     for (int j = 0; j < L->n; ++j)
       pair_entry(roots, (int64_t)j * r, &h[2 * (size_t)(own + (r - 1) * L->n + j)]);
-  cudaError_t e = cudaMalloc((void**)tw, sizeof(float4) * h.size());
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpy(*tw, h.data(), sizeof(float4) * h.size(), cudaMemcpyHostToDevice);
-  L->tw = *tw;
-  L->tw2 = *tw + 2 * own;
-  return e;
+  return at + 2 * (size_t)own;
 }
 
 // Launch configuration of `blocks` CTAs (a multiple of L.S) of the pair kernel
@@ -1032,17 +1032,34 @@ static constexpr int64_t kMaxSide = kDf64MaxSide;
 
 bool df64_fft_supported(int64_t nu, int64_t nv) { return df64_side_ok(nu) && df64_side_ok(nv); }
 
-// e^{-2 pi i t / len} for t = 0 .. count - 1 as df64 (float4: re hi, re lo, im hi, im lo)
-static void twiddles(int len, int count, float4* h) {
-  const long double two_pi = 6.283185307179586476925286766559L;
-  for (int t = 0; t < count; ++t) {
-    long double a = two_pi * (long double)t / (long double)len;
-    dd c = host_dd(cosl(a)), s = host_dd(-sinl(a));
-    h[t] = make_float4(c.h, c.l, s.h, s.l);
-  }
+// e^{-2 pi i t / len}, t = 0 .. len - 1, as df64 (float4: re hi, re lo, im hi, im lo)
+static void twiddles(int len, float4* h) {
+  const UnitRoots roots(len);
+  for (int t = 0; t < len; ++t) roots.pair(t, &h[t].x);
 }
 
-static cudaError_t make_line(int nline, FftLine* L, float4** tw) {
+static DftConst dft_constants() {
+  DftConst k;
+  const long double pi = 3.141592653589793238462643383279L;
+  k.c31 = host_dd(sinl(2 * pi / 3));
+  k.c51 = host_dd(cosl(2 * pi / 5));
+  k.c52 = host_dd(cosl(4 * pi / 5));
+  k.s51 = host_dd(sinl(2 * pi / 5));
+  k.s52 = host_dd(sinl(4 * pi / 5));
+  k.r2 = host_dd(sqrtl(2.0L) / 2);
+  for (int q = 1; q <= 3; ++q) {
+    k.c7[q - 1] = host_dd(cosl(2 * pi * q / 7));
+    k.s7[q - 1] = host_dd(sinl(2 * pi * q / 7));
+  }
+  for (int q = 1; q <= 5; ++q) {
+    k.c11[q - 1] = host_dd(cosl(2 * pi * q / 11));
+    k.s11[q - 1] = host_dd(sinl(2 * pi * q / 11));
+  }
+  return k;
+}
+
+// appends the line's twiddles
+static cudaError_t line_table(int nline, FftLine* L, std::vector<float4>* table) {
   std::memset(L, 0, sizeof(*L));
   const int S = df64_line_split(nline);
   if (S == 0) return cudaErrorInvalidValue;
@@ -1054,60 +1071,52 @@ static cudaError_t make_line(int nline, FftLine* L, float4** tw) {
   L->nst = lp.nst;
   L->threads = lp.threads;
   for (int i = 0; i < lp.nst; ++i) L->radix[i] = lp.radix[i];
-  const bool split = S > 1;
-  const int ntab = split ? n + nline : n;
-  std::vector<float4> h(ntab);
-  twiddles(n, n, h.data());
-  if (split) twiddles(nline, nline, h.data() + n);
-  cudaError_t e = cudaMalloc((void**)tw, sizeof(float4) * ntab);
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpy(*tw, h.data(), sizeof(float4) * ntab, cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return e;
-  L->tw = *tw;
-  L->tw2 = split ? *tw + n : nullptr;
-  const long double pi = 3.141592653589793238462643383279L;
-  L->k.c31 = host_dd(sinl(2 * pi / 3));
-  L->k.c51 = host_dd(cosl(2 * pi / 5));
-  L->k.c52 = host_dd(cosl(4 * pi / 5));
-  L->k.s51 = host_dd(sinl(2 * pi / 5));
-  L->k.s52 = host_dd(sinl(4 * pi / 5));
-  L->k.r2 = host_dd(sqrtl(2.0L) / 2);
-  for (int q = 1; q <= 3; ++q) {
-    L->k.c7[q - 1] = host_dd(cosl(2 * pi * q / 7));
-    L->k.s7[q - 1] = host_dd(sinl(2 * pi * q / 7));
-  }
-  for (int q = 1; q <= 5; ++q) {
-    L->k.c11[q - 1] = host_dd(cosl(2 * pi * q / 11));
-    L->k.s11[q - 1] = host_dd(sinl(2 * pi * q / 11));
-  }
+  const size_t at = table->size();
+  table->resize(at + n + (S > 1 ? nline : 0));
+  twiddles(n, table->data() + at);
+  if (S > 1) twiddles(nline, table->data() + at + n);
+  static const DftConst k = dft_constants();
+  L->k = k;
   return cudaSuccess;
 }
 
-static cudaError_t make_side(int n, SideFft* f) {
+static cudaError_t make_side(int n, int64_t most_lines, SideFft* f) {
   f->pairs = pair_plan(n, &f->pl) && pair_cluster_fits(f->pl);
-  if (!f->pairs) return make_line(n, &f->fl, &f->tw);
+  std::vector<float4> table;
+  size_t pair_split = 0, line = 0;
+  cudaError_t e = cudaSuccess;
   // sides of the radices 2 and 5 only, which pairs take in four stages with idle lanes: forward
   // and inverse at the pairs' speed against the lines', on square sides with pruning: 640 0.92 /
   // 1.65, 800 0.98 / 1.44, 1280 1.02 / 1.28, 1600 0.92 / 1.10 (other sides from 0.97 up: 128; 1152
   // 1.03 / 1.40, 960 and up)
-  f->fwd_lines = f->pl.S == 1 && n >= 640 && n % 5 == 0 && n % 3 && n % 7 && n % 11;
-  cudaError_t e = make_pairs(&f->pl, &f->tw);
-  if (e == cudaSuccess && f->fwd_lines) e = make_line(n, &f->fl, &f->twl);
+  f->fwd_lines = f->pairs && f->pl.S == 1 && n >= 640 && n % 5 == 0 && n % 3 && n % 7 && n % 11;
+  f->lines = !f->pairs || f->fwd_lines || (n <= kFewLines && most_lines <= 2 * kFewLines);   // see on_pairs
+  if (f->pairs) pair_split = pair_table(&f->pl, &table);
+  if (f->lines) {
+    line = table.size();
+    e = line_table(n, &f->fl, &table);
+  }
+  if (e == cudaSuccess) e = cudaMalloc((void**)&f->tw, sizeof(float4) * table.size());
+  if (e == cudaSuccess) e = cudaMemcpy(f->tw, table.data(), sizeof(float4) * table.size(), cudaMemcpyHostToDevice);
+  f->pl.tw = f->tw;
+  f->pl.tw2 = f->tw + pair_split;
+  f->fl.tw = f->tw + line;
+  f->fl.tw2 = f->fl.split > 1 ? f->fl.tw + f->fl.n : nullptr;
   return e;
 }
 
-cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
+cudaError_t df64_fft_create(int64_t nu, int64_t nv, int64_t batch, Df64Fft** out) {
   *out = nullptr;
   if (!df64_fft_supported(nu, nv)) return cudaErrorInvalidValue;
   Df64Fft* f = new Df64Fft();
   f->nu = (int)nu; f->nv = (int)nv;
   cudaError_t e = pair_smem_attributes();
-  if (e == cudaSuccess) e = make_side((int)nu, &f->u);
-  if (e == cudaSuccess) e = make_side((int)nv, &f->v);
+  if (e == cudaSuccess) e = make_side((int)nu, batch * nv, &f->u);
+  if (e == cudaSuccess) e = make_side((int)nv, batch * nu, &f->v);
   const int smax = (int)(2 * kMaxSide * sizeof(float4));
 #define WG_SMEM_ATTR(K, BYTES)                                                                   \
   if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, BYTES)
-  if (!f->u.pairs || !f->v.pairs || f->u.fwd_lines || f->v.fwd_lines) {
+  if (f->u.lines || f->v.lines) {
     WG_SMEM_ATTR((k_fft_lines<448, 2, false, false, false>), smax); WG_SMEM_ATTR((k_fft_lines<448, 2, false, true, false>), smax);
     WG_SMEM_ATTR((k_fft_lines<448, 2, true, false, false>), smax);  WG_SMEM_ATTR((k_fft_lines<448, 2, true, true, false>), smax);
     WG_SMEM_ATTR((k_fft_lines<832, 1, false, false, false>), smax); WG_SMEM_ATTR((k_fft_lines<832, 1, false, true, false>), smax);
@@ -1128,10 +1137,8 @@ cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out) {
 
 void df64_fft_destroy(Df64Fft* f) {
   if (f == nullptr) return;
-  for (SideFft* side : {&f->u, &f->v}) {
+  for (SideFft* side : {&f->u, &f->v})
     if (side->tw) cudaFree(side->tw);
-    if (side->twl) cudaFree(side->twl);
-  }
   delete f;
 }
 
@@ -1205,12 +1212,21 @@ static cudaError_t launch_lines(const FftLine& L, double2* data, int64_t batch, 
   return cudaGetLastError();
 }
 
-static bool on_pairs(const SideFft& f, int fwd) { return f.pairs && !(fwd && f.fwd_lines); }
+// Whether a pass over `lines` lines of a side runs on pairs of lines.  Forward passes of few short lines
+// do not: half as many CTAs then leave SMs idle, each takes longer, and the code of the pair
+// kernels, a stage of its own for every radix and place, comes from L2 or beyond.  Forward transforms of a
+// plan, line by line against in pairs, right after the last one / after 640 MB of other traffic: one plane of
+// 128^2 15.6 / 14.3 against 21.5 / 30.7 us, 512^2 23.6 / 26.6 against 31.8 / 45.1, 896^2 40.3 / 43.0 against
+// 42.0 / 57.3; 1024^2 48.3 / 49.2 against 44.1 / 59.4; planes of 128^2: 11 of them 20.9 / 20.5 against 21.6 /
+// 28.7, 15 of them 23.9 / 22.5 against 21.5 / 30.7; of 256^2, 11: 38.2 / 36.9 against 33.8 / 47.1.
+static bool on_pairs(const SideFft& f, int fwd, int64_t lines) {
+  return f.pairs && !(fwd && f.lines && (f.fwd_lines || lines <= kFewLines));
+}
 
 static cudaError_t launch_side(const SideFft& f, double2* data, int64_t batch, int64_t plane,
                                int lines, int64_t line_stride, int64_t elem_stride, int mode,
                                int fwd, int split, int skip, int lhalf, int shalf, cudaStream_t s) {
-  return on_pairs(f, fwd)
+  return on_pairs(f, fwd, batch * lines)
              ? launch_pairs(f.pl, data, batch, plane, lines, line_stride, elem_stride, fwd, split,
                             skip, lhalf, shalf, s)
              : launch_lines(f.fl, data, batch, plane, lines, line_stride, elem_stride, mode, fwd,
@@ -1258,7 +1274,9 @@ cudaError_t df64_fft_exec(Df64Fft* f, double2* data, int64_t batch, int sign, cu
   // only: complex128 data are converted before a first pass and after a second pass that they run
   const SideFft &first = prune && fwd ? f->u : f->v, &second = prune && fwd ? f->v : f->u;
   const bool in_pairs = fwd ? image_pairs : df64_planes, out_pairs = fwd ? df64_planes : image_pairs;
-  const bool conv_in = !in_pairs && on_pairs(first, fwd), conv_out = !out_pairs && on_pairs(second, fwd);
+  const int64_t of_u = batch * (prune ? 2 * (keep_cols / 2) : f->nv), of_v = batch * f->nu;   // lines of a pass
+  const bool conv_in = !in_pairs && on_pairs(first, fwd, &first == &f->u ? of_u : of_v);
+  const bool conv_out = !out_pairs && on_pairs(second, fwd, &second == &f->u ? of_u : of_v);
   const int mode_in = in_pairs || conv_in ? 2 : 0, mode_out = out_pairs || conv_out ? 2 : 1;
   cudaError_t e;
   auto convert = [&](int back) {

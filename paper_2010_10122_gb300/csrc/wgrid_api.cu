@@ -558,7 +558,7 @@ int wg_plan_create(const double* uvw, const double* freq, int64_t nrows, int64_t
       B = std::max<int64_t>(1, align_batch(B * 3 / 4));
     p->batch = B;
   } else if (use_df64) {
-    cudaError_t e = df64_fft_create(pp.nu, pp.nv, &p->dfft);
+    cudaError_t e = df64_fft_create(pp.nu, pp.nv, B, &p->dfft);
     if (e != cudaSuccess) return fail(set_error(WG_ERR_CUDA, "double-float FFT setup: %s", cudaGetErrorString(e)));
     p->fft_ws = 0;
     while (B > 1 && workspace_layout(p.get(), B, 0).total > budget)
@@ -1153,7 +1153,7 @@ static int fft_util_make(FftUtil& u, int64_t nu, int64_t nv, int64_t batch, int 
     if (precision != WG_F64 || !df64_fft_supported(nu, nv))
       return set_error(WG_ERR_ARG, "double-float FFT needs WG_F64 and sides with factors 2, 3, 5, 7, 11 "
                                    "up to 6400, or 2 or 4 times such a side up to 25600");
-    cudaError_t e = df64_fft_create(nu, nv, &u.d);
+    cudaError_t e = df64_fft_create(nu, nv, batch, &u.d);
     if (e != cudaSuccess) return set_error(WG_ERR_CUDA, "double-float FFT setup: %s", cudaGetErrorString(e));
     return WG_OK;
   }

@@ -77,7 +77,8 @@ int report_error(int code, const char* msg);
 // ---- double-float FFT (fft_df64.cu) -----------------------------------------------------
 struct Df64Fft;
 bool df64_fft_supported(int64_t nu, int64_t nv);
-cudaError_t df64_fft_create(int64_t nu, int64_t nv, Df64Fft** out);
+// batch: most planes of an execution (more are transformed as well)
+cudaError_t df64_fft_create(int64_t nu, int64_t nv, int64_t batch, Df64Fft** out);
 void df64_fft_destroy(Df64Fft* f);
 cudaError_t df64_fft_exec(Df64Fft* f, double2* data, int64_t batch, int sign, cudaStream_t s,
                           int64_t keep_rows = 0, int64_t keep_cols = 0, bool df64_planes = false,
