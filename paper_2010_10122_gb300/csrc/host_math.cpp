@@ -579,6 +579,11 @@ int degrid_shares(double densest, double mean, double least, double ctas, bool f
   return (int)std::max(1.0, std::min({32.0, std::ceil(densest / least), pays}));
 }
 
+MmaLaunches mma_launches(double densest, double mean, double ctas) {
+  if (!(densest > 2.0 * mean + 64.0) || densest < 0.03 * ctas) return kMmaEven;
+  return ctas < 1000.0 + 4.0 * densest ? kMmaDense : kMmaBoth;
+}
+
 int choose_plan(const PlanInput& in, PlanParams& out, char* err, int errlen) {
   auto fail = [&](const char* msg) {
     std::snprintf(err, errlen, "%s", msg);

@@ -149,6 +149,19 @@ double rounding_coefficient(double gain);                              // c(G) o
 // 1.01 with the 7 that densest / least alone would give; on 4000^2 without w 0.25 and 0.50.
 int degrid_shares(double densest, double mean, double least, double ctas, bool f32);
 
+// Launches of FP32 gridding on the tensor cores: one warp per quarter of a tile and plane group, four warps
+// for every quarter, or four for the dense tiles and one for the others, in two launches.  `densest` hits of
+// the fullest quarter against the `mean` over the warps the GPU holds at once, `ctas` tiles x plane groups.
+// Four warps pay where the fullest quarter is the run time: above twice the mean and four groups of 16 more,
+// and above 0.03 ctas, below which going through the tiles takes longer.  For every tile they cost 24 ns a
+// CTA (one CTA of 16 warps on an SM), a second launch 5, and it waits for the first: two launches from
+// 1000 + 4 densest CTAs up.  Fitted to 175 plans timed in all three forms (array and random observations, even
+// and crowded, 256^2 - 4096^2): 1.7 % above the best form on average.  One warp / four / two launches: 2e5
+// visibilities on 2816^2, half of them in 16 tiles: 1.23 / 3.87 / - ms; half of them in one: 4.75 / 3.95 / 2.14;
+// 2.6e6 on a 512^2 grid: 15.4 / 5.1 / 5.4; 2e6 on 8192^2 without w, half in 100 tiles: 1.52 / 2.89 / 1.19.
+enum MmaLaunches { kMmaEven = 1, kMmaDense = 4, kMmaBoth = 5 };
+MmaLaunches mma_launches(double densest, double mean, double ctas);
+
 struct PlanInput {
   int64_t nx, ny;
   double psx, psy;

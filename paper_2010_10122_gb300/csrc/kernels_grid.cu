@@ -1157,11 +1157,9 @@ k_grid_atomic(const Geom g, const __grid_constant__ Coef<R> coef, const IndexVie
 // GB300: 2048^2, 1e6 visibilities, 55 planes of 2816^2 2.46 -> 1.56 ms; 4096^2, 1e7 visibilities 15.0
 // -> 10.7 ms; 8192^2, 5e7 visibilities 117 -> 74 ms; 512^2, 1.2e5 visibilities 0.66 -> 0.17 ms.
 //
-// On small grids the few dense tiles at the grid's origin would be the whole run time: where the
-// densest quarter holds more than twice what a resident warp gets on average (and 64 more, four
-// groups, below which a split costs more than it gives), SPLIT = 4 warps share each quarter, taking
-// turns at the candidates, and their sums are added in a fixed order (the 512^2 case 0.34 -> 0.17 ms;
-// where it is not needed the partial groups cost more than that gives: 8192^2 74 -> 160 ms).
+// On small grids the few dense tiles at the grid's origin would be the whole run time: there SPLIT = 4 warps
+// share each quarter, taking turns at the candidates, and their sums are added in a fixed order (512^2, 1.2e5
+// visibilities: 0.34 -> 0.17 ms), for every tile or in a launch of its own for the dense ones: see mma_launches.
 // ---------------------------------------------------------------------------------------
 constexpr int kMmaTile = 32, kMmaPlanes = 4, kMmaQueue = 256, kMmaPad = 16;
 constexpr int kMmaRow = 48;   // kMmaPad zeros, up to 16 kernel values, zeros
@@ -1203,7 +1201,7 @@ template <int G, int SPLIT>
 __global__ void __launch_bounds__(128 * SPLIT, SPLIT == 1 ? 4 : 1)
 k_grid_mma(const Geom g, const __grid_constant__ Coef<float> coef, const IndexView<float> ix,
            const float2* __restrict__ vis, const float* __restrict__ wgt,
-           float2* __restrict__ planes, int b0, int nb) {
+           float2* __restrict__ planes, int b0, int nb, uint32_t dense) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int T = kMmaTile;
   const int alpha = g.alpha, aw = g.alpha_w;
@@ -1233,6 +1231,8 @@ k_grid_mma(const Geom g, const __grid_constant__ Coef<float> coef, const IndexVi
       total += __shfl_sync(0xffffffffu, at, 2 * s + 1) - lo[s];
     }
   }
+  // tiles of up to `dense` candidates are the SPLIT = 1 launch's, the others the SPLIT = 4 launch's
+  if (__any_sync(0xffffffffu, SPLIT == 1 ? total > dense : total < dense)) return;
   const int64_t pstride = (int64_t)g.nu * g.nv;
   float2* out = planes + (int64_t)(s0 - b0) * pstride + (int64_t)(tu * T + sr0 + gid) * g.nv +
                 tv * T + sc0 + 2 * tig;
@@ -1822,29 +1822,42 @@ static cudaError_t grid_atomic_g(const Geom& g, const Coef<R>& coef, const Index
 template <int G, int SPLIT>
 static cudaError_t grid_mma_split(const Geom& g, const Coef<float>& coef, const IndexView<float>& ix,
                                   const float2* vis, const float* wgt, float2* planes, int b0,
-                                  int nb, cudaStream_t s) {
+                                  int nb, uint32_t dense, cudaStream_t s) {
   const size_t smem = 4 * SPLIT * sizeof(MmaWarp);
   cudaError_t e = cudaFuncSetAttribute(k_grid_mma<G, SPLIT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int64_t ntiles = (int64_t)g.ntu * g.ntv;
   dim3 grid((unsigned)ntiles, (unsigned)((nb + kMmaPlanes - 1) / kMmaPlanes));
-  k_grid_mma<G, SPLIT><<<grid, 128 * SPLIT, smem, s>>>(g, coef, ix, vis, wgt, planes, b0, nb);
+  k_grid_mma<G, SPLIT><<<grid, 128 * SPLIT, smem, s>>>(g, coef, ix, vis, wgt, planes, b0, nb, dense);
   return cudaGetLastError();
+}
+
+// hits of the densest quarter (about half of its tile's visibilities, those whose planes meet the warp's)
+// and their mean over the warps the GPU holds at once (16 on each SM; a visibility meets 2.1 quarters
+// and (alpha + 3) / 4 plane groups)
+static double mma_mean(const Geom& g) {
+  return 2.1 * (double)g.nvis * (g.alpha_w + kMmaPlanes - 1) / kMmaPlanes / (152.0 * 16.0);
+}
+static MmaLaunches mma_form(const Geom& g, int nb) {
+  const double window = std::min(1.0, (double)(g.alpha_w + kMmaPlanes - 1) / g.nw);
+  return mma_launches(0.5 * (double)g.max_tile * window, mma_mean(g),
+                      (double)g.ntu * g.ntv * ((nb + kMmaPlanes - 1) / kMmaPlanes));
 }
 
 template <int G>
 static cudaError_t grid_mma(const Geom& g, const Coef<float>& coef, const IndexView<float>& ix,
                             const float2* vis, const float* wgt, float2* planes, int b0, int nb,
                             cudaStream_t s) {
-  // hits of the densest quarter (about half of its tile's visibilities, those whose planes meet
-  // the warp's) against the mean over the warps the GPU holds at once (16 on each SM; a visibility
-  // meets 2.1 quarters and (alpha + 3) / 4 plane groups)
-  const double window = std::min(1.0, (double)(g.alpha_w + kMmaPlanes - 1) / g.nw);
-  const double densest = 0.5 * (double)g.max_tile * window;
-  const double mean = 2.1 * (double)g.nvis * (g.alpha_w + kMmaPlanes - 1) / kMmaPlanes / (152.0 * 16.0);
-  if (densest > 2.0 * mean + 64.0) return grid_mma_split<G, 4>(g, coef, ix, vis, wgt, planes, b0, nb, s);
-  return grid_mma_split<G, 1>(g, coef, ix, vis, wgt, planes, b0, nb, s);
+  switch (mma_form(g, nb)) {
+    case kMmaEven: return grid_mma_split<G, 1>(g, coef, ix, vis, wgt, planes, b0, nb, 0xffffffffu, s);
+    case kMmaDense: return grid_mma_split<G, 4>(g, coef, ix, vis, wgt, planes, b0, nb, 0, s);
+    default: break;
+  }
+  // the dense tiles first; candidates: those of a tile and its three sources, four times the hits of a quarter
+  const uint32_t dense = (uint32_t)(0.25 * (2.0 * mma_mean(g) + 64.0));
+  const cudaError_t e = grid_mma_split<G, 4>(g, coef, ix, vis, wgt, planes, b0, nb, dense + 1, s);
+  return e != cudaSuccess ? e : grid_mma_split<G, 1>(g, coef, ix, vis, wgt, planes, b0, nb, dense, s);
 }
 
 static cudaError_t grid_band(const Geom& g, const Coef<float>& coef, const IndexView<float>& ix,
@@ -1883,6 +1896,14 @@ static int grid_variant_of(const Geom& g) {
   if (g.grid_variant != 0) return g.grid_variant;
   return sizeof(R) == 8 ? 2 : (g.tile == kMmaTile && g.gain <= kMmaMaxGain ? kVariantMma : 1);
 }
+
+// kernels that one launch_grid starts
+template <typename R>
+int grid_kernels(const Geom& g, int nb) {
+  return sizeof(R) == 4 && grid_variant_of<R>(g) == kVariantMma && mma_form(g, nb) == kMmaBoth ? 2 : 1;
+}
+template int grid_kernels<float>(const Geom&, int);
+template int grid_kernels<double>(const Geom&, int);
 
 template <typename R, int G>
 static cudaError_t grid_g(const Geom& g, const Coef<R>& coef, const IndexView<R>& ix,

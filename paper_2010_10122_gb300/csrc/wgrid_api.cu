@@ -871,7 +871,7 @@ static int grid_impl(wg_plan* p, const typename C2<R>::T* vis, const R* wgt, R* 
   IndexView<R> ix{p->off, p->idx, p->meta, (const Z4<R>*)p->z, (const typename C2<R>::T*)p->ph, wts};
   const Coef<R>& coef = *reinterpret_cast<const Coef<R>*>(sizeof(R) == 4 ? (const void*)&p->coef_f
                                                                          : (const void*)&p->coef_d);
-  int64_t nbatches = 0;
+  int64_t nbatches = 0, ngrid = 0;
   do {
     cudaError_t e = cudaSuccess;
     if (p->compact) {   // the records of the compact index, recomputed into the workspace
@@ -903,6 +903,7 @@ static int grid_impl(wg_plan* p, const typename C2<R>::T* vis, const R* wgt, R* 
       int nb = (int)std::min<int64_t>(p->batch, g.nw - b0);
       e = launch_grid<R>(g, coef, ix, vgrid, wgt, planes, (int)b0, nb, s);
       if (e != cudaSuccess) { rc = set_error(WG_ERR_CUDA, "grid: %s", cudaGetErrorString(e)); break; }
+      ngrid += grid_kernels<R>(g, nb);
       tm.mark(ST_GRID);
       if ((rc = run_fft(p, nb, planes, fftw, CUFFT_INVERSE, s)) != WG_OK) break;
       tm.mark(ST_FFT);
@@ -929,7 +930,7 @@ static int grid_impl(wg_plan* p, const typename C2<R>::T* vis, const R* wgt, R* 
     tm.finish(stats);
     stats->n_batches = nbatches; stats->n_planes = g.nw; stats->workspace_bytes = w.total;
     // grid + accumulate per batch, weights; the double-float FFT's two passes per batch
-    stats->n_kernels = 2 * nbatches + (wts_call != nullptr) +
+    stats->n_kernels = ngrid + nbatches + (wts_call != nullptr) +
                        (p->dfft != nullptr || p->ffft != nullptr ? 2 * nbatches : 0) +
                        (g.df64_planes ? 1 : 0) + (p->compact ? 1 : 0);
     stats->n_fft_calls = nbatches;

@@ -145,6 +145,8 @@ cudaError_t launch_weights(const Geom& g, const Coef<R>& coef, const IndexView<R
                            int64_t nvis_idx, R* wts, cudaStream_t s);
 // planes per degrid CTA (shared-memory budget); plane batches are multiples of it
 template <typename R>
+int grid_kernels(const Geom& g, int nb);
+template <typename R>
 int degrid_subbatch(const Geom& g);
 // partial sums: slot (sub-batch id - first sub-batch id of the visibility) x visibility position
 template <typename R>

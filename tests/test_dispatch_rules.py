@@ -12,6 +12,7 @@ WRAPPER = r"""
 extern "C" int shares(double densest, double mean, double least, double ctas, int f32) {
   return wg::degrid_shares(densest, mean, least, ctas, f32 != 0);
 }
+extern "C" int launches(double densest, double mean, double ctas) { return wg::mma_launches(densest, mean, ctas); }
 """
 
 
@@ -24,6 +25,7 @@ def rules(tmp_path_factory):
                            _build.CSRC + "/host_math.cpp", _build.CSRC + "/kernel_design.cpp", "-o", so])
     lib = ctypes.CDLL(so)
     lib.shares.argtypes = [ctypes.c_double] * 4 + [ctypes.c_int]
+    lib.launches.argtypes = [ctypes.c_double] * 3
     return lib
 
 
@@ -36,3 +38,12 @@ def rules(tmp_path_factory):
     (2386.8, 2960.3, 1472, 12150, 1, 1, 1), (2848.4, 4659.8, 2304, 20480, 0, 1, 1), (0.0, 0.0, 128, 1, 1, 1, 1)])
 def test_degrid_shares(rules, densest, mean, least, ctas, f32, lo, hi):
     assert lo <= rules.shares(densest, mean, least, ctas, f32) <= hi
+
+
+@pytest.mark.parametrize("densest,mean,ctas,form", [
+    (1518, 195, 1024, 4), (14855, 389, 5120, 4),                 # dense small grids: four warps everywhere
+    (538, 1727, 4096, 1), (170, 17, 26244, 1), (487, 47, 309760, 1),   # even, or too many tiles: one warp
+    (2556, 173, 15625, 5), (5935, 475, 77440, 5), (0, 0, 1, 1)])       # crowded large grids: two launches
+def test_mma_launches(rules, densest, mean, ctas, form):
+    got = rules.launches(densest, mean, ctas)
+    assert got == form
