@@ -773,35 +773,37 @@ cudaError_t launch_grid_vis_dd(const IndexView<double>& ix, const double2* vis, 
 // 8 planes take 11.4, and whole-warp 4 x 8 cells 11.4 where half-warps take 10.6 (3456^2 grid, 1e6
 // visibilities, alpha = 15; the plane-owner kernel 19.6).
 //
-// Shapes, by template (W warps x SPLIT):
-//  * <8, 1>: 16 x 16 cells, every warp walks the whole chunk.
-//  * <2, 4>: 8 x 8 cells, four sets of two warps, each taking every fourth visibility, their sums
+// Shapes, by template (W warps x SPLIT, PG planes):
+//  * <8, 1, 8>: 16 x 16 cells, every warp walks the whole chunk.
+//  * <2, 4, 8>: 8 x 8 cells, four sets of two warps, each taking every fourth visibility, their sums
 //    added in order at the end: for plans whose densest tile would be the run time.
+//  * <8, 1, 2>: the first with two planes, for grids without w: 40 registers, six CTAs per SM (2560^2, 20 000
+//    visibilities, alpha = 6: 104 us with eight planes, 78 with two, the plane-owner kernel 82).
 constexpr int kCellsPlanes = 8;
 template <int W>
 struct CellsTile {   // cells and visibilities per set of a CTA
   static constexpr int rows = W == 8 ? 16 : 8, cols = W >= 4 ? 16 : 8;
   static constexpr int vis = W == 8 ? 64 : 32;
 };
-template <int W, int SPLIT>
+template <int W, int SPLIT, int PG>
 struct CellsStage {
   static constexpr int kChunk = CellsTile<W>::vis * SPLIT;
   // row kChunk: no visibility
   float2 wu[kChunk + 1][kMaxG], wv[kChunk + 1][kMaxG];   // kernel values as pairs
-  float4 dq[kChunk + 1][kCellsPlanes + 1];   // data x w kernel value by plane: re hi, im hi, re lo, im lo
+  float4 dq[kChunk + 1][PG + 1];   // data x w kernel value by plane: re hi, im hi, re lo, im lo
   int head[kChunk + 1];   // footprint origin (row + 64, column + 64 << 8), plane pairs met << 16; or 0
   int cum[4], first[4];   // visibilities before each source tile; index position minus that
 };
 
-template <int W, int SPLIT>
-__global__ void __launch_bounds__(32 * W * SPLIT, 32 / (W * SPLIT))
+template <int W, int SPLIT, int PG>
+__global__ void __launch_bounds__(32 * W * SPLIT, (PG == 2 ? 48 : 32) / (W * SPLIT))
 k_grid_cells_dd(const Geom g, const __grid_constant__ Coef<double> coef, const IndexView<double> ix,
                 const float4* __restrict__ vis, float4* __restrict__ planes, int b0, int nb) {
   extern __shared__ __align__(16) unsigned char smem[];
   double* sc = reinterpret_cast<double*>(smem);
-  using Stage = CellsStage<W, SPLIT>;
+  using Stage = CellsStage<W, SPLIT, PG>;
   Stage& sm = *reinterpret_cast<Stage*>(smem + (kMaxDeg + 1) * kMaxG * sizeof(double));
-  constexpr int TR = CellsTile<W>::rows, TC = CellsTile<W>::cols, G = 16, PG = kCellsPlanes, N = 32 * W;
+  constexpr int TR = CellsTile<W>::rows, TC = CellsTile<W>::cols, G = 16, N = 32 * W;
   const int alpha = g.alpha, aw = g.alpha_w;
   const int nqv = g.nv / TC, nqu = g.nu / TR, peru = g.tile / TR, perv = g.tile / TC;
   const int tr = blockIdx.x / nqv, qv = blockIdx.x - tr * nqv;
@@ -835,7 +837,7 @@ k_grid_cells_dd(const Geom g, const __grid_constant__ Coef<double> coef, const I
     }
     if (lane < 4) { sm.cum[lane] = (int)c; sm.first[lane] = (int)(lo - (c - n)); }
   }
-  if (threadIdx.x < kCellsPlanes) sm.dq[Stage::kChunk][threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (threadIdx.x < PG) sm.dq[Stage::kChunk][threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (threadIdx.x == 0) sm.head[Stage::kChunk] = 0;
   f2 ah[PG], al[PG];   // this lane's cell: (re, im) high parts, low parts
 #pragma unroll
@@ -1741,16 +1743,16 @@ static cudaError_t degrid_g(const Geom& g, const Coef<R>& coef, const IndexView<
   return cudaGetLastError();
 }
 
-template <int W, int SPLIT>
+template <int W, int SPLIT, int PG>
 static cudaError_t grid_cells_split(const Geom& g, const Coef<double>& coef, const IndexView<double>& ix,
                                     const float4* vis, float4* planes, int b0, int nb, cudaStream_t s) {
-  const size_t smem = coef_bytes<double>() + sizeof(CellsStage<W, SPLIT>);
-  cudaError_t e = cudaFuncSetAttribute(k_grid_cells_dd<W, SPLIT>,
+  const size_t smem = coef_bytes<double>() + sizeof(CellsStage<W, SPLIT, PG>);
+  cudaError_t e = cudaFuncSetAttribute(k_grid_cells_dd<W, SPLIT, PG>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)((int64_t)(g.nu / CellsTile<W>::rows) * (g.nv / CellsTile<W>::cols)),
-            (unsigned)((nb + kCellsPlanes - 1) / kCellsPlanes));
-  k_grid_cells_dd<W, SPLIT><<<grid, 32 * W * SPLIT, smem, s>>>(g, coef, ix, vis, planes, b0, nb);
+            (unsigned)((nb + PG - 1) / PG));
+  k_grid_cells_dd<W, SPLIT, PG><<<grid, 32 * W * SPLIT, smem, s>>>(g, coef, ix, vis, planes, b0, nb);
   return cudaGetLastError();
 }
 
@@ -1765,8 +1767,9 @@ static cudaError_t grid_cells_dd(const Geom& g, const Coef<double>& coef, const 
   const double densest = g.max_tile * std::min(1.0, groups / g.nw) *
                          std::min(1.0, reach / ((double)g.tile * g.tile));
   const double mean = g.nvis * groups / kCellsPlanes * reach / 32 / (152.0 * 32.0);
-  if (densest > 1.2 * mean + 32.0) return grid_cells_split<2, 4>(g, coef, ix, vis, planes, b0, nb, s);
-  return grid_cells_split<8, 1>(g, coef, ix, vis, planes, b0, nb, s);
+  if (densest > 1.2 * mean + 32.0) return grid_cells_split<2, 4, kCellsPlanes>(g, coef, ix, vis, planes, b0, nb, s);
+  if (g.nw <= 2) return grid_cells_split<8, 1, 2>(g, coef, ix, vis, planes, b0, nb, s);
+  return grid_cells_split<8, 1, kCellsPlanes>(g, coef, ix, vis, planes, b0, nb, s);
 }
 
 template <typename R, int G>
