@@ -1897,7 +1897,13 @@ static int grid_variant_of(const Geom& g) {
   const bool band_ok = sizeof(R) == 4 && g.alpha <= 8 && g.tile == kBandTile;
   if (g.grid_variant == 3) return band_ok ? 3 : 1;
   if (g.grid_variant != 0) return g.grid_variant;
-  return sizeof(R) == 8 ? 2 : (g.tile == kMmaTile && g.gain <= kMmaMaxGain ? kVariantMma : 1);
+  if (sizeof(R) == 8) return 2;
+  // the narrowest kernels on a single plane with many visibilities and no dominating tile: half of a group's
+  // lanes and three of a warp's four planes idle (1e6 visibilities on 1024 x 768, alpha = 4: 257 us by atomics,
+  // 296 by the tensor cores; on 2816^2 219 and 236; 2e6 on 2048^2 356 and 399, on 1024^2 442 and 427; on 672 x
+  // 512, where the densest tile is the run time, 405 and 224; 2e4 on 1024 x 768 23 and 19)
+  const bool thin = g.alpha <= 4 && g.nw == 1 && mma_mean(g) > 400.0 && mma_form(g, 1) == kMmaEven;
+  return g.tile == kMmaTile && g.gain <= kMmaMaxGain && !thin ? kVariantMma : 1;
 }
 
 // kernels that one launch_grid starts
