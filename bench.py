@@ -238,10 +238,8 @@ DF64_BUTTERFLY = {2: 44, 3: 160, 4: 176, 5: 464, 7: 870, 8: 600, 11: 2050}
 
 def df64_radices(n):
     """Radix plan of a double-float line transform (8s and 4s for the power of two, a single 2
-    only for n = 2 x odd, then 5, 3, 7, 11) -- the plan of the library's line kernels.  The
-    accounting counts this transform for every side: the kernels on pairs of lines take other
-    radices, up to 12, with fewer operations (3456 points as 4 x 864, radices 8 6 6 3: 430 per
-    element where this count has 460)."""
+    only for n = 2 x odd, then 5, 3, 7, 11) -- the plan of the library's kernels of one line per
+    CTA or cluster."""
     m, p2 = n, 0
     while m % 2 == 0:
         m //= 2
@@ -303,12 +301,27 @@ def df64_line_ops(n):
     return (n // S) * (DF64_BUTTERFLY[S] + 38 * (S - 1)) + S * df64_part_ops(n // S)
 
 
-def df64_fft_kernel(n):
-    """The kernel a double-float line of n points runs on: pairs of lines, except between 3072 and
-    4096 points with a factor 11 or 35 (one line per CTA or cluster)."""
-    if 3072 < n < 4096 and (n % 11 == 0 or n % 35 == 0):
-        return "k_fft_lines_cluster" if df64_line_split(n) > 1 else "k_fft_lines"
-    return "k_fft_pairs"
+# The same count for the kernels on pairs of lines (paper_2010_10122_gb300/csrc/fft_engine.cuh), per line:
+# radix 3 with a half-and-subtract of 13, the odd primes with one product less per output pair, 6, 10
+# and 12 by coprime factors, 9 as 3 x 3 with four twiddle products
+PAIR_BUTTERFLY = {2: 44, 3: 150, 4: 176, 5: 428, 6: 432, 7: 822, 8: 600, 9: 1052, 10: 1076, 11: 1970,
+                  12: 1128}
+
+
+def df64_pass(n, direction):
+    """(kernel, FP32 instructions of one line) of a double-float pass over lines of n points, as the library
+    plans it."""
+    from paper_2010_10122_gb300 import wgrid
+    pairs, parts, radices = wgrid.fft_df64_line(n, forward=direction == "degrid")
+    if not pairs:
+        return ("k_fft_lines_cluster" if parts > 1 else "k_fft_lines"), df64_line_ops(n)
+    m = n // parts
+    ops = m * (PAIR_BUTTERFLY[parts] + 38 * (parts - 1)) if parts > 1 else 0
+    ns = 1
+    for r in radices:
+        ops += parts * (m // r) * (PAIR_BUTTERFLY[r] + (38 * (r - 1) if ns > 1 else 0))
+        ns *= r
+    return "k_fft_pairs", ops
 
 
 # DRAM bytes the double-float FFT moved per algorithmic byte (one 16-byte read and one 16-byte
@@ -858,11 +871,11 @@ def main():
         # double-float plane FFT: FP32-ALU (issue) bound; work = its FP32 arithmetic
         # instructions; one pass over the ny image columns (length nu), one over all nu rows
         nu, nv, nw = info_d["nu"], info_d["nv"], info_d["nw"]
-        ops = nw * (obs.npix_y * df64_line_ops(nu) + nu * df64_line_ops(nv))
+        (kname, ops_u), (_, ops_v) = df64_pass(nu, dir_d), df64_pass(nv, dir_d)
+        ops = nw * (obs.npix_y * ops_u + nu * ops_v)
         peak = 152 * 128 * 2.07e9   # SMs x FP32 lanes x max SM clock, one instruction per lane
         ach = ops / (stage_ms[dom] * 1e-3)
         abytes = nw * df64_fft_bytes(obs.npix_x, obs.npix_y, nu, nv, dir_d)
-        kname = df64_fft_kernel(nu)
         roof = {"bound": "alu", "kernel": f"{kname} (double-float plane FFT, row + column pass)",
                 "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s", "frac": ach / peak,
                 "traffic": DF64_DRAM_PER_ALGORITHMIC_BYTE * abytes,

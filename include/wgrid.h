@@ -88,24 +88,26 @@ typedef struct wg_options {
   double force_sigma;      /* >0: only consider this oversampling factor (tests) */
   int tile;                /* uv tile side in cells (16 or 32; 0 = automatic) */
   int grid_variant;        /* gridding accumulation: 0 = automatic (WG_F32: tensor cores with
-                              32-cell tiles and a rounding_gain up to 40, deterministic,
-                              else shared-memory atomics; WG_F64:
+                              32-cell tiles and a rounding_gain up to 40, deterministic, but
+                              for alpha = 4 without w where no tile is much denser than the
+                              others; else shared-memory atomics; WG_F64:
                               plane-owner warps), 1 = shared-memory atomics, 2 =
                               plane-owner warps (deterministic), 3 = row-band owner warps
                               (WG_F32, alpha <= 8, 32-cell tiles: each warp owns 4 rows of the
                               tile in every plane; deterministic; other plans fall back to 1);
                               WG_F64 plans with the double-float FFT always keep the sums of
                               their double-float pairs in registers (each lane owns a cell in
-                              8 planes; deterministic) */
+                              8 planes, 2 without w; deterministic) */
   int fft_impl;            /* plane FFTs: 0 = automatic (WG_F32: cuFFT C2C; WG_F64: the
                               cheaper of 2 and 3 whose predicted error fits epsilon),
                               1 = cuFFT 2-D, 2 = the library's double-float FFT (WG_F64 only,
                               grid sides up to 6400 with prime factors 2, 3, 5, 7, 11, and
-                              sides up to 25600 that are 2 or 4 times such a side; two lines
-                              at a time, above 2048 points on thread-block clusters); its ~5e-15 rounding is amplified by the
-                              1 / psi correction, so the planner may raise sigma for it; the
-                              uv planes are then kept as double-float pairs and (de)gridded in
-                              pair arithmetic),
+                              sides up to 25600 that are 2 or 4 times such a side; most sides
+                              up to 16384 two lines at a time, above 2048 points on thread-block
+                              clusters, see wg_fft_df64_line; its ~5e-15 rounding is amplified
+                              by the 1 / psi correction, so the planner may raise sigma for it;
+                              the uv planes are then kept as double-float pairs and (de)gridded
+                              in pair arithmetic),
                               3 = pruned cuFFT Z2Z (WG_F64 only: 1-D passes that skip the
                               plane rows outside the image),
                               4 = the library's FP32 FFT (WG_F32 only, never chosen
@@ -325,6 +327,12 @@ int wg_kernel_search(int alpha, double sigma, double beta0, double mu0, double* 
 int wg_plan_params(int64_t npix_x, int64_t npix_y, double pixsize_x, double pixsize_y,
                    double epsilon, int precision, const wg_options* opt, double umax,
                    double vmax, double wmin, double wmax, int64_t nvis, wg_plan_info* info);
+
+/* Kernel of the double-float FFT (fft_impl 2) for a pass over many lines of n points, forward (degrid) or
+ * inverse (grid): *pairs 1 = two lines at a time, 0 = one; *parts CTAs per line (a cluster above 1); the
+ * *nradix radices (at most 24) that transform one CTA's n / *parts points.  Returns WG_ERR_ARG for a side
+ * that the transform does not support. */
+int wg_fft_df64_line(int64_t n, int forward, int* pairs, int* parts, int* nradix, int* radix);
 
 /* Planner calibration: time the batched 2-D FFT of `batch` n x n planes on the current device,
  * `reps` executions after one warm-up, and return the mean time per plane in milliseconds.

@@ -1080,16 +1080,21 @@ static cudaError_t line_table(int nline, FftLine* L, std::vector<float4>* table)
   return cudaSuccess;
 }
 
+// sides of the radices 2 and 5 only, which pairs take in four stages with idle lanes: forward
+// and inverse at the pairs' speed against the lines', on square sides with pruning: 640 0.92 /
+// 1.65, 800 0.98 / 1.44, 1280 1.02 / 1.28, 1600 0.92 / 1.10 (other sides from 0.97 up: 128; 1152
+// 1.03 / 1.40, 960 and up)
+static bool forward_by_lines(const PairLine& pl) {
+  const int n = pl.n;
+  return pl.S == 1 && n >= 640 && n % 5 == 0 && n % 3 && n % 7 && n % 11;
+}
+
 static cudaError_t make_side(int n, int64_t most_lines, SideFft* f) {
   f->pairs = pair_plan(n, &f->pl) && pair_cluster_fits(f->pl);
   std::vector<float4> table;
   size_t pair_split = 0, line = 0;
   cudaError_t e = cudaSuccess;
-  // sides of the radices 2 and 5 only, which pairs take in four stages with idle lanes: forward
-  // and inverse at the pairs' speed against the lines', on square sides with pruning: 640 0.92 /
-  // 1.65, 800 0.98 / 1.44, 1280 1.02 / 1.28, 1600 0.92 / 1.10 (other sides from 0.97 up: 128; 1152
-  // 1.03 / 1.40, 960 and up)
-  f->fwd_lines = f->pairs && f->pl.S == 1 && n >= 640 && n % 5 == 0 && n % 3 && n % 7 && n % 11;
+  f->fwd_lines = f->pairs && forward_by_lines(f->pl);
   f->lines = !f->pairs || f->fwd_lines || (n <= kFewLines && most_lines <= 2 * kFewLines);   // see on_pairs
   if (f->pairs) pair_split = pair_table(&f->pl, &table);
   if (f->lines) {
@@ -1103,6 +1108,22 @@ static cudaError_t make_side(int n, int64_t most_lines, SideFft* f) {
   f->fl.tw = f->tw + line;
   f->fl.tw2 = f->fl.split > 1 ? f->fl.tw + f->fl.n : nullptr;
   return e;
+}
+
+int df64_fft_line(int64_t n, bool forward, bool* pairs, int* parts, int* radix) {
+  if (!df64_side_ok(n)) return 0;
+  PairLine pl;
+  *pairs = pair_plan((int)n, &pl) && !(forward && forward_by_lines(pl));
+  if (*pairs) {
+    *parts = pl.S;
+    std::copy(pl.radix, pl.radix + pl.nst, radix);
+    return pl.nst;
+  }
+  Df64LinePlan lp;
+  *parts = df64_line_split(n);
+  df64_line_plan(n / *parts, &lp);
+  std::copy(lp.radix, lp.radix + lp.nst, radix);
+  return lp.nst;
 }
 
 cudaError_t df64_fft_create(int64_t nu, int64_t nv, int64_t batch, Df64Fft** out) {

@@ -1209,6 +1209,16 @@ int wg_fft2d(void* data, int64_t nu, int64_t nv, int64_t batch, int precision, i
   return WG_OK;
 }
 
+int wg_fft_df64_line(int64_t n, int forward, int* pairs, int* parts, int* nradix, int* radix) {
+  if (pairs == nullptr || parts == nullptr || nradix == nullptr || radix == nullptr)
+    return set_error(WG_ERR_ARG, "NULL argument");
+  bool p = false;
+  *nradix = df64_fft_line(n, forward != 0, &p, parts, radix);
+  if (*nradix == 0) return set_error(WG_ERR_ARG, "the double-float FFT does not support a side of %lld", (long long)n);
+  *pairs = p ? 1 : 0;
+  return WG_OK;
+}
+
 int wg_fft_f32_tune(int cols, int max_points, int per_thread) {
   if (f32_fft_tune(cols, max_points, per_thread) != 0)
     return set_error(WG_ERR_ARG, "wg_fft_f32_tune: cols 1, 2, 4 or 8; max_points 64 .. 12800; "

@@ -77,6 +77,9 @@ int report_error(int code, const char* msg);
 // ---- double-float FFT (fft_df64.cu) -----------------------------------------------------
 struct Df64Fft;
 bool df64_fft_supported(int64_t nu, int64_t nv);
+// Kernel of a pass over many lines of a side: pairs of lines or one, CTAs per line, radices of a CTA's
+// part (at most 24); returns their number, 0 for a side that is not supported.  Host only.
+int df64_fft_line(int64_t n, bool forward, bool* pairs, int* parts, int* radix);
 // batch: most planes of an execution (more are transformed as well)
 cudaError_t df64_fft_create(int64_t nu, int64_t nv, int64_t batch, Df64Fft** out);
 void df64_fft_destroy(Df64Fft* f);

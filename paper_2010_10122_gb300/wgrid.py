@@ -103,6 +103,7 @@ SIGNATURES = {
                             _I64, ctypes.POINTER(PlanInfo)]),
     "wg_fft_time": (_I, [_I64, _I, _I64, _I, _I, ctypes.POINTER(_D)]),
     "wg_fft2d": (_I, [_VP, _I64, _I64, _I64, _I, _I, _I, _VP]),
+    "wg_fft_df64_line": (_I, [_I64, _I] + [ctypes.POINTER(_I)] * 4),
     "wg_fma_peak": (_I, [_I, ctypes.POINTER(_D)]),
     "wg_fft_f32_tune": (_I, [_I, _I, _I]),
     "wg_version": (ctypes.c_char_p, []),
@@ -439,6 +440,15 @@ def plan_params(npix_x, npix_y, pixsize_x, pixsize_y, epsilon, precision="f32", 
                                 float(epsilon), _prec(precision), ctypes.byref(o), float(umax),
                                 float(vmax), float(wmin), float(wmax), int(nvis), ctypes.byref(inf)))
     return inf.as_dict()
+
+
+def fft_df64_line(n, forward=True):
+    """(pairs, parts, radices) of the double-float FFT's kernel for passes over lines of n points
+    (wg_fft_df64_line)."""
+    pairs, parts, m, radix = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), (ctypes.c_int * 24)()
+    _check(lib().wg_fft_df64_line(int(n), int(bool(forward)), ctypes.byref(pairs), ctypes.byref(parts),
+                                  ctypes.byref(m), radix))
+    return bool(pairs.value), parts.value, list(radix[:m.value])
 
 
 def fft_time(n, precision="f32", batch=1, reps=3, impl=1) -> float:
