@@ -454,7 +454,10 @@ double rounding_coefficient(double gain) { return 0.065 * (1.0 + gain / 2000.0);
 
 // Measured plane-transform times on GB300, written by calibrate_fft.py: batched cuFFT 2-D C2C
 // and Z2Z, the library's double-float FFT and its FP32 FFT (0 where not measured or not
-// supported), full (unpruned) transforms.
+// supported), full (unpruned) transforms.  The double-float column is that of the kernels of one line
+// per CTA: the kernels on pairs of lines take 0.55 - 1 of it (4096^2 0.73 -> 0.50 ms forward).  It is kept
+// because it chooses grids and FFT kinds, and with them the results; FP64 plans may therefore be
+// somewhat larger or smaller than the cheapest one.
 struct FftRow {
   int64_t n;
   double ms32, ms64, msdf, msf32;
@@ -491,8 +494,8 @@ static double fft_ms_square(int64_t n, int kind, int prec) {
 // pruned kinds transform only the image lines in one of their two passes.  Z2Z: half the work
 // scales with the image fraction.  Double-float FFT: its pruned column pass (the slower pass
 // per line) and the pruned loads / stores of its row pass leave 0.15 + 0.85 x the image
-// fraction of the full transform (measured on GB300: 0.542 ms for a 3456^2 plane with a 2048^2
-// image, against 0.828 ms for the full transform).
+// fraction of the full transform (measured with one line per CTA: 0.542 ms for a 3456^2 plane with a
+// 2048^2 image, against 0.828 ms for the full transform).
 static double fft_ms_cells(int64_t nu, int64_t nv, double cu, double cv, int kind, int64_t nx, int64_t ny) {
   double full = 0.5 * (cu + cv) * (double)nu * nv;
   // image fraction of a side, the geometric mean over the two (square planes: nx / nu); a single
@@ -534,9 +537,11 @@ static std::vector<int64_t> size_candidates(int64_t nmin, int64_t mult, int kind
 // per cell and the w-screen phase per image pixel; per visibility the (de)gridding work,
 // alpha planes x alpha rows x the lanes of the visibility's group (G = 4, 8 or 16 >= alpha;
 // the FP64 gridding kernel spreads its lanes over the alpha^2 cells instead, so FP64 counts
-// the mean of G and alpha).  The per-cell / per-pixel / per-visibility constants are measured
-// stage times of this library on GB300 (2048^2 image, 1e6 visibilities, alpha = G = 8 in FP32
-// and 16 in FP64) divided by the units processed.
+// the mean of G and alpha).  The per-cell / per-pixel / per-visibility constants are stage times measured
+// on GB300 (2048^2 image, 1e6 visibilities, alpha = G = 8 in FP32 and 16 in FP64) divided by the units
+// processed, with gridding by shared-memory atomics (FP32) and plane-owner warps (FP64): the
+// tensor cores and register accumulators take 0.6 and 0.55 of that.  Kept for the same reason as the
+// table above.
 static double plan_cost(int prec, int kind, int64_t nu, int64_t nv, int64_t nw, int alpha,
                         int64_t nvis, int64_t nx, int64_t ny) {
   double cells = (double)nu * nv;

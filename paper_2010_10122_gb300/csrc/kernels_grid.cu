@@ -157,7 +157,7 @@ __device__ __forceinline__ void degrid_rows(const Geom& g, int tu, int tv, int p
 // Bound by the staged bytes from L2 (half of the time of double-float planes on 16-cell tiles, where
 // the halo makes 3.6 times the tile's cells) and then by the latency of the footprint sums.  So the
 // index ranges of all planes come in one load, rows are copied without a division per cell, the
-// next visibility's index entry is loaded ahead, and dense tiles go to several CTAs (see degrid_g).
+// next visibility's index entry is loaded ahead, and dense tiles go to several CTAs (see degrid_shares).
 // Measured before and after, FP32: 1e6 visibilities on a 2048^2 image, alpha = 8, 0.69 -> 0.62 ms; 1e7
 // on 4096^2 4.10 -> 3.90; with a tenth of 8e5 visibilities in one tile, alpha = 6, 3.15 -> 0.63.  (Real
 // and imaginary part packed in one FMA: 0.74 / 0.66 / 0.74 ms with one / two / four planes at once.)
@@ -503,7 +503,7 @@ __global__ void k_degrid_finalize(const Geom g, const IndexView<R> ix,
 }
 
 // ---------------------------------------------------------------------------------------
-// grid, plane-owner variant (default for FP64)
+// grid, plane-owner variant (FP64 planes of plans with cuFFT; FP32 on request)
 //
 // CTA = (uv tile, sub-batch of bs planes).  Warp w owns planes w, w + 8, ... of the
 // sub-batch: it alone updates their T x T accumulators, so the updates are plain shared-memory
@@ -566,7 +566,8 @@ __device__ __forceinline__ void owner_add(const GridStage<R, G>* __restrict__ st
     wt[m] = ok ? stg->wt[v][c] : (R)0;
     off[m] = ok ? (fp.ru + i) * pitch + fp.rv + j : dummy;
   }
-  // loads, arithmetic and stores in separate sweeps (see owner_add_dd)
+  // loads, arithmetic and stores in separate sweeps: the cells of one lane are distinct, but the compiler
+  // cannot see that, and interleaved loads and stores would serialise the MC update chains
   for (int pl = p1; pl < phi; pl += kOwnerWarps) {
     const CT dq = stg->dq[v][pl + qoff];
     CT* base = acc + pl * plane_elems;
@@ -971,7 +972,7 @@ k_grid_cells_dd(const Geom g, const __grid_constant__ Coef<double> coef, const I
 }
 
 // ---------------------------------------------------------------------------------------
-// grid, shared-atomic variant (default for FP32)
+// grid, shared-atomic variant (FP32 plans that do not take the tensor cores, see grid_variant_of)
 //
 // CTA = (uv tile, sub-batch of planes), owning the T x T cells of those planes as separate real
 // and imaginary accumulators in shared memory.  A warp handles one visibility at a time: lane
@@ -1128,22 +1129,25 @@ k_grid_atomic(const Geom g, const __grid_constant__ Coef<R> coef, const IndexVie
 }
 
 // ---------------------------------------------------------------------------------------
-// grid on the tensor cores (default for FP32 with 32-cell tiles)
+// grid on the tensor cores (automatic for most FP32 plans with 32-cell tiles, see grid_variant_of)
 //
 // Gridding visibilities onto 16 x 16 cells of a plane is a matrix product over the visibilities k:
 // cells[i][j] += sum_k wu_k[i] (wv_k[j] ww_k d_k), 16 rows against 16 columns x (re, im), and one
 // mma.m16n8k16 adds 16 visibilities to 16 x 8 cells.  (mma.sync, not tcgen05: the operands are
-// made in registers, 16 visibilities at a time for 16 x 16 cells, and the tensor pipe is at 16 %.)
-// The shared-memory atomics of k_grid_atomic execute as compare-and-swap loops: about 1050 warp
-// instructions per visibility (alpha 6, 1.6e6 visibilities on 42 planes of 2048^2) against 430 here.
+// made in registers, 16 visibilities at a time for 16 x 16 cells, and the tensor pipe is active 16 % of the
+// time with alpha 6, 26 % with alpha 8.)  The shared-memory atomics of k_grid_atomic execute as
+// compare-and-swap loops: about 1050 warp instructions per visibility (alpha 6, 1.6e6 visibilities on 42 planes of
+// 2048^2) against 430 here; 616 with alpha 8 (5e5 visibilities on 33 planes of 1408^2).
 //
-// FP32 accuracy is kept: each factor is cut exactly into three bf16 parts (8 + 8 + 8 significant
-// bits; groups of products with the w kernel below 2^-63 are summed in FP32 instead) and all products of parts down to 2^-24 are summed, the leading ones 8 visibilities at a
-// time and the other seven over 16, each from zero, and added to FP32 accumulators with
-// round-to-nearest (the tensor core drops what lies 24 bits below its largest addend and rounds
-// towards zero, so nothing is carried on in it).  Rounding error of the gridded image against an
-// FP64 plan with the same kernel and grid, ten plans of 200^2 - 1024^2 and both narrow and wide
-// (e^(3 N(0,1))) data: 2.0 - 5.2e-7, 0.85 - 0.99 times the atomics'.
+// FP32 accuracy is kept: each factor is cut exactly into three bf16 parts (8 + 8 + 8 significant bits; planes
+// of 16 visibilities whose data times w kernel all lie below 2^-63 are summed in FP32 instead, because the parts
+// would reach into the bf16 subnormals), and all products of parts down to 2^-24 are summed, the leading ones
+// 8 visibilities at a time and the other seven over 16, each from zero, and added to FP32 accumulators with
+// round-to-nearest (the tensor core drops what lies 24 bits below its largest addend and rounds towards
+// zero, so nothing is carried on in it).  Rounding error of the gridded image against an FP64 plan with
+// the same kernel and grid, ten plans of 200^2 - 1024^2 and both narrow and wide (e^(3 N(0,1))) data: 2.0 -
+// 5.2e-7, 0.85 - 0.99 times the atomics'; on dense cells, where the atomics add more often, less (see
+// kMmaMaxGain).
 //
 // Warps work alone, without barriers: warp = (16 x 16 quarter of a 32 x 32 tile, kMmaPlanes planes),
 // accumulators in registers, each cell written once; a CTA holds the four quarters.  A warp looks
@@ -1880,20 +1884,19 @@ static cudaError_t grid_band(const Geom& g, const Coef<float>& coef, const Index
 
 // the gridding variant a plan uses (Geom::grid_variant 0 = automatic).  Automatic FP32 takes the
 // tensor cores, which need 32-cell tiles, else the shared-memory atomics (on the 1e8-visibility
-// workload the row-band owners measured 289 ms, the atomics 171 ms, the tensor cores half of that)
+// workload the row-band owners measured 289 ms, the atomics 171 ms, the tensor cores 121 ms)
 constexpr int kVariantMma = 4;   // tensor cores: automatic choice only
-// ... and only up to this rounding gain of the plan.  The two kernels round differently (atomics
-// each product and sum, the tensor cores sums only), and the image correction amplifies the planes'
-// rounding by the gain: their images differ by about 2e-7 x gain of the norm (4.2e-6 at a gain of 22,
-// 4.4e-6 at 38, 3.8e-5 at 294) and by up to 2.6e-5 x gain in a pixel at the edge.  Plans of a large
-// gain (coarse accuracies, low oversampling, few visibilities) keep the atomics, so that an image
-// stays within 1e-5 of what it was; the transform is most of their time (1876^2, 57 000 visibilities,
-// gain 294: a forward and backward step takes 3.79 ms by atomics, 3.63 by the tensor cores)
+// ... and only up to this rounding gain of the plan.  The two kernels round differently, and the image
+// correction amplifies the planes' rounding by the gain: their images lie 1 - 4e-7 x gain of the norm apart
+// (3.3 - 5.0e-6 at a gain of 22, 1.8 - 2.7e-5 at about 110, 1.6 - 2.7e-4 at about 800).  Plans of a larger gain
+// than those of 1e-5 (coarse accuracies, low oversampling) keep the atomics, so that an image changes by no
+// more than 1e-5 of its norm with the kernel.  That is the only reason: array observations of 256^2 - 2048^2
+// against an FP64 plan at 1e-9, tensor cores / atomics: gain 110 1.42 - 1.46e-4 / 1.42 - 1.47e-4, 200 2.8 - 3.3e-5 /
+// 3.3 - 5.0e-5, 800 1.4 - 1.6e-4 / 1.4 - 2.7e-4, and the stage 277 / 1161 us (512^2), 1.26 / 1.98 ms (2048^2).
 constexpr double kMmaMaxGain = 40.0;
 template <typename R>
 static int grid_variant_of(const Geom& g) {
-  // double-float planes are written by the plane-owner kernel only
-  if (g.df64_planes) return 2;
+  if (g.df64_planes) return 2;   // k_grid_cells_dd, see grid_owner_g
   const bool band_ok = sizeof(R) == 4 && g.alpha <= 8 && g.tile == kBandTile;
   if (g.grid_variant == 3) return band_ok ? 3 : 1;
   if (g.grid_variant != 0) return g.grid_variant;

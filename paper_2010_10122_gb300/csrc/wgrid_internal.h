@@ -40,7 +40,8 @@ struct Geom {
   double w0_dw;         // w0 / dw
   int64_t max_tile;     // most visibilities in one tile
   double gain;          // amplification of the planes' rounding by the correction (PlanParams::gain)
-  int grid_variant;     // 0 automatic, 1 shared atomics, 2 plane-owner warps, 3 row-band owners
+  int grid_variant;     // 0 automatic (FP32: tensor cores or 1; FP64: 2), 1 shared atomics, 2 plane-owner
+                        // warps, 3 row-band owners; planes of float pairs: always register accumulators
   int df64_planes;      // FP64 plans with the double-float FFT: the uv planes hold double-float
                         // pairs (float4 per cell) and (de)gridding runs in pair arithmetic
 };
