@@ -1711,6 +1711,14 @@ int degrid_subbatch(const Geom& g) {
   return (int)std::max<size_t>(1, (degrid_smem_budget<R>() - coef_bytes<R>()) / degrid_plane_bytes<R>(g));
 }
 
+// Allows a kernel all the dynamic shared memory of a CTA (227 KB).  Every launch sets the same value: host
+// threads that launch a kernel with different sizes at the same time would otherwise lower each other's
+// limit between setting it and the launch.
+template <typename K>
+static cudaError_t allow_shared(K kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+}
+
 template <typename R, int G>
 static cudaError_t degrid_g(const Geom& g, const Coef<R>& coef, const IndexView<R>& ix,
                             const typename C2<R>::T* planes, int b0, int nb, int bs,
@@ -1730,7 +1738,7 @@ static cudaError_t degrid_g(const Geom& g, const Coef<R>& coef, const IndexView<
     if (g.df64_planes) {
       auto launch = [&](auto kernel, bool packed) {
         const size_t bytes = smem - coef_bytes<R>() + degrid_dd_fixed(packed, ix.wts != nullptr);
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        cudaError_t e = allow_shared(kernel);
         if (e != cudaSuccess) return e;
         kernel<<<grid, kThreads, bytes, s>>>(g, coef, ix, planes, b0, nb, bs, partial, nvis_idx, least);
         return cudaGetLastError();
@@ -1740,8 +1748,7 @@ static cudaError_t degrid_g(const Geom& g, const Coef<R>& coef, const IndexView<
       return launch(k_degrid_dd<G, false>, false);
     }
   }
-  cudaError_t e = cudaFuncSetAttribute(k_degrid<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_shared(k_degrid<R, G>);
   if (e != cudaSuccess) return e;
   k_degrid<R, G><<<grid, kThreads, smem, s>>>(g, coef, ix, planes, b0, nb, bs, partial, nvis_idx, least);
   return cudaGetLastError();
@@ -1751,8 +1758,7 @@ template <int W, int SPLIT, int PG>
 static cudaError_t grid_cells_split(const Geom& g, const Coef<double>& coef, const IndexView<double>& ix,
                                     const float4* vis, float4* planes, int b0, int nb, cudaStream_t s) {
   const size_t smem = coef_bytes<double>() + sizeof(CellsStage<W, SPLIT, PG>);
-  cudaError_t e = cudaFuncSetAttribute(k_grid_cells_dd<W, SPLIT, PG>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared(k_grid_cells_dd<W, SPLIT, PG>);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)((int64_t)(g.nu / CellsTile<W>::rows) * (g.nv / CellsTile<W>::cols)),
             (unsigned)((nb + PG - 1) / PG));
@@ -1798,8 +1804,7 @@ static cudaError_t grid_owner_g(const Geom& g, const Coef<R>& coef, const IndexV
       return grid_cells_dd(g, coef, ix, reinterpret_cast<const float4*>(vis),
                            reinterpret_cast<float4*>(planes), b0, nb, s);
   }
-  cudaError_t e = cudaFuncSetAttribute(k_grid_owner<R, G>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared(k_grid_owner<R, G>);
   if (e != cudaSuccess) return e;
   k_grid_owner<R, G><<<grid, kOwnerThreads, smem, s>>>(g, coef, ix, vis, wgt, planes, b0, nb, bs, pitch);
   return cudaGetLastError();
@@ -1817,8 +1822,7 @@ static cudaError_t grid_atomic_g(const Geom& g, const Coef<R>& coef, const Index
   int bs = (int)std::max<size_t>(1, (kGridAtomicSmemBudget - coef_bytes<R>()) / per);
   bs = std::min(bs, nb);
   size_t smem = coef_bytes<R>() + (size_t)bs * per;
-  cudaError_t e = cudaFuncSetAttribute(k_grid_atomic<R, G>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared(k_grid_atomic<R, G>);
   if (e != cudaSuccess) return e;
   int64_t ntiles = (int64_t)g.ntu * g.ntv;
   dim3 grid((unsigned)ntiles, (unsigned)((nb + bs - 1) / bs));
@@ -1831,8 +1835,7 @@ static cudaError_t grid_mma_split(const Geom& g, const Coef<float>& coef, const 
                                   const float2* vis, const float* wgt, float2* planes, int b0,
                                   int nb, uint32_t dense, cudaStream_t s) {
   const size_t smem = 4 * SPLIT * sizeof(MmaWarp);
-  cudaError_t e = cudaFuncSetAttribute(k_grid_mma<G, SPLIT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared(k_grid_mma<G, SPLIT>);
   if (e != cudaSuccess) return e;
   int64_t ntiles = (int64_t)g.ntu * g.ntv;
   dim3 grid((unsigned)ntiles, (unsigned)((nb + kMmaPlanes - 1) / kMmaPlanes));
@@ -1873,8 +1876,7 @@ static cudaError_t grid_band(const Geom& g, const Coef<float>& coef, const Index
   const int bs = std::min(kBandPlanes, nb);
   const size_t smem = coef_bytes<float>() + sizeof(BandStage) +
                       (size_t)bs * kBandTile * kBandPitch * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(k_grid_band, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_shared(k_grid_band);
   if (e != cudaSuccess) return e;
   int64_t ntiles = (int64_t)g.ntu * g.ntv;
   dim3 grid((unsigned)ntiles, (unsigned)((nb + bs - 1) / bs));
