@@ -1379,14 +1379,16 @@ k_grid_mma(const Geom g, const __grid_constant__ Coef<float> coef, const IndexVi
 #pragma unroll
         for (int pl = 0; pl < kMmaPlanes; ++pl) {
           float2 d[4];
-          bool sizable = false, any = false;
+          float most = 0.f;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             d[q] = sm.dw[2 * tig + (q & 1) + (q & 2) * 4][pl];
-            sizable = sizable || !(fabsf(d[q].x) < 0x1p-63f) || !(fabsf(d[q].y) < 0x1p-63f);
-            any = any || d[q].x != 0.f || d[q].y != 0.f;
+            most = fmaxf(most, fmaxf(fabsf(d[q].x), fabsf(d[q].y)));
           }
-          if (!__any_sync(0xffffffffu, sizable)) {
+          if (!__any_sync(0xffffffffu, most >= 0x1p-63f)) {
+            bool any = false;   // (a NaN counts)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) any = any || d[q].x != 0.f || d[q].y != 0.f;
             if (!__any_sync(0xffffffffu, any)) continue;
             // the slices of such data would reach into the bf16 subnormals, which end at 2^-133: in FP32
             // as they are, each lane the cells of its fragments
